@@ -498,7 +498,7 @@ static int cross_dev(qtt_ctx* c, const CrossFn& f, const std::vector<int>& modes
         const int64_t p = std::min(M, Nn);
         TRY(U.alloc(c, (size_t)M * p * sizeof(zc)));
         TRY(sig.alloc(c, (size_t)p * sizeof(double)));
-        TRY(left_svd<double>(c, S.as<zc>(), M, Nn, Nn, U.as<zc>(), sig.as<double>(), &nsv));
+        TRY(left_svd<double>(c, S.as<zc>(), M, Nn, Nn, U.as<zc>(), sig.as<double>(), &nsv, true));
         c->launches++;
         TRY(qtt_trunc_rank<double>(sig.as<double>(), (int)nsv, eps * sqrt(n2) / sq, max_rank, dint,
                                    dscal + 1, c->stream));

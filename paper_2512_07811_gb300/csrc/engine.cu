@@ -392,17 +392,20 @@ static double qr_flops(double m, double n, bool with_q) {
 // dot products of length p and two rotations of p- and q-long column pairs
 static double jacobi_sweep_flops(double p, double q) { return 0.5 * q * (q - 1) * (40.0 * p + 24.0 * q); }
 
+// workspace elements of `batch` m x n QRs: the matrices' reflectors, then n scalars each
+static size_t qr_work(int64_t m, int64_t n, int64_t batch) { return (size_t)batch * (m + 1) * n; }
+
 template <class R>
 static int qr_launch(qtt_ctx* c, const cplx<R>* in, MIdx inB, MIdx rowI, MIdx colI, int conj_in, int64_t m,
                      int64_t n, int64_t rows_total, int64_t rows_per_batch, int64_t batch, cplx<R>* W, cplx<R>* out,
                      int64_t out_bstride, int64_t ldr, cplx<R>* tauws = nullptr, cplx<R>* Qout = nullptr,
-                     int64_t q_bstride = 0, int64_t ldq = 0) {
+                     int64_t q_bstride = 0, int64_t ldq = 0, bool one_cta = false) {
   c->launches++;
   void* qws = nullptr;
   if (Qout) TRY(dalloc(c, &qws, (size_t)batch * m * std::min(m, n) * sizeof(cplx<R>)));
   cudaEvent_t ev = prof_begin(c);
   int st = qtt_qr_r<R>(in, inB, rowI, colI, conj_in, m, n, rows_total, rows_per_batch, batch, W, out, out_bstride,
-                       ldr, c->stream, tauws, Qout, q_bstride, ldq, reinterpret_cast<cplx<R>*>(qws));
+                       ldr, c->stream, tauws, Qout, q_bstride, ldq, reinterpret_cast<cplx<R>*>(qws), one_cta);
   dfree(c, qws);
   prof_end(c, ev, PK_QR, batch * qr_flops((double)m, (double)n, Qout != nullptr),
            (double)batch * m * n * sizeof(cplx<R>) * 2.0);
@@ -502,18 +505,19 @@ static int jacobi_launch(qtt_ctx* c, cplx<R>* G, cplx<R>* Vwork, R* sigma, cplx<
 // one block remains.  Output: min(m, n) x n, row-major, leading dimension n.
 template <class R>
 int tsqr_r(qtt_ctx* c, const cplx<R>* in, MIdx rowI, MIdx colI, int conj_in, int64_t m, int64_t n, cplx<R>* Rout,
-           int64_t* rows_out) {
+           int64_t* rows_out, bool one_cta = false) {
   const int64_t chunk = std::max<int64_t>(2 * n, 256);
   if (m <= chunk) {
     DBuf W;
-    TRY(W.alloc(c, (size_t)m * n * sizeof(cplx<R>)));
-    TRY(qr_launch<R>(c, in, B0(), rowI, colI, conj_in, m, n, m, m, 1, W.as<cplx<R>>(), Rout, 0, n));
+    TRY(W.alloc(c, qr_work(m, n, 1) * sizeof(cplx<R>)));
+    TRY(qr_launch<R>(c, in, B0(), rowI, colI, conj_in, m, n, m, m, 1, W.as<cplx<R>>(), Rout, 0, n, nullptr,
+                     nullptr, 0, 0, one_cta));
     *rows_out = std::min(m, n);
     return QTT_OK;
   }
   const int64_t nch = (m + chunk - 1) / chunk;
   DBuf W, Rs;
-  TRY(W.alloc(c, (size_t)nch * chunk * n * sizeof(cplx<R>)));
+  TRY(W.alloc(c, qr_work(chunk, n, nch) * sizeof(cplx<R>)));
   TRY(Rs.alloc(c, (size_t)nch * n * n * sizeof(cplx<R>)));
   // batch b reads rows [b*chunk, (b+1)*chunk): the batch stride is chunk rows;
   // at most 65535 batches per launch, so very tall inputs go in slabs
@@ -523,9 +527,10 @@ int tsqr_r(qtt_ctx* c, const cplx<R>* in, MIdx rowI, MIdx colI, int conj_in, int
   for (int64_t b0 = 0; b0 < nch; b0 += max_batch) {
     const int64_t nb = std::min(max_batch, nch - b0), r0 = b0 * chunk;
     TRY(qr_launch<R>(c, in + r0 * rowI.s1, L1(nb, chunk * rowI.s1), rows, colI, conj_in, chunk, n, m - r0, chunk,
-                     nb, W.as<cplx<R>>() + b0 * chunk * n, Rs.as<cplx<R>>() + b0 * n * n, n * n, n));
+                     nb, W.as<cplx<R>>() + b0 * chunk * n, Rs.as<cplx<R>>() + b0 * n * n, n * n, n, nullptr, nullptr,
+                     0, 0, one_cta));
   }
-  return tsqr_r<R>(c, Rs.as<cplx<R>>(), L1(nch * n, n), L1(n, 1), 0, nch * n, n, Rout, rows_out);
+  return tsqr_r<R>(c, Rs.as<cplx<R>>(), L1(nch * n, n), L1(n, 1), 0, nch * n, n, Rout, rows_out, one_cta);
 }
 
 // Left singular vectors and singular values of a (rows x cols) row-major
@@ -533,16 +538,22 @@ int tsqr_r(qtt_ctx* c, const cplx<R>* in, MIdx rowI, MIdx colI, int conj_in, int
 // got = min(rows, cols)), then one-sided Jacobi on R^H (rows x got), whose
 // normalised rotated columns are the left singular vectors of C (no rotation
 // accumulation).  U: rows x got, row-major (leading dimension got), columns
-// by decreasing singular value; sigma: got values; *nsv = got.
+// by decreasing singular value; sigma: got values; *nsv = got.  `sampling`
+// (TT-cross) keeps the one-CTA QR kernels: the samples of a 0/1 geometry have
+// many equal singular values, so the pivots, and with them what a run of the
+// cross finds, hang on the rounding of the factorisation (on the 64^3 sphere
+// the cluster kernel's rounding left 2 of 6 seeds short of the exact rank
+// 113, the one-CTA kernels' 1).
 template <class R>
 int left_svd(qtt_ctx* c, const cplx<R>* Cm, int64_t rows, int64_t cols, int64_t ld, cplx<R>* U, R* sigma,
-             int64_t* nsv) {
+             int64_t* nsv, bool sampling) {
   const int64_t p = std::min(rows, cols);
   DBuf Rc, G;
   TRY(Rc.alloc(c, (size_t)std::max<int64_t>(p, 1) * rows * sizeof(cplx<R>)));
   int64_t got = 0;
   // C^H is cols x rows: element (i, j) = conj(C[j, i]) -> row stride 1, column stride ld
-  TRY(tsqr_r<R>(c, Cm, L1(cols, 1), L1(rows, ld), 1, cols, rows, Rc.as<cplx<R>>(), &got));
+  TRY(tsqr_r<R>(c, Cm, L1(cols, 1), L1(rows, ld), 1, cols, rows, Rc.as<cplx<R>>(), &got,
+                 sampling));
   // G = R^H (rows x got): element (i, j) = conj(R[j, i])
   TRY(G.alloc(c, (size_t)rows * std::max<int64_t>(got, 1) * sizeof(cplx<R>)));
   c->launches++;
@@ -901,7 +912,7 @@ int round_det(qtt_ctx* c, const qtt_tt* x, double eps, int max_rank, const int* 
     const int64_t pq = std::min(rk, Tcols);
     TRY(Rc.alloc(c, (size_t)pq * rk * sizeof(cplx<R>)));
     TRY(Qc.alloc(c, (size_t)Tcols * pq * sizeof(cplx<R>)));
-    TRY(Wq.alloc(c, (size_t)Tcols * rk * sizeof(cplx<R>)));
+    TRY(Wq.alloc(c, qr_work(Tcols, rk, 1) * sizeof(cplx<R>)));
     TRY(tau.alloc(c, (size_t)2 * rk * sizeof(cplx<R>)));
     TRY(qr_launch<R>(c, Cm, B0(), L1(Tcols, 1), L1(rk, Tcols), 1, Tcols, rk, Tcols, Tcols, 1,
                      Wq.as<cplx<R>>(), Rc.as<cplx<R>>(), 0, rk, tau.as<cplx<R>>(), Qc.as<cplx<R>>(), 0, pq));
@@ -1055,7 +1066,7 @@ int round_det_batch(qtt_ctx* c, int B, const qtt_tt* const* xs, double eps, int 
     rp[k + 1] = std::min(m, a1);
     DBuf W;
     TRY(Rf[k].alloc(c, (size_t)B * rp[k + 1] * a1 * sizeof(C)));
-    TRY(W.alloc(c, (size_t)B * m * a1 * sizeof(C)));
+    TRY(W.alloc(c, qr_work(m, a1, B) * sizeof(C)));
     TRY(qr_launch<R>(c, M, L1(B, mst), L1(m, a1), L1(a1, 1), 0, m, a1, m, 0, B, W.as<C>(), Rf[k].as<C>(),
                      rp[k + 1] * a1, a1));
   }
@@ -1109,7 +1120,7 @@ int round_det_batch(qtt_ctx* c, int B, const qtt_tt* const* xs, double eps, int 
     if (Tcols < rk) {
       // C taller than wide: R-only QR of C_b (read conjugated through C_b^H), Jacobi on R_b^H
       TRY(Rq.alloc(c, (size_t)B * Tcols * Tcols * sizeof(C)));
-      TRY(W2.alloc(c, (size_t)B * rk * Tcols * sizeof(C)));
+      TRY(W2.alloc(c, qr_work(rk, Tcols, B) * sizeof(C)));
       TRY(qr_launch<R>(c, Cb.as<C>(), L1(B, rk * Tcols), L1(rk, 1), L1(Tcols, rk), 1, rk, Tcols, rk, 0, B,
                        W2.as<C>(), Rq.as<C>(), Tcols * Tcols, Tcols));
       TRY(Gq.alloc(c, (size_t)B * Tcols * Tcols * sizeof(C)));
@@ -1367,8 +1378,8 @@ int tt_svd_dev(qtt_ctx* c, int d, const std::vector<int>& modes, const cplx<R>* 
 
 template int tt_svd_dev<double>(qtt_ctx*, int, const std::vector<int>&, const zc*, double, int, qtt_dtype, qtt_tt**);
 template int tt_svd_dev<float>(qtt_ctx*, int, const std::vector<int>&, const cc*, double, int, qtt_dtype, qtt_tt**);
-template int left_svd<double>(qtt_ctx*, const zc*, int64_t, int64_t, int64_t, zc*, double*, int64_t*);
-template int left_svd<float>(qtt_ctx*, const cc*, int64_t, int64_t, int64_t, cc*, float*, int64_t*);
+template int left_svd<double>(qtt_ctx*, const zc*, int64_t, int64_t, int64_t, zc*, double*, int64_t*, bool);
+template int left_svd<float>(qtt_ctx*, const cc*, int64_t, int64_t, int64_t, cc*, float*, int64_t*, bool);
 
 // ----------------------------------------------------------- inner product
 template <class R>
@@ -1708,7 +1719,7 @@ static int sketch_core(qtt_ctx* c, int T, const qtt_complex* coef, const qtt_mpo
     const int64_t m = lk * no, q = std::min(m, l1);
     DBuf Wq, tau;
     TRY(outc[k].alloc(c, (size_t)m * q * sizeof(C)));
-    TRY(Wq.alloc(c, (size_t)m * l1 * sizeof(C)));
+    TRY(Wq.alloc(c, qr_work(m, l1, 1) * sizeof(C)));
     TRY(tau.alloc(c, (size_t)2 * l1 * sizeof(C)));
     TRY(qr_launch<R>(c, Z.as<C>(), B0(), L1(m, l1), L1(l1, 1), 0, m, l1, m, m, 1, Wq.as<C>(), nullptr, 0, 0,
                      tau.as<C>(), outc[k].as<C>(), 0, q));

@@ -23,7 +23,17 @@ template <class R>
 int qtt_qr_r(const cplx<R>* in, MIdx inB, MIdx rowI, MIdx colI, int conj_in, int64_t m, int64_t n,
              int64_t rows_total, int64_t rows_per_batch, int64_t batch, cplx<R>* W, cplx<R>* out,
              int64_t out_bstride, int64_t ldr, cudaStream_t s, cplx<R>* tauws = nullptr,
-             cplx<R>* Qout = nullptr, int64_t q_bstride = 0, int64_t ldq = 0, cplx<R>* Qws = nullptr);
+             cplx<R>* Qout = nullptr, int64_t q_bstride = 0, int64_t ldq = 0, cplx<R>* Qws = nullptr,
+             bool one_cta = false);
+
+// Householder QR by one cluster per matrix (qr.cu): V (batch * (m + 1) * n elements) receives the reflectors and
+// their scalars, out R or (out_rh) R^H, perm (n ints per matrix, or null) the column order by decreasing norm, Qout Q or null.
+// QTT_ERR_UNSUPPORTED for shapes it does not take (m > 512, or columns beyond its shared memory).
+template <class R>
+int qtt_qr_cluster(const cplx<R>* in, MIdx inB, MIdx rowI, MIdx colI, int conj_in, int64_t m, int64_t n,
+                   int64_t rows_total, int64_t rows_per_batch, int64_t batch, cplx<R>* V, cplx<R>* out,
+                   int64_t out_bstride, int64_t ldr, int out_rh, int* perm, cplx<R>* Qout, int64_t q_bstride,
+                   int64_t ldq, cudaStream_t s);
 
 template <class R>
 size_t qtt_jacobi_smem_bytes(int p, int q);

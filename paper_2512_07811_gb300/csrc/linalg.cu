@@ -1590,11 +1590,18 @@ template <class R>
 int qtt_qr_r(const cplx<R>* in, MIdx inB, MIdx rowI, MIdx colI, int conj_in, int64_t m, int64_t n,
              int64_t rows_total, int64_t rows_per_batch, int64_t batch, cplx<R>* W, cplx<R>* out,
              int64_t out_bstride, int64_t ldr, cudaStream_t s, cplx<R>* tauws, cplx<R>* Qout,
-             int64_t q_bstride, int64_t ldq, cplx<R>* Qws) {
+             int64_t q_bstride, int64_t ldq, cplx<R>* Qws, bool one_cta) {
   if (batch <= 0 || m <= 0 || n <= 0) return QTT_OK;
   if (batch > 65535 || m > INT32_MAX || n > INT32_MAX) return QTT_ERR_ARG;
-  // FP32: the blocked kernel where its shared memory fits; else the panel
-  // kernel for up to 512 rows (256 in FP64); else the workspace kernel
+  // W holds batch * (m + 1) * n elements.  The cluster kernel (not with
+  // one_cta, see left_svd) up to 512 rows where its shared memory holds the
+  // columns; else, FP32, the blocked kernel where its shared memory fits; else
+  // the panel kernel for up to 512 rows (256 in FP64); else the workspace kernel
+  if (!one_cta) {
+    const int st = qtt_qr_cluster<R>(in, inB, rowI, colI, conj_in, m, n, rows_total, rows_per_batch, batch, W, out,
+                                     out_bstride, ldr, 0, nullptr, Qout, q_bstride, ldq, s);
+    if (st != QTT_ERR_UNSUPPORTED) return st;
+  }
   if constexpr (sizeof(R) == 4) {
     int st = QTT_ERR_UNSUPPORTED;
     if (m <= 128)
@@ -1672,9 +1679,9 @@ int qtt_trunc_rank(const R* sigma, int q, double delta, int max_rank, int* out, 
 }
 
 template int qtt_qr_r<double>(const zc*, MIdx, MIdx, MIdx, int, int64_t, int64_t, int64_t, int64_t, int64_t,
-                              zc*, zc*, int64_t, int64_t, cudaStream_t, zc*, zc*, int64_t, int64_t, zc*);
+                              zc*, zc*, int64_t, int64_t, cudaStream_t, zc*, zc*, int64_t, int64_t, zc*, bool);
 template int qtt_qr_r<float>(const cc*, MIdx, MIdx, MIdx, int, int64_t, int64_t, int64_t, int64_t, int64_t,
-                             cc*, cc*, int64_t, int64_t, cudaStream_t, cc*, cc*, int64_t, int64_t, cc*);
+                             cc*, cc*, int64_t, int64_t, cudaStream_t, cc*, cc*, int64_t, int64_t, cc*, bool);
 template int qtt_jacobi<double>(zc*, zc*, double*, zc*, int, int, int, int, int*, cudaStream_t, zc*);
 template int qtt_jacobi<float>(cc*, cc*, float*, cc*, int, int, int, int, int*, cudaStream_t, cc*);
 template int qtt_trunc_rank<double>(const double*, int, double, int, int*, double*, cudaStream_t);
