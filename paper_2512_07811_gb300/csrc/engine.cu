@@ -533,6 +533,65 @@ int tsqr_r(qtt_ctx* c, const cplx<R>* in, MIdx rowI, MIdx colI, int conj_in, int
   return tsqr_r<R>(c, Rs.as<cplx<R>>(), L1(nch * n, n), L1(n, 1), 0, nch * n, n, Rout, rows_out, one_cta);
 }
 
+// ---------------------------------------------- SVD by sorted QR + Jacobi
+// Right singular vectors of `batch` m x n matrices C (element (i, j) of matrix
+// b at in[inB(b) + rowI(i) + colI(j)], conjugated if conj_in): C P = Q R with
+// the columns of C in the order P of decreasing norm (R only), then one-sided
+// Jacobi on the columns of R^H, whose rotated columns are the right vectors of
+// C P.  The sort is what pays: R^H then has its large columns first and is
+// close to diagonal already, and Jacobi takes 6-7 sweeps where C^H itself, or
+// an unsorted R^H, takes 14-21 (rounding matrices of 64 to 128 columns with
+// singular values over six decades).  Vh: min(m, n) x n per matrix, rows by
+// decreasing singular value; trunc, delta(s), max_rank, mask as in qtt_svd.
+// fits: whether the two cluster kernels take the shape (m beyond 512 rows is
+// first reduced by a TSQR, single matrices only).
+template <class R>
+static bool svd_right_fits(int64_t m, int64_t n, int64_t batch, const MIdx& rowI) {
+  if (n > 512) return false;
+  if (m > 512) {
+    if (batch != 1 || rowI.n2 != 1 || n > 256) return false;
+    m = n;
+  }
+  return qtt_qr_cluster_fits<R>(m, n, batch) && qtt_svd_fits<R>((int)n, (int)std::min(m, n), (int)batch);
+}
+
+template <class R>
+static int svd_right(qtt_ctx* c, const cplx<R>* in, MIdx inB, MIdx rowI, MIdx colI, int conj_in, int64_t m, int64_t n,
+                     int64_t batch, cplx<R>* Vh, R* sigma, int* trunc, double delta, const double* deltas,
+                     int max_rank, int mask) {
+  DBuf R1, W, G, perm;
+  if (m > 512) {
+    TRY(R1.alloc(c, (size_t)n * n * sizeof(cplx<R>)));
+    int64_t got = 0;
+    TRY(tsqr_r<R>(c, in, rowI, colI, conj_in, m, n, R1.as<cplx<R>>(), &got));
+    in = R1.as<cplx<R>>();
+    inB = B0();
+    m = got;
+    rowI = L1(m, n);
+    colI = L1(n, 1);
+    conj_in = 0;
+  }
+  const int64_t q = std::min(m, n);
+  TRY(W.alloc(c, qr_work(m, n, batch) * sizeof(cplx<R>)));
+  TRY(G.alloc(c, (size_t)batch * n * q * sizeof(cplx<R>)));
+  TRY(perm.alloc(c, (size_t)batch * n * sizeof(int)));
+  c->launches += 2;
+  cudaEvent_t ev = prof_begin(c);
+  TRY(qtt_qr_cluster<R>(in, inB, rowI, colI, conj_in, m, n, m, 0, batch, W.as<cplx<R>>(), G.as<cplx<R>>(), n * q, q, 1,
+                        perm.as<int>(), nullptr, 0, 0, c->stream));
+  prof_end(c, ev, PK_QR, batch * qr_flops((double)m, (double)n, false), (double)batch * m * n * sizeof(cplx<R>) * 2.0);
+  prof_shape(c, ev, m, n, 0, batch, 0);
+  int idx;
+  int* slot = prof_sweep_slot(c, &idx);
+  ev = prof_begin(c);
+  TRY(qtt_svd<R>(G.as<cplx<R>>(), perm.as<int>(), Vh, sigma, trunc, delta, deltas, max_rank, mask, (int)n, (int)q,
+                 (int)batch, 60, slot, c->stream));
+  prof_end(c, ev, PK_JACOBI, 0.0, (double)batch * n * q * sizeof(cplx<R>) * 2.0, idx,
+           batch * jacobi_sweep_flops((double)n, (double)q));
+  prof_shape(c, ev, n, q, 0, batch);
+  return QTT_OK;
+}
+
 // Left singular vectors and singular values of a (rows x cols) row-major
 // matrix C (leading dimension ld): C^H = Q R by TSQR (R only, got x rows,
 // got = min(rows, cols)), then one-sided Jacobi on R^H (rows x got), whose
@@ -548,6 +607,17 @@ template <class R>
 int left_svd(qtt_ctx* c, const cplx<R>* Cm, int64_t rows, int64_t cols, int64_t ld, cplx<R>* U, R* sigma,
              int64_t* nsv, bool sampling) {
   const int64_t p = std::min(rows, cols);
+  if (!sampling && svd_right_fits<R>(cols, rows, 1, L1(cols, 1))) {
+    // right vectors of C^H; U is the adjoint of what svd_right returns
+    DBuf Vh;
+    TRY(Vh.alloc(c, (size_t)p * rows * sizeof(cplx<R>)));
+    TRY(svd_right<R>(c, Cm, B0(), L1(cols, 1), L1(rows, ld), 1, cols, rows, 1, Vh.as<cplx<R>>(), sigma, nullptr, 0.0,
+                     nullptr, 0, 0));
+    c->launches++;
+    TRY(qtt_copy_strided<R>(Vh.as<cplx<R>>(), L1(rows, 1), L1(p, rows), rows, p, 1, U, p, c->stream));
+    *nsv = p;
+    return QTT_OK;
+  }
   DBuf Rc, G;
   TRY(Rc.alloc(c, (size_t)std::max<int64_t>(p, 1) * rows * sizeof(cplx<R>)));
   int64_t got = 0;
@@ -708,13 +778,12 @@ static int polar_truncate_dev(qtt_ctx* c, const cplx<R>* A, int64_t m, int64_t q
 // r_{k+1} unfoldings have orthonormal columns), so every R factor is the
 // identity and the left sweep is skipped.
 //
-// The SVD of C_k is taken by one-sided Jacobi on C_k^H itself (C^H V = W,
-// right singular vectors W / |W|): its Gram matrix equals that of the
-// triangular factor of a QR of C_k^H, so a QR first would not shorten the
-// sweeps; it pays only when C_k is far wider than tall.  The right vectors
-// come from the rotated data, not from the accumulated rotations V, whose
-// rounding error would leak into the kept subspace (about 10x larger rounding
-// error in FP32).
+// The SVD of C_k: a QR of C_k with sorted columns, then one-sided Jacobi on
+// R^H (svd_right).  Shapes that those kernels do not take go by one-sided
+// Jacobi on C_k^H itself (C^H V = W, right singular vectors W / |W|), or on the
+// R^H of an unsorted QR.  The right vectors come from the rotated data, not
+// from the accumulated rotations V, whose rounding error would leak into the
+// kept subspace (about 10x larger rounding error in FP32).
 template <class R>
 int round_det(qtt_ctx* c, const qtt_tt* x, double eps, int max_rank, const int* forced, qtt_round_info* info,
               qtt_tt** yout, bool left_orth, bool polar) {
@@ -804,6 +873,42 @@ int round_det(qtt_ctx* c, const qtt_tt* x, double eps, int max_rank, const int* 
     DBuf Cb, U, UG, sig, Rc, Qc, Wq, tau, Vw;
     // Jacobi on G = C^H (Tcols x rk, row-major) unless C is so wide that a QR
     // of C^H first pays for itself
+    if (!polar && svd_right_fits<R>(rk, Tcols, 1, L1(rk, Tcols))) {
+      const cplx<R>* Cm = T;  // R factor is the identity for a left-orthogonal train
+      if (!left_orth) {
+        TRY(Cb.alloc(c, (size_t)rk * Tcols * sizeof(cplx<R>)));
+        TRY(mm<R>(c, rk, Tcols, a0, Rf[k - 1].as<cplx<R>>(), a0, 1, 0, T, Tcols, 1, 0, Cb.as<cplx<R>>(), Tcols, 1));
+        Cm = Cb.as<cplx<R>>();
+      }
+      TRY(dbg_finite<R>(c, Cm, rk * Tcols, "round sweep2 C", k));
+      // the core is the first t rows of the vectors' buffer
+      const int64_t q = std::min(rk, Tcols);
+      TRY(newc[k].alloc(c, (size_t)q * Tcols * sizeof(cplx<R>)));
+      const int cap = forced ? (int)std::min<int64_t>(forced[k], q) : max_rank;
+      TRY(svd_right<R>(c, Cm, B0(), L1(rk, Tcols), L1(Tcols, 1), 0, rk, Tcols, 1, newc[k].as<cplx<R>>(), nullptr, dint,
+                       forced ? -1.0 : delta, nullptr, cap, 0));
+      int hv[4];
+      TRY(sync_read(c, hv, dint, sizeof(hv)));
+      double tl;
+      memcpy(&tl, hv + 2, sizeof(double));
+      const int t = hv[0];
+      if (!forced) capped |= hv[1];
+      tail2 += tl * tl;
+      nr[k] = t;
+      const cplx<R>* Vh = newc[k].as<cplx<R>>();
+      TRY(dbg_finite<R>(c, Vh, t * Tcols, "round sweep2 Vh", k));
+      // P = T V (a0 x t); T_{k-1} = A_{k-1} P
+      DBuf P, Tn;
+      TRY(P.alloc(c, (size_t)a0 * t * sizeof(cplx<R>)));
+      TRY(mm<R>(c, a0, t, Tcols, T, Tcols, 1, 0, Vh, 1, Tcols, 1, P.as<cplx<R>>(), t, 1));
+      const int64_t pr = (int64_t)r[k - 1] * n[k - 1];
+      TRY(Tn.alloc(c, (size_t)pr * t * sizeof(cplx<R>)));
+      TRY(mm<R>(c, pr, t, a0, A(k - 1), a0, 1, 0, P.as<cplx<R>>(), t, 1, 0, Tn.as<cplx<R>>(), t, 1));
+      Tb = std::move(Tn);
+      T = Tb.as<cplx<R>>();
+      Trows = r[k - 1];
+      continue;
+    }
     const int64_t jp = Tcols;
     int64_t jq = rk;
     // Jacobi on C^H directly only where one of the fast single-launch
@@ -1098,6 +1203,7 @@ int round_det_batch(qtt_ctx* c, int B, const qtt_tt* const* xs, double eps, int 
   }
   // ---- sweep 2
   std::vector<DBuf> newc(d);
+  std::vector<int64_t> nst(d, 0);   // elements between the trains' new cores
   std::vector<int> tmax(d + 1, 1);
   std::vector<std::vector<int>> tb(B, std::vector<int>(d + 1, 1));
   std::vector<double> tail2(B, 0.0);
@@ -1108,10 +1214,48 @@ int round_det_batch(qtt_ctx* c, int B, const qtt_tt* const* xs, double eps, int 
   int64_t tst = xst;
   for (int k = d - 1; k >= 1; --k) {
     const int64_t nk = n[k], Tcols = nk * tmax[k + 1], rk = rp[k], a0 = r[k];
-    if (!(Tcols <= 4 * rk || Tcols * rk <= 4096)) return QTT_ERR_UNSUPPORTED;
+    const bool fast = svd_right_fits<R>(rk, Tcols, B, L1(rk, Tcols));
+    if (!fast && !(Tcols <= 4 * rk || Tcols * rk <= 4096)) return QTT_ERR_UNSUPPORTED;
     // C_b^H (Tcols x rk) = (R_{k-1,b} T_b)^H, written transposed
     DBuf Cb, Rq, Gq, W2, X, sig;
     TRY(Cb.alloc(c, (size_t)B * rk * Tcols * sizeof(C)));
+    if (fast) {
+      // C_b, its right vectors (zero beyond each train's rank), the ranks
+      const int64_t q = std::min(rk, Tcols);
+      TRY(gemm<R>(c, bgemm<R>(B, rk, Tcols, a0, rk * a0, L1(rk, a0), L1(a0, 1), tst, L1(a0, Tcols), L1(Tcols, 1),
+                              rk * Tcols, L1(rk, Tcols), L1(Tcols, 1)),
+                  Rf[k - 1].as<C>(), T, Cb.as<C>()));
+      nst[k] = q * Tcols;
+      TRY(newc[k].alloc(c, (size_t)B * nst[k] * sizeof(C)));
+      TRY(svd_right<R>(c, Cb.as<C>(), L1(B, rk * Tcols), L1(rk, Tcols), L1(Tcols, 1), 0, rk, Tcols, B,
+                       newc[k].as<C>(), nullptr, dtr, 0.0, dnorm, max_rank, 1));
+      TRY(sync_read(c, hv.data(), dtr, (size_t)4 * B * sizeof(int)));
+      int tm = 1;
+      for (int b = 0; b < B; ++b) {
+        double tl;
+        memcpy(&tl, &hv[(size_t)4 * b + 2], sizeof(double));
+        tb[b][k] = hv[(size_t)4 * b];
+        capped[b] |= hv[(size_t)4 * b + 1];
+        tail2[b] += tl * tl;
+        tm = std::max(tm, tb[b][k]);
+      }
+      tmax[k] = tm;
+      // P_b = T_b V_b (a0 x tm); T_{k-1,b} = A_{k-1,b} P_b
+      DBuf P, Tn;
+      TRY(P.alloc(c, (size_t)B * a0 * tm * sizeof(C)));
+      TRY(gemm<R>(c, bgemm<R>(B, a0, tm, Tcols, tst, L1(a0, Tcols), L1(Tcols, 1), nst[k], L1(Tcols, 1),
+                              L1(tm, Tcols), a0 * tm, L1(a0, tm), L1(tm, 1), 0, 1),
+                  T, newc[k].as<C>(), P.as<C>()));
+      const int64_t pr = (int64_t)r[k - 1] * n[k - 1];
+      TRY(Tn.alloc(c, (size_t)B * pr * tm * sizeof(C)));
+      TRY(gemm<R>(c, bgemm<R>(B, pr, tm, a0, xst, L1(pr, a0), L1(a0, 1), a0 * tm, L1(a0, tm), L1(tm, 1), pr * tm,
+                              L1(pr, tm), L1(tm, 1)),
+                  A(k - 1), P.as<C>(), Tn.as<C>()));
+      Tb = std::move(Tn);
+      T = Tb.as<C>();
+      tst = pr * tm;
+      continue;
+    }
     TRY(gemm<R>(c, bgemm<R>(B, rk, Tcols, a0, rk * a0, L1(rk, a0), L1(a0, 1), tst, L1(a0, Tcols), L1(Tcols, 1),
                             rk * Tcols, L1(rk, 1), L1(Tcols, rk), 1, 1),
                 Rf[k - 1].as<C>(), T, Cb.as<C>()));
@@ -1165,6 +1309,7 @@ int round_det_batch(qtt_ctx* c, int B, const qtt_tt* const* xs, double eps, int 
     c->launches++;
     TRY(qtt_mask_cols_batch<R>(X.as<C>(), Tcols * jq, Tcols, jq, jq, dtr, 4, B, c->stream));
     // padded core k of train b = X_b[:, :tm]^H (tm x Tcols)
+    nst[k] = tm * Tcols;
     TRY(newc[k].alloc(c, (size_t)B * tm * Tcols * sizeof(C)));
     c->launches++;
     TRY(qtt_copy_batch<R>(X.as<C>(), Tcols * jq, L1(tm, 1), L1(Tcols, jq), tm, Tcols, 1, newc[k].as<C>(), Tcols,
@@ -1224,7 +1369,7 @@ int round_det_batch(qtt_ctx* c, int B, const qtt_tt* const* xs, double eps, int 
   for (int k = 0; k < d; ++k) {
     const C* src = k == 0 ? T : newc[k].as<C>();
     c->launches++;
-    TRY(qtt_crop_batch<R>(src, (int64_t)tmax[k] * n[k] * tmax[k + 1], tmax[k], n[k], tmax[k + 1],
+    TRY(qtt_crop_batch<R>(src, k == 0 ? (int64_t)n[0] * tmax[1] : nst[k], tmax[k], n[k], tmax[k + 1],
                           dptrs + (size_t)k * B, dt01 + (size_t)k * B, dt01 + (size_t)d * B + (size_t)k * B, B,
                           c->stream));
   }

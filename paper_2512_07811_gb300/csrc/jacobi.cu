@@ -1,0 +1,519 @@
+// One-sided Jacobi SVD of small dense matrices by one thread-block cluster per
+// matrix, with the truncation rule at its end.
+//
+// G (p x q, columns rotated to mutual orthogonality) gives the left singular
+// vectors of G as normalised rotated columns.  The columns, padded with zero
+// columns to 2 NC bs, form NB = 2 NC blocks of bs, two per CTA: position i
+// ("top") and NB - 1 - i ("bottom") of the round-robin tournament of the
+// blocks.  In a block-round a CTA rotates the bs x bs cross pairs of its two
+// blocks in bs rounds of bs disjoint pairs, one warp per pair, the top column
+// in registers throughout; in the first block-round of a sweep also the pairs
+// inside each block.  In the last round the rotated columns are written straight
+// from registers to the shared memory of the CTA that holds them next, so a
+// block exchange costs one cluster barrier.
+//
+// What bounds it: a sweep is a chain of about q rounds, each the latency of one
+// pair (dot product, warp reduction, rotation scalars, rotation, barrier), in
+// FP64 also the FP64 pipe (a warp instruction holds it 16 cycles, a dependent
+// one takes 75).  Hence
+//   * the squared column norms are carried along, |a|^2 -+ |g|^2 / w, and summed
+//     anew once a sweep and after a drop below a twentieth, which leaves one
+//     inner product per pair instead of three;
+//   * the rotation needs two reciprocal square roots and no division (see
+//     rotate_pair);
+//   * a sweep in which every rotation was small is the last one: the next
+//     would only confirm it (see `big2`).
+// The caller sorts and QR-factors the matrix first (jacobi on R^H), which cuts
+// the sweeps from 14-21 to 6-7 on the roundings' matrices.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
+#include "common.cuh"
+#include "dense.cuh"
+#include "kernels.h"
+
+namespace {
+
+namespace cg = cooperative_groups;
+using dense::Lim;
+
+template <class R>
+struct JacArgs {
+  const cplx<R>* G;       // p x q row-major, matrices p*q apart
+  const int* perm;        // row i of G is component perm[i] of the vectors (p apart), or null
+  cplx<R>* Vh;            // q x p row-major: row j the conjugate of vector j, by decreasing singular value
+  R* sigma;               // q, or null
+  int* trunc;             // 4 per matrix: rank kept, 1 if max_rank cut it, discarded tail (double); or null
+  double delta;           // threshold of the tail
+  const double* deltas;   // per matrix instead of delta, or null
+  int max_rank;           // 0: no cap
+  int mask;               // rows of Vh from the kept rank on are zeroed
+  int p, q, bs, max_sweeps;
+  int* sweeps;
+};
+
+template <class R>
+struct JacThreads {
+  static constexpr int value = sizeof(R) == 8 ? 256 : 512;  // FP64 columns take twice the registers
+};
+
+template <class R>
+__device__ __forceinline__ cplx<R> wsum_c(cplx<R> w, int lane) {
+  if constexpr (sizeof(R) == 4) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      w.re += __shfl_xor_sync(0xffffffffu, w.re, o);
+      w.im += __shfl_xor_sync(0xffffffffu, w.im, o);
+    }
+    return w;
+  } else {
+    const bool up = lane & 16;
+    R v = (up ? w.im : w.re) + __shfl_xor_sync(0xffffffffu, up ? w.re : w.im, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return cplx<R>(__shfl_sync(0xffffffffu, v, 0), __shfl_sync(0xffffffffu, v, 16));
+  }
+}
+
+// reciprocal square root that only steers a rotation angle
+__device__ __forceinline__ float rsqrt_fast(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double rsqrt_fast(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  return fma(0.5 * y, fma(-x * y, y, 1.0), y);
+}
+
+template <class R, int RPL>
+__device__ __forceinline__ R col_norm2(const cplx<R> (&x)[RPL]) {
+  R s = 0, s1 = 0;
+#pragma unroll
+  for (int u = 0; u < RPL; ++u) {
+    if (u & 1) s1 += abs2(x[u]); else s += abs2(x[u]);
+  }
+  return dense::wsum(s + s1);
+}
+
+// Rotates columns x, y (rows on the lanes) to orthogonality; al, be their
+// squared norms.  With g = x^H y, d = (be - al) / 2, h = sqrt(d^2 + |g|^2) and
+// w = |d| + h, the smaller root has tan = |g| / w and w^2 + |g|^2 = 2 h w, so
+// with r = 1 / sqrt(w^2 + |g|^2): cos = w r, sin e^{i arg g} = g r (signed by
+// d), and the norms change by |g|^2 / w = 2 |g|^2 h r^2.  cos^2 + sin^2 = 1 to
+// the accuracy of r, whatever h is.  Returns 0 (orthogonal to tol, or |g|^2
+// below the normal range), 1 (rotated), 3 (rotated, not small: |cos of the
+// angle between x and y| or the sine weighted by the norms' ratio above
+// sqrt(big2)).
+template <class R, int RPL>
+__device__ __forceinline__ int rotate_pair(cplx<R> (&x)[RPL], cplx<R> (&y)[RPL], R& al, R& be, R tol2, R big2,
+                                           int lane) {
+  cplx<R> g(0, 0), g1(0, 0);
+#pragma unroll
+  for (int u = 0; u < RPL; ++u) {
+    if (u & 1) cfma_conj(g1, x[u], y[u]); else cfma_conj(g, x[u], y[u]);
+  }
+  g = wsum_c(g + g1, lane);
+  const R ag2 = abs2(g), ab = al * be;
+  if (!(ag2 > tol2 * ab) || !(ag2 >= Lim<R>::tiny)) return 0;
+  const R d = R(0.5) * (be - al), h2 = fma(d, d, ag2);
+  const R h = h2 * rsqrt_fast(h2), w = fabs(d) + h;
+  const R r = dense::rsqrt_nr(fma(w, w, ag2));
+  const R cs = w * r, sr = d >= R(0) ? r : -r;
+  const cplx<R> f(sr * g.re, sr * g.im);
+  const R s2 = ag2 * (r * r), dl = (h + h) * s2;
+  const int code = ag2 > big2 * ab || s2 * fmax(al, be) > big2 * fmin(al, be) ? 3 : 1;
+#pragma unroll
+  for (int u = 0; u < RPL; ++u) {
+    const cplx<R> a = x[u], b = y[u];
+    x[u].re = fma(cs, a.re, fma(-f.re, b.re, -f.im * b.im));
+    x[u].im = fma(cs, a.im, fma(-f.re, b.im, f.im * b.re));
+    y[u].re = fma(cs, b.re, fma(f.re, a.re, -f.im * a.im));
+    y[u].im = fma(cs, b.im, fma(f.re, a.im, f.im * a.re));
+  }
+  const R al0 = al, be0 = be;
+  const R sd = d >= R(0) ? dl : -dl;
+  al = al0 - sd;
+  be = be0 + sd;
+  if (!(al > R(0.05) * al0)) al = col_norm2<R, RPL>(x);
+  if (!(be > R(0.05) * be0)) be = col_norm2<R, RPL>(y);
+  return code;
+}
+
+__device__ __forceinline__ int jac_exponent(float a) { return a > 0 && a <= FLT_MAX ? max(ilogbf(a), -110) : -110; }
+__device__ __forceinline__ int jac_exponent(double a) { return a > 0 && a <= DBL_MAX ? max(ilogb(a), -1000) : -1000; }
+__device__ __forceinline__ float jac_pow2(float, int e) { return ldexpf(1.f, e); }
+__device__ __forceinline__ double jac_pow2(double, int e) { return ldexp(1.0, e); }
+
+template <class R, int RPL>
+__global__ void __launch_bounds__(JacThreads<R>::value, 1)
+jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
+  typedef cplx<R> C;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int NC = (int)cluster.num_blocks(), NB = 2 * NC, rank = (int)cluster.block_rank();
+  const int p = a.p, q = a.q, bs = a.bs, qp = NB * bs;
+  constexpr int LD = 32 * RPL;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nthr = blockDim.x;  // bs warps
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* slots = reinterpret_cast<C*>(smem_raw);                 // [4][bs][LD]
+  double* scan = reinterpret_cast<double*>(slots + (size_t)4 * bs * LD);  // 2 of the truncation rule
+  R* nrm = reinterpret_cast<R*>(scan + 2);                   // [4][bs] squared norms
+  R* norms = nrm + 4 * bs;                                   // [qp] final norms
+  R* sorted = norms + qp;                                    // [qp]
+  int* flags = reinterpret_cast<int*>(sorted + qp);          // [2][NC] sweep flags, then [NC] exponents
+  int* s_int = flags + 3 * 16;                               // [0] sweep flags of this CTA, [1] kept rank
+  const int64_t bt = blockIdx.y;
+  const C* G = a.G + bt * (int64_t)p * q;
+  auto col = [&](int slot, int j) { return slots + ((size_t)slot * bs + j) * LD; };
+  int top = 0, bot = 1, in_top = 2, in_bot = 3;
+  if (threadIdx.x == 0) s_int[0] = 0;
+  cluster.sync();
+  // initial blocks (rank on top, NB-1-rank below), and the power of two that
+  // brings the largest component near 1 (FP32: near 2^14, so that squares of
+  // squared norms of columns down to 1e-14 of the largest stay normal)
+  int esc;
+  {
+    R amax = 0;
+    for (int e = threadIdx.x; e < 2 * bs * LD; e += nthr) {
+      const int i = e / (2 * bs), jj = e - i * 2 * bs, half = jj / bs, j = jj - half * bs;
+      const int c = (half == 0 ? rank : NB - 1 - rank) * bs + j;
+      C v(0, 0);
+      if (c < q && i < p) v = G[(int64_t)i * q + c];
+      col(half == 0 ? top : bot, j)[i] = v;
+      amax = fmax(amax, fmax(fabs(v.re), fabs(v.im)));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+    if (lane == 0) sorted[w] = amax;
+    __syncthreads();
+    if (w == 0) {
+      R t = lane < bs ? sorted[lane] : R(0);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t = fmax(t, __shfl_xor_sync(0xffffffffu, t, o));
+      if (lane < NC) cluster.map_shared_rank(flags, lane)[32 + rank] = jac_exponent(t);
+    }
+    cluster.sync();
+    esc = flags[32];
+    for (int i = 1; i < NC; ++i) esc = max(esc, flags[32 + i]);
+    if (sizeof(R) == 4) esc -= 14;
+    const R sg = jac_pow2(R(0), -esc);
+    for (int e = threadIdx.x; e < 2 * bs * LD; e += nthr) slots[e] = sg * slots[e];
+    __syncthreads();
+  }
+  const R tol = Lim<R>::eps * sqrt(R(p > 1 ? p : 1)), tol2 = tol * tol;
+  // Quadratic regime: a rotation by sin s_ij of a pair (i, j) puts back s_ij g_jk
+  // into an annihilated g_ik.  With c the largest cosine and s the largest
+  // sine weighted by the norms' ratio of a sweep, the cosines after it are at
+  // most about sqrt(q) s c; with both at most sqrt(tol / sqrt(q)) / 2 they are
+  // below tol / 4, and the next sweep would rotate nothing.
+  const R big2 = R(0.25) * tol / sqrt(R(q));
+  C x[RPL], y[RPL];
+  auto load = [&](C(&v)[RPL], const C* s) {
+#pragma unroll
+    for (int u = 0; u < RPL; ++u) v[u] = s[lane + 32 * u];
+  };
+  auto store = [&](const C(&v)[RPL], C* s) {
+#pragma unroll
+    for (int u = 0; u < RPL; ++u) s[lane + 32 * u] = v[u];
+  };
+  const int posn[2] = {rank, NB - 1 - rank};
+  int dst_cta[2], dst_top[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int np = posn[h] == 0 ? 0 : (posn[h] == 1 ? NB - 1 : posn[h] - 1);
+    dst_top[h] = np < NC;
+    dst_cta[h] = np < NC ? np : NB - 1 - np;
+  }
+  int sweep = 0;
+  for (; sweep < a.max_sweeps; ++sweep) {
+    int wf = 0;
+    // fresh norms of both blocks
+    load(x, col(top, w));
+    load(y, col(bot, w));
+    {
+      const R na = col_norm2<R, RPL>(x), nb = col_norm2<R, RPL>(y);
+      if (lane == 0) {
+        nrm[top * bs + w] = na;
+        nrm[bot * bs + w] = nb;
+      }
+    }
+    __syncthreads();
+    // pairs inside each block (round-robin of bs columns, one bye if bs is odd)
+    const int be_ = bs + (bs & 1), half = be_ / 2;
+    for (int s = 0; s + 1 < be_; ++s) {
+      for (int kk = w; kk < 2 * half; kk += bs) {
+        const int slot = kk < half ? top : bot, k = kk < half ? kk : kk - half;
+        const int j0 = k == 0 ? 0 : 1 + (k - 1 + s) % (be_ - 1);
+        const int k1 = be_ - 1 - k;
+        const int j1 = 1 + (k1 - 1 + s) % (be_ - 1);
+        if (j0 >= bs || j1 >= bs) continue;
+        load(x, col(slot, j0));
+        load(y, col(slot, j1));
+        R al = nrm[slot * bs + j0], be = nrm[slot * bs + j1];
+        const int f = rotate_pair<R, RPL>(x, y, al, be, tol2, big2, lane);
+        if (f) {
+          wf |= f;
+          store(x, col(slot, j0));
+          store(y, col(slot, j1));
+          if (lane == 0) {
+            nrm[slot * bs + j0] = al;
+            nrm[slot * bs + j1] = be;
+          }
+        }
+      }
+      __syncthreads();
+    }
+    for (int br = 0; br < NB - 1; ++br) {
+      load(x, col(top, w));
+      R al = nrm[top * bs + w];
+      int c = w;
+      for (int s = 0; s < bs; ++s) {
+        load(y, col(bot, c));
+        R be = nrm[bot * bs + c];
+        const int f = rotate_pair<R, RPL>(x, y, al, be, tol2, big2, lane);
+        wf |= f;
+        if (s + 1 < bs) {
+          if (f) {
+            store(y, col(bot, c));
+            if (lane == 0) nrm[bot * bs + c] = be;
+          }
+          __syncthreads();
+          c = c + 1 == bs ? 0 : c + 1;
+        } else if (NC > 1) {
+          // both blocks to their next CTA, straight from the registers
+          const int st = dst_top[0] ? in_top : in_bot, sb = dst_top[1] ? in_top : in_bot;
+          C* rs = cluster.map_shared_rank(slots, dst_cta[0]);
+          store(x, rs + ((size_t)st * bs + w) * LD);
+          C* rb = cluster.map_shared_rank(slots, dst_cta[1]);
+          store(y, rb + ((size_t)sb * bs + c) * LD);
+          if (lane == 0) {
+            cluster.map_shared_rank(nrm, dst_cta[0])[st * bs + w] = al;
+            cluster.map_shared_rank(nrm, dst_cta[1])[sb * bs + c] = be;
+          }
+        } else {
+          store(x, col(top, w));
+          store(y, col(bot, c));
+          if (lane == 0) {
+            nrm[top * bs + w] = al;
+            nrm[bot * bs + c] = be;
+          }
+        }
+      }
+      if (br == NB - 2) {
+        if (lane == 0 && wf) atomicOr(&s_int[0], wf);
+        __syncthreads();
+        if (threadIdx.x < NC) cluster.map_shared_rank(flags, threadIdx.x)[(sweep & 1) * 16 + rank] = s_int[0];
+      }
+      if (NC > 1) {
+        cluster.sync();
+        int t = top;
+        top = in_top;
+        in_top = t;
+        t = bot;
+        bot = in_bot;
+        in_bot = t;
+      } else {
+        __syncthreads();
+      }
+    }
+    int any = 0;
+    for (int i = 0; i < NC; ++i) any |= flags[(sweep & 1) * 16 + i];
+    if (threadIdx.x == 0) s_int[0] = 0;  // next written after this sweep's barriers
+    __syncthreads();
+    if (!(any & 2)) {
+      ++sweep;
+      break;
+    }
+  }
+  if (bt == 0 && rank == 0 && threadIdx.x == 0 && a.sweeps) *a.sweeps = sweep;
+  // column norms (whole columns are local), gathered in every CTA
+  load(x, col(top, w));
+  load(y, col(bot, w));
+  const R nx = sqrt(col_norm2<R, RPL>(x)), ny = sqrt(col_norm2<R, RPL>(y));
+  const int cx = rank * bs + w, cy = (NB - 1 - rank) * bs + w;
+  if (lane < NC) {
+    R* rn = cluster.map_shared_rank(norms, lane);
+    rn[cx] = nx;
+    rn[cy] = ny;
+  }
+  cluster.sync();
+  // order by decreasing norm (ties by index; a NaN first, so that it stays a permutation)
+  auto key = [&](int i) {
+    const R v = norms[i];
+    return v == v ? v : Lim<R>::big;
+  };
+  auto place = [&](int c) {
+    const R v = key(c);
+    int rk = 0;
+    for (int i = lane; i < q; i += 32) {
+      const R u = key(i);
+      rk += (u > v) || (u == v && i < c);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) rk += __shfl_xor_sync(0xffffffffu, rk, o);
+    return rk;
+  };
+  const R sb = jac_pow2(R(0), esc);
+  for (int c = w; c < q; c += nthr >> 5) {
+    const int rk = place(c);
+    if (lane == 0) sorted[rk] = norms[c] * sb;
+  }
+  __syncthreads();
+  if (a.sigma && rank == 0)
+    for (int i = threadIdx.x; i < q; i += nthr) a.sigma[bt * q + i] = sorted[i];
+  int keep = q;
+  if (a.trunc) {
+    // smallest t >= 1 with sqrt(sum_{j >= t} s_j^2) <= delta, sums in double
+    // by a suffix scan over the lanes, 32 values at a time from the end
+    if (w == 0) {
+      const double delta = a.deltas ? a.deltas[bt] : a.delta;
+      double tail = 0.0;
+      int t = q;
+      bool stop = false;
+      for (int hi = q; hi > 1 && !stop; hi -= 32) {
+        const int j = hi - 1 - lane;  // lane 0 the last value
+        const double v = j >= 1 ? (double)sorted[j] : 0.0;
+        double s = v * v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const double u = __shfl_up_sync(0xffffffffu, s, o);
+          if (lane >= o) s += u;
+        }
+        s += tail;
+        const unsigned ok = __ballot_sync(0xffffffffu, j >= 1 && sqrt(s) <= delta);
+        const int n = __ffs(~ok) - 1;  // leading lanes whose sums stay within delta (-1: all 32)
+        const int cnt = n < 0 ? 32 : n;
+        t -= cnt;
+        if (cnt > 0) tail = __shfl_sync(0xffffffffu, s, cnt - 1);
+        stop = cnt < 32;
+      }
+      int capped = 0;
+      if (a.max_rank > 0 && t > a.max_rank) {
+        double s = 0.0;
+        for (int j = a.max_rank + lane; j < t; j += 32) s += (double)sorted[j] * (double)sorted[j];
+        tail += dense::wsum(s);
+        t = a.max_rank;
+        capped = 1;
+      }
+      if (lane == 0) {
+        s_int[1] = t;
+        if (rank == 0) {
+          int* o = a.trunc + 4 * bt;
+          o[0] = t;
+          o[1] = capped;
+          *reinterpret_cast<double*>(o + 2) = sqrt(tail);
+        }
+      }
+    }
+    __syncthreads();
+    keep = s_int[1];
+  }
+  // vectors, conjugated, one per row; columns with a subnormal norm carry no usable direction
+  const int* perm = a.perm ? a.perm + bt * p : nullptr;
+  C* Vh = a.Vh + bt * (int64_t)p * q;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int c = h == 0 ? cx : cy;
+    if (c >= q) continue;
+    const int rk = place(c);
+    const R v = h == 0 ? nx : ny;
+    R f = v > Lim<R>::tiny * R(4) ? R(1) / v : R(0);
+    if (a.mask && rk >= keep) f = 0;
+#pragma unroll
+    for (int u = 0; u < RPL; ++u) {
+      const int i = lane + 32 * u;
+      if (i >= p) continue;
+      const C g = h == 0 ? x[u] : y[u];
+      C o(g.re * f, -g.im * f);
+      if (f == R(0)) o = C(0, 0);
+      Vh[(int64_t)rk * p + (perm ? perm[i] : i)] = o;
+    }
+  }
+}
+
+struct JacPlan {
+  int nc, bs, rpl;
+  size_t smem;
+};
+
+int jac_slices(int p) {
+  const int nu = (p + 31) / 32;
+  return nu <= 6 ? nu : nu <= 8 ? 8 : nu <= 12 ? 12 : 16;
+}
+
+template <class R>
+bool jac_plan(int p, int q, int batch, JacPlan* pl) {
+  if (p < 1 || q < 1 || p > 512 || q > 512 || batch < 1 || batch > 65535) return false;
+  const int rpl = jac_slices(p), wmax = JacThreads<R>::value / 32;
+  int ncmax = 16;
+  while (ncmax > 1 && ncmax * batch > 160) ncmax /= 2;
+  int nc = 1;
+  if (sizeof(R) == 4) {
+    nc = q <= 16 ? 1 : q <= 32 ? 2 : q <= 64 ? 4 : q <= 128 ? 8 : 16;
+  } else {
+    nc = q <= 4 ? 1 : q <= 8 ? 2 : q <= 16 ? 4 : q <= 32 ? 8 : 16;
+  }
+  nc = std::min(nc, ncmax);
+  for (; nc <= 16; nc *= 2) {
+    const int bs = (q + 2 * nc - 1) / (2 * nc);
+    const size_t sm = (size_t)4 * bs * 32 * rpl * sizeof(cplx<R>) + 16 + (4 * bs + (size_t)4 * nc * bs) * sizeof(R) +
+                      (48 + 4) * sizeof(int) + 16;
+    if (bs <= wmax && sm <= 200 * 1024) {
+      *pl = JacPlan{nc, bs, rpl, sm};
+      return true;
+    }
+  }
+  return false;
+}
+
+template <class R, int RPL>
+int launch(const JacArgs<R>& a, const JacPlan& pl, int batch, cudaStream_t s) {
+  const void* fn = (const void*)jacobi_cluster2_kernel<R, RPL>;
+  if (qtt_allow_max_smem(fn) != QTT_OK) return QTT_ERR_CUDA;
+  if (pl.nc > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+    return QTT_ERR_CUDA;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)pl.nc, (unsigned)batch, 1);
+  cfg.blockDim = dim3(32 * pl.bs, 1, 1);
+  cfg.dynamicSmemBytes = pl.smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)pl.nc;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, jacobi_cluster2_kernel<R, RPL>, a) == cudaSuccess ? QTT_OK : QTT_ERR_CUDA;
+}
+
+}  // namespace
+
+template <class R>
+bool qtt_svd_fits(int p, int q, int batch) {
+  JacPlan pl;
+  return jac_plan<R>(p, q, batch, &pl);
+}
+
+template <class R>
+int qtt_svd(const cplx<R>* G, const int* perm, cplx<R>* Vh, R* sigma, int* trunc, double delta, const double* deltas,
+            int max_rank, int mask, int p, int q, int batch, int max_sweeps, int* sweeps, cudaStream_t s) {
+  JacPlan pl;
+  if (!jac_plan<R>(p, q, batch, &pl)) return QTT_ERR_UNSUPPORTED;
+  const JacArgs<R> a{G, perm, Vh, sigma, trunc, delta, deltas, max_rank, mask, p, q, pl.bs, max_sweeps, sweeps};
+  switch (pl.rpl) {
+    case 1: return launch<R, 1>(a, pl, batch, s);
+    case 2: return launch<R, 2>(a, pl, batch, s);
+    case 3: return launch<R, 3>(a, pl, batch, s);
+    case 4: return launch<R, 4>(a, pl, batch, s);
+    case 5: return launch<R, 5>(a, pl, batch, s);
+    case 6: return launch<R, 6>(a, pl, batch, s);
+    case 8: return launch<R, 8>(a, pl, batch, s);
+    case 12: return launch<R, 12>(a, pl, batch, s);
+    default: return launch<R, 16>(a, pl, batch, s);
+  }
+}
+template bool qtt_svd_fits<float>(int, int, int);
+template bool qtt_svd_fits<double>(int, int, int);
+template int qtt_svd<float>(const cc*, const int*, cc*, float*, int*, double, const double*, int, int, int, int, int, int,
+                            int*, cudaStream_t);
+template int qtt_svd<double>(const zc*, const int*, zc*, double*, int*, double, const double*, int, int, int, int, int,
+                             int, int*, cudaStream_t);

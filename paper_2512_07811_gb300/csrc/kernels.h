@@ -35,6 +35,20 @@ int qtt_qr_cluster(const cplx<R>* in, MIdx inB, MIdx rowI, MIdx colI, int conj_i
                    int64_t out_bstride, int64_t ldr, int out_rh, int* perm, cplx<R>* Qout, int64_t q_bstride,
                    int64_t ldq, cudaStream_t s);
 
+// One-sided Jacobi SVD by one cluster per matrix (jacobi.cu): left singular vectors of G (p x q row-major, matrices
+// p*q apart), conjugated, one per row of Vh (q x p) by decreasing singular value, component i of G's rows at perm[i]
+// (p per matrix; null: i).  sigma (q, or null); trunc (4 ints per matrix, or null): the rank that the tail threshold
+// delta (deltas[b] if not null) and max_rank (0: no cap) keep, 1 if the cap cut it, the discarded tail as a double;
+// mask: rows of Vh from that rank on are zeroed.  QTT_ERR_UNSUPPORTED where qtt_svd_fits is false.
+template <class R>
+bool qtt_svd_fits(int p, int q, int batch);
+template <class R>
+int qtt_svd(const cplx<R>* G, const int* perm, cplx<R>* Vh, R* sigma, int* trunc, double delta, const double* deltas,
+            int max_rank, int mask, int p, int q, int batch, int max_sweeps, int* sweeps, cudaStream_t s);
+// whether qtt_qr_cluster takes the shape with sorted columns
+template <class R>
+bool qtt_qr_cluster_fits(int64_t m, int64_t n, int64_t batch);
+
 template <class R>
 size_t qtt_jacobi_smem_bytes(int p, int q);
 template <class R>

@@ -549,6 +549,14 @@ int launch(const QrArgs<R>& a, const QrPlan& pl, int64_t batch, cudaStream_t s) 
 }  // namespace
 
 template <class R>
+bool qtt_qr_cluster_fits(int64_t m, int64_t n, int64_t batch) {
+  QrPlan pl;
+  return batch >= 1 && batch <= 65535 && qr_plan<R>(m, n, batch, true, &pl);
+}
+template bool qtt_qr_cluster_fits<float>(int64_t, int64_t, int64_t);
+template bool qtt_qr_cluster_fits<double>(int64_t, int64_t, int64_t);
+
+template <class R>
 int qtt_qr_cluster(const cplx<R>* in, MIdx inB, MIdx rowI, MIdx colI, int conj_in, int64_t m, int64_t n,
                    int64_t rows_total, int64_t rows_per_batch, int64_t batch, cplx<R>* V, cplx<R>* out,
                    int64_t out_bstride, int64_t ldr, int out_rh, int* perm, cplx<R>* Qout, int64_t q_bstride,
