@@ -198,13 +198,18 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
     for (int e = threadIdx.x; e < 2 * bs * LD; e += nthr) slots[e] = sg * slots[e];
     __syncthreads();
   }
-  const R tol = Lim<R>::eps * sqrt(R(p > 1 ? p : 1)), tol2 = tol * tol;
+  // Pairs are rotated down to a cosine of eps / 2 (the inner product's own
+  // rounding is below that): what is left of the cosines is the vectors'
+  // non-orthogonality, which the truncated train inherits once per bond (a
+  // tolerance of eps sqrt(p) made it the largest error of a rounding, 1e-5 at
+  // 128 columns).
+  const R tol = R(0.5) * Lim<R>::eps, tol2 = tol * tol;
   // Quadratic regime: a rotation by sin s_ij of a pair (i, j) puts back s_ij g_jk
   // into an annihilated g_ik.  With c the largest cosine and s the largest
   // sine weighted by the norms' ratio of a sweep, the cosines after it are at
-  // most about sqrt(q) s c; with both at most sqrt(tol / sqrt(q)) / 2 they are
-  // below tol / 4, and the next sweep would rotate nothing.
-  const R big2 = R(0.25) * tol / sqrt(R(q));
+  // most about sqrt(q) s c; with both at most sqrt(tol / sqrt(q)) they are at
+  // most tol, and the next sweep would rotate nothing.
+  const R big2 = tol / sqrt(R(q));
   C x[RPL], y[RPL];
   auto load = [&](C(&v)[RPL], const C* s) {
 #pragma unroll
