@@ -193,7 +193,7 @@ static int tc_route(qtt_ctx* c, const GemmDesc& g0, cc alpha, cc beta, const cc*
 }
 
 // ------------------------------------------------------ GEMM tile autotuner
-// The first CUDA-core GEMM of a shape (element size, M, N, K, batch and which
+// The first FP32 CUDA-core GEMM of a shape (element size, M, N, K, batch and which
 // operand indices are contiguous) with enough work times the two tile edges
 // (32, 64) once, at the split count the rule gives the shape, with CUDA
 // events on the caller's stream into a scratch output, and caches the
@@ -262,9 +262,9 @@ static int tune_gemm(qtt_ctx* c, const GemmDesc& g, const cplx<R>* A, const cplx
 template <class R>
 static int simt_gemm(qtt_ctx* c, const GemmDesc& g, cplx<R> alpha, cplx<R> beta, const cplx<R>* A, const cplx<R>* B,
                      cplx<R>* C) {
-  int tile = 0, splits = qtt_gemm_splits(g);
+  int tile = 0, splits = sizeof(R) == 8 ? qtt_gemm_splits_f64(g) : qtt_gemm_splits(g);
   const bool beta0 = beta.re == R(0) && beta.im == R(0);
-  if (beta0 && (double)g.M * g.N * g.K * g.batch >= 4.0e6) {
+  if (sizeof(R) == 4 && beta0 && (double)g.M * g.N * g.K * g.batch >= 4.0e6) {
     const bool a_kfast = unit_inner(g.kA) && !unit_inner(g.mA);
     const bool b_kfast = unit_inner(g.kB) && !unit_inner(g.nB);
     const TuneKey key{{(int64_t)sizeof(R), g.M, g.N, g.K, g.batch, (int64_t)a_kfast, (int64_t)b_kfast}};
@@ -280,6 +280,7 @@ static int simt_gemm(qtt_ctx* c, const GemmDesc& g, cplx<R> alpha, cplx<R> beta,
     splits = it->second.second;
   }
   void* P = nullptr;
+  splits = (int)std::min<int64_t>(splits, std::max<int64_t>(1, 65535 / std::max<int64_t>(1, g.batch)));
   if (splits > 1 && dalloc(c, &P, (size_t)splits * g.batch * g.M * g.N * sizeof(cplx<R>))) return QTT_ERR_OOM;
   c->launches += splits > 1 ? 2 : 1;
   cudaEvent_t ev = prof_begin(c);

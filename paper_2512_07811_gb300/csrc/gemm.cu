@@ -168,6 +168,89 @@ gemm_midx_kernel(GemmDesc g, cplx<R> alpha, cplx<R> beta,
   }
 }
 
+// FP64 kernel: one output per thread, BM x BN outputs per CTA.  An SM issues two
+// FP64 FMAs a clock, so one warp's complex multiply-add holds its pipe for 64
+// cycles and the shared-memory traffic of one output per thread is hidden
+// under it; what counts is how many SMs work and how much of a tile is
+// padding.  With 32 x 32 tiles (the only choice below 38 tiles of 64 x 64)
+// 64 x 148 x 74 ran on 10 SMs in 94 us and 256 x 4 x 310, batch 144, spent seven
+// eighths of 2560 us on padding; see f64_tile() for the choice.  Sums run over
+// k in order, as in gemm_midx_kernel.
+template <int BM, int BN>
+__global__ void __launch_bounds__(BM * BN)
+gemm_f64_kernel(GemmDesc g, zc alpha, zc beta, const zc* __restrict__ A, const zc* __restrict__ B, zc* __restrict__ C,
+                int splits, int64_t kchunk, zc* __restrict__ P) {
+  constexpr int NT = BM * BN, BK = 16;
+  __shared__ zc As[BK][BM + 1], Bs[BK][BN + 1];
+  const int64_t b = blockIdx.z / splits;
+  const int split = blockIdx.z - (int)(b * splits);
+  const int64_t kbeg = (int64_t)split * kchunk, kend = min(g.K, kbeg + kchunk);
+  const int64_t m0 = (int64_t)blockIdx.y * BM, n0 = (int64_t)blockIdx.x * BN;
+  const int tid = threadIdx.x, tn = tid % BN, tm = tid / BN;
+  const zc* Ab = A + midx_off(g.bA, b);
+  const zc* Bb = B + midx_off(g.bB, b);
+  const bool a_kfast = midx_unit_inner(g.kA) && !midx_unit_inner(g.mA);
+  const bool b_kfast = midx_unit_inner(g.kB) && !midx_unit_inner(g.nB);
+  constexpr int LA = (BM * BK + NT - 1) / NT, LB = (BN * BK + NT - 1) / NT;
+  zc ra[LA], rb[LB];
+  auto fetch = [&](int64_t k0) {
+#pragma unroll
+    for (int l = 0; l < LA; ++l) {
+      const int e = tid + l * NT, mm = a_kfast ? e / BK : e % BM, kk = a_kfast ? e % BK : e / BM;
+      zc v(0, 0);
+      if (e < BM * BK && m0 + mm < g.M && k0 + kk < kend) {
+        v = Ab[midx_off(g.mA, m0 + mm) + midx_off(g.kA, k0 + kk)];
+        if (g.conjA) v.im = -v.im;
+      }
+      ra[l] = v;
+    }
+#pragma unroll
+    for (int l = 0; l < LB; ++l) {
+      const int e = tid + l * NT, nn = b_kfast ? e / BK : e % BN, kk = b_kfast ? e % BK : e / BN;
+      zc v(0, 0);
+      if (e < BN * BK && n0 + nn < g.N && k0 + kk < kend) {
+        v = Bb[midx_off(g.nB, n0 + nn) + midx_off(g.kB, k0 + kk)];
+        if (g.conjB) v.im = -v.im;
+      }
+      rb[l] = v;
+    }
+  };
+  zc acc(0, 0);
+  if (kbeg < kend) fetch(kbeg);
+  for (int64_t k0 = kbeg; k0 < kend; k0 += BK) {
+#pragma unroll
+    for (int l = 0; l < LA; ++l) {
+      const int e = tid + l * NT;
+      if (e < BM * BK) As[a_kfast ? e % BK : e / BM][a_kfast ? e / BK : e % BM] = ra[l];
+    }
+#pragma unroll
+    for (int l = 0; l < LB; ++l) {
+      const int e = tid + l * NT;
+      if (e < BN * BK) Bs[b_kfast ? e % BK : e / BN][b_kfast ? e / BK : e % BN] = rb[l];
+    }
+    __syncthreads();
+    if (k0 + BK < kend) fetch(k0 + BK);
+    const int kn = (int)min((int64_t)BK, kend - k0);
+    if (kn == BK) {
+#pragma unroll
+      for (int kk = 0; kk < BK; ++kk) cfma(acc, As[kk][tm], Bs[kk][tn]);
+    } else {
+      for (int kk = 0; kk < kn; ++kk) cfma(acc, As[kk][tm], Bs[kk][tn]);
+    }
+    __syncthreads();
+  }
+  const int64_t m = m0 + tm, n = n0 + tn;
+  if (m >= g.M || n >= g.N) return;
+  if (splits > 1) {
+    P[(((int64_t)split * g.batch + b) * g.M + m) * g.N + n] = acc;
+    return;
+  }
+  const int64_t o = midx_off(g.bC, b) + midx_off(g.mC, m) + midx_off(g.nC, n);
+  zc v = alpha * acc;
+  if (beta.re != 0.0 || beta.im != 0.0) v = v + beta * C[o];
+  C[o] = v;
+}
+
 // C[b][m][n] = alpha sum_s P[s][b][m][n] + beta C[b][m][n], summed in split order
 template <class R>
 __global__ void splitk_reduce_kernel(GemmDesc g, cplx<R> alpha, cplx<R> beta, const cplx<R>* __restrict__ P,
@@ -187,6 +270,63 @@ __global__ void splitk_reduce_kernel(GemmDesc g, cplx<R> alpha, cplx<R> beta, co
 }
 
 }  // namespace
+
+// FP64 tile (BM, BN): 64 x 64 outputs (gemm_midx_kernel) where that makes two
+// waves of CTAs; else one output per thread, 256 per CTA where that fills the
+// SMs and 64 where not, the tile four wide in a dimension of at most four.
+static void f64_tile(const GemmDesc& g, int* bm, int* bn) {
+  const int64_t t64 = ((g.M + 63) / 64) * ((g.N + 63) / 64) * g.batch;
+  if (g.M > 32 && g.N > 32 && t64 >= 304) {
+    *bm = *bn = 64;
+    return;
+  }
+  const bool big = (g.M * g.N * g.batch) / 256 >= 152;
+  if (g.N <= 4) {
+    *bm = big ? 64 : 16;
+    *bn = 4;
+  } else if (g.M <= 4) {
+    *bm = 4;
+    *bn = big ? 64 : 16;
+  } else {
+    *bm = *bn = big && g.M > 8 && g.N > 8 ? 16 : 8;
+  }
+}
+
+// K splits of an FP64 contraction: about one CTA per SM, at least 64 of K each
+int qtt_gemm_splits_f64(const GemmDesc& g) {
+  int bm, bn;
+  f64_tile(g, &bm, &bn);
+  const int64_t tiles = ((g.M + bm - 1) / bm) * ((g.N + bn - 1) / bn) * g.batch;
+  if (tiles >= 76 || g.K < 128) return 1;
+  return (int)std::min<int64_t>(32, std::min<int64_t>((g.K + 63) / 64, std::max<int64_t>(1, 152 / tiles)));
+}
+
+static int launch_f64(const GemmDesc& g, zc alpha, zc beta, const zc* A, const zc* B, zc* C, int splits,
+                      int64_t kchunk, zc* P, cudaStream_t s) {
+  int bm, bn;
+  f64_tile(g, &bm, &bn);
+  // a grid has at most 65535 tiles along m: taller ones take the wide tile
+  if ((g.M + bm - 1) / bm > 65535) bm = bn = 64;
+  const dim3 grid((unsigned)((g.N + bn - 1) / bn), (unsigned)((g.M + bm - 1) / bm), (unsigned)(g.batch * splits));
+  if (grid.y > 65535) return QTT_ERR_ARG;
+#define QTT_F64(X, Y) gemm_f64_kernel<X, Y><<<grid, X * Y, 0, s>>>(g, alpha, beta, A, B, C, splits, kchunk, P)
+  if (bm == 64 && bn == 64)
+    gemm_midx_kernel<double, 64, 64, 8, 4, 4><<<grid, 256, 0, s>>>(g, alpha, beta, A, B, C, splits, kchunk, P);
+  else if (bm == 16 && bn == 16)
+    QTT_F64(16, 16);
+  else if (bm == 8)
+    QTT_F64(8, 8);
+  else if (bm == 64)
+    QTT_F64(64, 4);
+  else if (bm == 16)
+    QTT_F64(16, 4);
+  else if (bn == 64)
+    QTT_F64(4, 64);
+  else
+    QTT_F64(4, 16);
+#undef QTT_F64
+  return QTT_OK;
+}
 
 // Tile edge of qtt_gemm_ex: 64, or 32 for thin shapes and for grids of
 // 64 x 64 tiles that would not fill a quarter of the SMs.
@@ -217,7 +357,10 @@ int qtt_gemm_ex(const GemmDesc& g, cplx<R> alpha, cplx<R> beta, const cplx<R>* A
   constexpr int BK = sizeof(R) == 8 ? 8 : 16;
   const int64_t zdim = g.batch * splits;
   if (zdim > 65535) return QTT_ERR_ARG;
-  if (thin) {
+  if constexpr (sizeof(R) == 8) {
+    const int st = launch_f64(g, alpha, beta, A, B, C, splits, kchunk, P, s);
+    if (st != QTT_OK) return st;
+  } else if (thin) {
     dim3 grid((unsigned)((g.N + 31) / 32), (unsigned)((g.M + 31) / 32), (unsigned)zdim);
     if (grid.y > 65535) return QTT_ERR_ARG;
     gemm_midx_kernel<R, 32, 32, BK, 2, 2><<<grid, 256, 0, s>>>(g, alpha, beta, A, B, C, splits, kchunk, P);

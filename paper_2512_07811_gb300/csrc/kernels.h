@@ -12,6 +12,7 @@ int qtt_gemm(const GemmDesc& g, cplx<R> alpha, cplx<R> beta, const cplx<R>* A, c
 
 // split-K aware variant: `splits` K ranges, partials in P (splits x batch x M x N), see qtt_gemm_splits
 int qtt_gemm_splits(const GemmDesc& g);
+int qtt_gemm_splits_f64(const GemmDesc& g);  // the same for FP64 contractions (tile chosen by shape, never tuned)
 // tile: 0 = the rule (gemm_tile), else 32 or 64
 template <class R>
 int qtt_gemm_ex(const GemmDesc& g, cplx<R> alpha, cplx<R> beta, const cplx<R>* A, const cplx<R>* B, cplx<R>* C,
