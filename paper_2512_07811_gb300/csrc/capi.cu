@@ -109,14 +109,17 @@ int tt_finite(qtt_ctx* c, const qtt_tt* x, int* finite) {
   void* flag;
   TRY(dalloc(c, &flag, sizeof(int)));
   cudaMemsetAsync(flag, 0, sizeof(int), c->stream);
-  for (int k = 0; k < x->d; ++k) {
-    int64_t cnt = (int64_t)x->r[k] * x->n[k] * x->r[k + 1];
+  each_table(x->d, [&](int k0, int n) {
+    CoreTable t;
+    t.n = n;
+    for (int i = 0; i < n; ++i) {
+      t.src[i] = core_ptr<char>(x, k0 + i);
+      t.cnt[i] = (int64_t)x->r[k0 + i] * x->n[k0 + i] * x->r[k0 + i + 1];
+    }
     c->launches++;
-    if (x->dtype == QTT_C128)
-      qtt_isfinite<double>(core_ptr<zc>(x, k), cnt, reinterpret_cast<int*>(flag), c->stream);
-    else
-      qtt_isfinite<float>(core_ptr<cc>(x, k), cnt, reinterpret_cast<int*>(flag), c->stream);
-  }
+    return x->dtype == QTT_C128 ? qtt_cores_isfinite<double>(t, reinterpret_cast<int*>(flag), c->stream)
+                                : qtt_cores_isfinite<float>(t, reinterpret_cast<int*>(flag), c->stream);
+  });
   int h = 0;
   int s = sync_read(c, &h, flag, sizeof(int));
   dfree(c, flag);
@@ -161,44 +164,62 @@ int make_sketch(qtt_ctx* c, const std::vector<int>& modes, const std::vector<int
   int st;
   qtt_tt* S = tt_alloc(c, d, modes, r, dt, &st);
   if (!S) return st;
-  for (int k = 0; k < d; ++k) {
-    int64_t cnt = (int64_t)r[k] * modes[k] * r[k + 1];
-    double scale = 1.0 / sqrt((double)modes[k] * r[k + 1]);
-    const int64_t M = (int64_t)modes[k] * r[k + 1];
-    c->launches++;
-    int s;
-    if (k > 0 && r[k] == M)
-      s = dt == QTT_C128 ? qtt_identity_core<double>(1, M, core_ptr<zc>(S, k), c->stream)
-                         : qtt_identity_core<float>(1, M, core_ptr<cc>(S, k), c->stream);
-    else
-      s = dt == QTT_C128
-              ? qtt_fill_gaussian<double>(core_ptr<zc>(S, k), cnt, seed, (stream_id << 8) + k, scale, c->stream)
-              : qtt_fill_gaussian<float>(core_ptr<cc>(S, k), cnt, seed, (stream_id << 8) + k, scale, c->stream);
-    if (s) {
-      tt_free(S);
-      return s;
+  const int s = each_table(d, [&](int k0, int n) {
+    SketchTable t;
+    t.n = n;
+    t.seed = seed;
+    t.stream = (stream_id << 8) + k0;
+    for (int i = 0; i < n; ++i) {
+      const int k = k0 + i;
+      const int64_t M = (int64_t)modes[k] * r[k + 1];
+      t.dst[i] = core_ptr<char>(S, k);
+      t.cnt[i] = (int64_t)r[k] * M;
+      t.M[i] = k > 0 && r[k] == M ? M : 0;
+      t.scale[i] = 1.0 / sqrt((double)M);
     }
+    c->launches++;
+    return dt == QTT_C128 ? qtt_fill_sketch<double>(t, c->stream) : qtt_fill_sketch<float>(t, c->stream);
+  });
+  if (s) {
+    tt_free(S);
+    return s;
   }
   *out = S;
   return QTT_OK;
+}
+
+// one launch over the cores: dst[k] = src[k] in dtype `dt` (from dtype `from`)
+static int move_cores(qtt_ctx* c, int d, qtt_dtype from, qtt_dtype dt, const std::vector<const void*>& src,
+                      const std::vector<void*>& dst, const std::vector<int64_t>& cnt) {
+  return each_table(d, [&](int k0, int n) {
+    CoreTable t;
+    t.n = n;
+    for (int i = 0; i < n; ++i) {
+      t.src[i] = src[k0 + i];
+      t.dst[i] = dst[k0 + i];
+      t.cnt[i] = cnt[k0 + i];
+    }
+    c->launches++;
+    return qtt_cores_move(t, from == dt ? 0 : (dt == QTT_C64 ? 1 : 2), (int)dtype_size(dt), c->stream);
+  });
 }
 
 int convert_tt(qtt_ctx* c, const qtt_tt* x, qtt_dtype dt, qtt_tt** out) {
   int st;
   qtt_tt* y = tt_alloc(c, x->d, x->n, x->r, dt, &st);
   if (!y) return st;
+  std::vector<const void*> src(x->d);
+  std::vector<void*> dst(x->d);
+  std::vector<int64_t> cnt(x->d);
   for (int k = 0; k < x->d; ++k) {
-    int64_t cnt = (int64_t)x->r[k] * x->n[k] * x->r[k + 1];
-    if (x->dtype == dt) {
-      cudaMemcpyAsync(core_ptr<char>(y, k), core_ptr<char>(x, k), cnt * dtype_size(dt), cudaMemcpyDeviceToDevice,
-                      c->stream);
-    } else if (dt == QTT_C64) {
-      c->launches++;
-      qtt_convert_z2c(core_ptr<zc>(x, k), core_ptr<cc>(y, k), cnt, c->stream);
-    } else {
-      c->launches++;
-      qtt_convert_c2z(core_ptr<cc>(x, k), core_ptr<zc>(y, k), cnt, c->stream);
-    }
+    src[k] = core_ptr<char>(x, k);
+    dst[k] = core_ptr<char>(y, k);
+    cnt[k] = (int64_t)x->r[k] * x->n[k] * x->r[k + 1];
+  }
+  st = move_cores(c, x->d, x->dtype, dt, src, dst, cnt);
+  if (st) {
+    tt_free(y);
+    return st;
   }
   *out = y;
   return QTT_OK;
@@ -209,18 +230,19 @@ int convert_mpo(qtt_ctx* c, const qtt_mpo* A, qtt_dtype dt, qtt_mpo** out) {
   qtt_mpo* B = mpo_alloc(c, A->d, A->no, A->ni, A->g, dt, &st);
   if (!B) return st;
   B->diag = A->diag;
+  B->ident = A->ident;
+  std::vector<const void*> src(A->d);
+  std::vector<void*> dst(A->d);
+  std::vector<int64_t> cnt(A->d);
   for (int k = 0; k < A->d; ++k) {
-    int64_t cnt = (int64_t)A->g[k] * A->no[k] * A->ni[k] * A->g[k + 1];
-    if (A->dtype == dt) {
-      cudaMemcpyAsync(core_ptr<char>(B, k), core_ptr<char>(A, k), cnt * dtype_size(dt), cudaMemcpyDeviceToDevice,
-                      c->stream);
-    } else if (dt == QTT_C64) {
-      c->launches++;
-      qtt_convert_z2c(core_ptr<zc>(A, k), core_ptr<cc>(B, k), cnt, c->stream);
-    } else {
-      c->launches++;
-      qtt_convert_c2z(core_ptr<cc>(A, k), core_ptr<zc>(B, k), cnt, c->stream);
-    }
+    src[k] = core_ptr<char>(A, k);
+    dst[k] = core_ptr<char>(B, k);
+    cnt[k] = (int64_t)A->g[k] * A->no[k] * A->ni[k] * A->g[k + 1];
+  }
+  st = move_cores(c, A->d, A->dtype, dt, src, dst, cnt);
+  if (st) {
+    mpo_free(B);
+    return st;
   }
   *out = B;
   return QTT_OK;
@@ -1128,7 +1150,7 @@ int build_ops(qtt_ctx* c, const qtt_rve* rve, const double* C1, const double* C2
   for (int k = 1; k < d; ++k) {
     c->launches++;
     TRY(qtt_identity_core<double>(1, 2, core_ptr<zc>(ops->dCa, k), c->stream));
-    ops->dCa->diag[k] = 1;
+    ops->dCa->diag[k] = ops->dCa->ident[k] = 1;
   }
   // bond k of the full operator sits between site k-1 and site k; spatial
   // site k holds phase core k-1, so bond k equals the phase train's bond k-1
@@ -1180,6 +1202,7 @@ int build_ops(qtt_ctx* c, const qtt_rve* rve, const double* C1, const double* C2
     c->launches++;
     qtt_identity_core<double>(1, nc, core_ptr<zc>(Q, 0), c->stream);
     Q->diag[0] = Qi->diag[0] = 1;
+    Q->ident[0] = Qi->ident[0] = 1;
     for (int p = 0; p < dsp; ++p) {
       const int dm = sm.dim[p], pos = sm.pos[p];
       const int k = p + 1;
@@ -1240,29 +1263,19 @@ int ms_solve(qtt_ctx* c, const qtt_rve* rve, const double* C1h, const double* C2
   uint64_t call = 1;
   int st;
   // unit E trains, probe trains e_I (x) ones, e_I (x) chi
-  auto make_rank1 = [&](const std::vector<double>& ctrl, const qtt_tt* spatial, qtt_tt** out) -> int {
-    std::vector<int> r(d + 1, 1);
-    if (spatial)
-      for (int k = 1; k <= d; ++k) r[k] = spatial->r[k - 1];
-    qtt_tt* x = tt_alloc(c, d, modes, r, dt, &st);
+  auto make_constant = [&](const std::vector<double>& ctrl, qtt_tt** out) -> int {
+    qtt_tt* x = tt_alloc(c, d, modes, std::vector<int>(d + 1, 1), dt, &st);
     if (!x) return st;
-    std::vector<C> h(nc);
-    for (int i = 0; i < nc; ++i) h[i] = C((R)ctrl[i], 0);
-    TRY(upload(c, core_ptr<char>(x, 0), h.data(), nc * sizeof(C)));
+    std::vector<char> h(x->bytes, 0);
+    for (int i = 0; i < nc; ++i) reinterpret_cast<C*>(h.data())[i] = C((R)ctrl[i], 0);
     for (int k = 1; k < d; ++k) {
-      if (spatial) {
-        int64_t cnt = (int64_t)spatial->r[k - 1] * 2 * spatial->r[k];
-        if (dt == QTT_C128) {
-          cudaMemcpyAsync(core_ptr<char>(x, k), core_ptr<char>(spatial, k - 1), cnt * sizeof(zc),
-                          cudaMemcpyDeviceToDevice, c->stream);
-        } else {
-          c->launches++;
-          qtt_convert_z2c(core_ptr<zc>(spatial, k - 1), core_ptr<cc>(x, k), cnt, c->stream);
-        }
-      } else {
-        C two[2] = {C(1, 0), C(1, 0)};
-        TRY(upload(c, core_ptr<char>(x, k), two, sizeof(two)));
-      }
+      C* core = reinterpret_cast<C*>(h.data() + x->off[k]);
+      core[0] = core[1] = C(1, 0);
+    }
+    const int s = upload(c, x->data, h.data(), x->bytes);
+    if (s) {
+      tt_free(x);
+      return s;
     }
     *out = x;
     return QTT_OK;
@@ -1505,7 +1518,7 @@ int ms_solve(qtt_ctx* c, const qtt_rve* rve, const double* C1h, const double* C2
     std::vector<double> e(nc, 0.0);
     e[lc] = 1.0;
     qtt_tt* E = nullptr;
-    TRY(make_rank1(e, nullptr, &E));
+    TRY(make_constant(e, &E));
     const double normE = sqrt(Nvox);
     qtt_tt* x = nullptr;
     TRY(convert_tt(c, E, dt, &x));
@@ -1682,22 +1695,20 @@ int ms_solve(qtt_ctx* c, const qtt_rve* rve, const double* C1h, const double* C2
     if (it > o.max_iter) it = o.max_iter;
     // sigma = C1 <eps> + (C2 - C1) <chi eps>
     std::vector<double> m1(2 * nc), m2(2 * nc);
-    for (int I = 0; I < nc; ++I) {
-      std::vector<double> eI(nc, 0.0);
-      eI[I] = 1.0;
-      qtt_tt *u = nullptr, *v = nullptr;
-      TRY(make_rank1(eI, nullptr, &u));
-      TRY(make_rank1(eI, O.chi, &v));
-      double a[2], b[2];
-      int s = dot_dev<R>(c, u, x, a);
-      if (!s) s = dot_dev<R>(c, v, x, b);
-      tt_free(u);
-      tt_free(v);
-      if (s) return s;
-      m1[2 * I] = a[0] / Nvox;
-      m1[2 * I + 1] = a[1] / Nvox;
-      m2[2 * I] = b[0] / Nvox;
-      m2[2 * I + 1] = b[1] / Nvox;
+    {
+      struct Held {
+        qtt_tt* p = nullptr;
+        ~Held() { tt_free(p); }
+      } chi_r;
+      const qtt_tt* chi = O.chi;
+      if (chi && chi->dtype != dt) {
+        TRY(convert_tt(c, O.chi, dt, &chi_r.p));
+        chi = chi_r.p;
+      }
+      TRY(control_sums<R>(c, x, nullptr, m1.data()));
+      TRY(control_sums<R>(c, x, chi, m2.data()));
+      for (auto& v : m1) v /= Nvox;
+      for (auto& v : m2) v /= Nvox;
     }
     for (int I = 0; I < nc; ++I) {
       double sr = 0, si = 0;

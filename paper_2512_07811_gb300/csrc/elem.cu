@@ -276,18 +276,91 @@ __device__ __forceinline__ void philox4x32_10(uint32_t ctr[4], uint32_t key[2]) 
 // Real Gaussian entries N(0, scale^2) stored as complex with zero imaginary
 // part: Box-Muller on two 32-bit uniforms per entry; counter = (index, stream).
 template <class R>
+__device__ __forceinline__ cplx<R> gaussian_entry(int64_t e, uint64_t seed, uint64_t stream, double scale) {
+  uint32_t ctr[4] = {(uint32_t)e, (uint32_t)((uint64_t)e >> 32), (uint32_t)stream, (uint32_t)(stream >> 32)};
+  uint32_t key[2] = {(uint32_t)seed, (uint32_t)(seed >> 32)};
+  philox4x32_10(ctr, key);
+  double u1 = ((double)ctr[0] + 0.5) * 2.3283064365386963e-10;   // (0, 1)
+  double u2 = ((double)ctr[1] + 0.5) * 2.3283064365386963e-10;
+  double rad = sqrt(-2.0 * log(u1));
+  double sn, cs;
+  sincospi(2.0 * u2, &sn, &cs);
+  return cplx<R>((R)(scale * rad * cs), R(0));
+}
+
+template <class R>
 __global__ void gaussian_kernel(cplx<R>* out, int64_t count, uint64_t seed, uint64_t stream, double scale) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < count;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    uint32_t ctr[4] = {(uint32_t)e, (uint32_t)((uint64_t)e >> 32), (uint32_t)stream, (uint32_t)(stream >> 32)};
-    uint32_t key[2] = {(uint32_t)seed, (uint32_t)(seed >> 32)};
-    philox4x32_10(ctr, key);
-    double u1 = ((double)ctr[0] + 0.5) * 2.3283064365386963e-10;   // (0, 1)
-    double u2 = ((double)ctr[1] + 0.5) * 2.3283064365386963e-10;
-    double rad = sqrt(-2.0 * log(u1));
-    double sn, cs;
-    sincospi(2.0 * u2, &sn, &cs);
-    out[e] = cplx<R>((R)(scale * rad * cs), R(0));
+       e += (int64_t)gridDim.x * blockDim.x)
+    out[e] = gaussian_entry<R>(e, seed, stream, scale);
+}
+
+// The cores of a train in one launch (blockIdx.y = core): a core is small and a
+// launch of its own costs more than its bytes.
+__global__ void cores_move_kernel(const __grid_constant__ CoreTable t, int what, int elem) {
+  const int k = blockIdx.y;
+  const int64_t n = t.cnt[k];
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+    if (what == 1) {
+      const zc v = static_cast<const zc*>(t.src[k])[e];
+      static_cast<cc*>(t.dst[k])[e] = cc((float)v.re, (float)v.im);
+    } else if (what == 2) {
+      const cc v = static_cast<const cc*>(t.src[k])[e];
+      static_cast<zc*>(t.dst[k])[e] = zc((double)v.re, (double)v.im);
+    } else if (elem == 8) {
+      static_cast<cc*>(t.dst[k])[e] = static_cast<const cc*>(t.src[k])[e];
+    } else {
+      static_cast<zc*>(t.dst[k])[e] = static_cast<const zc*>(t.src[k])[e];
+    }
+  }
+}
+
+template <class R>
+__global__ void cores_isfinite_kernel(const __grid_constant__ CoreTable t, int* flag) {
+  const int k = blockIdx.y;
+  const cplx<R>* x = static_cast<const cplx<R>*>(t.src[k]);
+  const int64_t n = t.cnt[k];
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
+    if (!isfinite(x[e].re) || !isfinite(x[e].im)) atomicExch(flag, 1);
+}
+
+template <class R>
+__global__ void fill_sketch_kernel(const __grid_constant__ SketchTable t) {
+  const int k = blockIdx.y;
+  cplx<R>* out = static_cast<cplx<R>*>(t.dst[k]);
+  const int64_t n = t.cnt[k], M = t.M[k];
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
+    out[e] = M > 0 ? cplx<R>(e / M == e % M ? R(1) : R(0), R(0))
+                   : gaussian_entry<R>(e, t.seed, t.stream + (uint64_t)k, t.scale[k]);
+}
+
+template <class R>
+__global__ void add_cores_kernel(const __grid_constant__ AddTable<R> t) {
+  const int k = blockIdx.y;
+  const bool first = k == t.first, last = k == t.last;
+  const int xa = t.xa[k], xb = t.xb[k], ya = t.ya[k], yb = t.yb[k], n = t.nk[k];
+  const int za = first ? 1 : xa + ya, zb = last ? 1 : xb + yb;
+  const int64_t total = (int64_t)za * n * zb;
+  const cplx<R>* x = t.x[k];
+  const cplx<R>* y = t.y[k];
+  cplx<R>* z = t.z[k];
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    const int c = (int)(e % zb);
+    const int64_t u = e / zb;
+    const int j = (int)(u % n), r = (int)(u / n);
+    const int ry = first ? r : r - xa, cy = last ? c : c - xb;
+    cplx<R> v(0, 0);
+    // x in the leading rows and columns; on the first core row 0 is x's in the
+    // leading columns and y's beyond, on the last core column 0 likewise by rows
+    // (a train of one core does not come here)
+    if (r < xa && c < xb) {
+      v = x[((int64_t)r * n + j) * xb + c];
+      if (first && !t.ua) v = mul_rn(t.a, v);
+    } else if (ry >= 0 && cy >= 0) {
+      v = y[((int64_t)ry * n + j) * yb + cy];
+      if (first && !t.ub) v = mul_rn(t.b, v);
+    }
+    z[e] = v;
   }
 }
 
@@ -623,3 +696,41 @@ template int qtt_herm_shift<double>(const zc*, int64_t, double, zc*, cudaStream_
 template int qtt_herm_shift<float>(const cc*, int64_t, double, cc*, cudaStream_t);
 template int qtt_half_identity_plus<double>(zc*, int64_t, double*, cudaStream_t);
 template int qtt_half_identity_plus<float>(cc*, int64_t, double*, cudaStream_t);
+
+static int64_t table_max(const int64_t* cnt, int n) {
+  int64_t m = 1;
+  for (int k = 0; k < n; ++k) m = std::max(m, cnt[k]);
+  return m;
+}
+static dim3 table_grid(int64_t max_count, int n) {
+  return dim3((unsigned)std::min<int64_t>((max_count + 255) / 256, 512), (unsigned)n);
+}
+int qtt_cores_move(const CoreTable& t, int what, int elem, cudaStream_t s) {
+  if (t.n <= 0) return QTT_OK;
+  cores_move_kernel<<<table_grid(table_max(t.cnt, t.n), t.n), 256, 0, s>>>(t, what, elem);
+  return cudaGetLastError() == cudaSuccess ? QTT_OK : QTT_ERR_CUDA;
+}
+template <class R>
+int qtt_cores_isfinite(const CoreTable& t, int* flag, cudaStream_t s) {
+  if (t.n <= 0) return QTT_OK;
+  cores_isfinite_kernel<R><<<table_grid(table_max(t.cnt, t.n), t.n), 256, 0, s>>>(t, flag);
+  return cudaGetLastError() == cudaSuccess ? QTT_OK : QTT_ERR_CUDA;
+}
+template <class R>
+int qtt_fill_sketch(const SketchTable& t, cudaStream_t s) {
+  if (t.n <= 0) return QTT_OK;
+  fill_sketch_kernel<R><<<table_grid(table_max(t.cnt, t.n), t.n), 256, 0, s>>>(t);
+  return cudaGetLastError() == cudaSuccess ? QTT_OK : QTT_ERR_CUDA;
+}
+template <class R>
+int qtt_add_cores(const AddTable<R>& t, int64_t max_count, cudaStream_t s) {
+  if (t.n <= 0) return QTT_OK;
+  add_cores_kernel<R><<<table_grid(max_count, t.n), 256, 0, s>>>(t);
+  return cudaGetLastError() == cudaSuccess ? QTT_OK : QTT_ERR_CUDA;
+}
+template int qtt_cores_isfinite<double>(const CoreTable&, int*, cudaStream_t);
+template int qtt_cores_isfinite<float>(const CoreTable&, int*, cudaStream_t);
+template int qtt_fill_sketch<double>(const SketchTable&, cudaStream_t);
+template int qtt_fill_sketch<float>(const SketchTable&, cudaStream_t);
+template int qtt_add_cores<double>(const AddTable<double>&, int64_t, cudaStream_t);
+template int qtt_add_cores<float>(const AddTable<float>&, int64_t, cudaStream_t);

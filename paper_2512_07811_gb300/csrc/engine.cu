@@ -156,6 +156,7 @@ qtt_mpo* mpo_alloc(qtt_ctx* c, int d, const std::vector<int>& no, const std::vec
   A->ni = ni;
   A->g = g;
   A->diag.assign(d, 0);
+  A->ident.assign(d, 0);
   A->dtype = dt;
   A->off.resize(d);
   size_t tot = 0;
@@ -1128,14 +1129,21 @@ int round_det(qtt_ctx* c, const qtt_tt* x, double eps, int max_rank, const int* 
   int st;
   qtt_tt* y = tt_alloc(c, d, n, nr, x->dtype, &st);
   if (!y) return st;
-  for (int k = 0; k < d; ++k) {
-    const void* src = (k == 0) ? (const void*)T : newc[k].p;
-    size_t bytes = (size_t)nr[k] * n[k] * nr[k + 1] * sizeof(cplx<R>);
-    if (cudaMemcpyAsync(static_cast<char*>(y->data) + y->off[k], src, bytes, cudaMemcpyDeviceToDevice, c->stream) !=
-        cudaSuccess) {
-      tt_free(y);
-      return QTT_ERR_CUDA;
+  st = each_table(d, [&](int k0, int cnt) {
+    CoreTable t;
+    t.n = cnt;
+    for (int i = 0; i < cnt; ++i) {
+      const int k = k0 + i;
+      t.src[i] = (k == 0) ? (const void*)T : newc[k].p;
+      t.dst[i] = static_cast<char*>(y->data) + y->off[k];
+      t.cnt[i] = (int64_t)nr[k] * n[k] * nr[k + 1];
     }
+    c->launches++;
+    return qtt_cores_move(t, 0, sizeof(cplx<R>), c->stream);
+  });
+  if (st) {
+    tt_free(y);
+    return st;
   }
   (void)Trows;
   if (info) {
@@ -1448,15 +1456,46 @@ int add_dev(qtt_ctx* c, cplx<R> a, const qtt_tt* x, cplx<R> b, const qtt_tt* y, 
   int st;
   qtt_tt* z = tt_alloc(c, d, x->n, r, x->dtype, &st);
   if (!z) return st;
-  cudaMemsetAsync(z->data, 0, z->bytes, c->stream);
   typedef cplx<R> C;
   const C one(1, 0);
+  if (d > 1) {
+    st = each_table(d, [&](int k0, int cnt) {
+      AddTable<R> t;
+      t.n = cnt;
+      t.first = k0 == 0 ? 0 : -1;
+      t.last = k0 + cnt == d ? cnt - 1 : -1;
+      t.a = a;
+      t.b = b;
+      t.ua = a.re == R(1) && a.im == R(0);
+      t.ub = b.re == R(1) && b.im == R(0);
+      int64_t most = 1;
+      for (int i = 0; i < cnt; ++i) {
+        const int k = k0 + i;
+        t.x[i] = core_ptr<C>(x, k);
+        t.y[i] = core_ptr<C>(y, k);
+        t.z[i] = core_ptr<C>(z, k);
+        t.xa[i] = x->r[k];
+        t.xb[i] = x->r[k + 1];
+        t.ya[i] = y->r[k];
+        t.yb[i] = y->r[k + 1];
+        t.nk[i] = x->n[k];
+        most = std::max<int64_t>(most, (int64_t)r[k] * x->n[k] * r[k + 1]);
+      }
+      c->launches++;
+      return qtt_add_cores<R>(t, most, c->stream);
+    });
+    if (st) {
+      tt_free(z);
+      return st;
+    }
+    *out = z;
+    return QTT_OK;
+  }
+  cudaMemsetAsync(z->data, 0, z->bytes, c->stream);
   for (int k = 0; k < d; ++k) {
     const int64_t n = x->n[k];
-    const int64_t xa = x->r[k], xb = x->r[k + 1], ya = y->r[k], yb = y->r[k + 1];
     C* Z = core_ptr<C>(z, k);
-    const int64_t zb = r[k + 1];
-    if (d == 1) {
+    {
       // z = a x + b y elementwise (single core)
       c->launches += 2;
       int s1 = qtt_place_block<R>(core_ptr<C>(x, 0), 1, n, 1, Z, 1, 0, 0, a, c->stream);
@@ -1491,16 +1530,6 @@ int add_dev(qtt_ctx* c, cplx<R> a, const qtt_tt* x, cplx<R> b, const qtt_tt* y, 
         return s2;
       }
       break;
-    }
-    const int64_t xoff0 = 0, xoff1 = 0;
-    const int64_t yoff0 = (k == 0) ? 0 : xa;
-    const int64_t yoff1 = (k == d - 1) ? 0 : xb;
-    c->launches += 2;
-    int s1 = qtt_place_block<R>(core_ptr<C>(x, k), xa, n, xb, Z, zb, xoff0, xoff1, k == 0 ? a : one, c->stream);
-    int s2 = qtt_place_block<R>(core_ptr<C>(y, k), ya, n, yb, Z, zb, yoff0, yoff1, k == 0 ? b : one, c->stream);
-    if (s1 || s2) {
-      tt_free(z);
-      return s1 ? s1 : s2;
     }
   }
   *out = z;
@@ -1620,6 +1649,75 @@ int dot_dev(qtt_ctx* c, const qtt_tt* x, const qtt_tt* y, double out[2]) {
 template int dot_dev<double>(qtt_ctx*, const qtt_tt*, const qtt_tt*, double*);
 template int dot_dev<float>(qtt_ctx*, const qtt_tt*, const qtt_tt*, double*);
 
+// One chain for every control index: W (nc x (ra) x rb) starts as the control core.
+template <class R>
+int control_sums(qtt_ctx* c, const qtt_tt* x, const qtt_tt* chi, double* out) {
+  typedef cplx<R> C;
+  const int d = x->d, nc = x->n[0];
+  DBuf W;
+  const C* w = core_ptr<C>(x, 0);  // (1, nc, r_1)
+  int64_t ra = 1;
+  for (int k = 1; k < d; ++k) {
+    const int64_t b0 = x->r[k], b1 = x->r[k + 1], n = x->n[k];
+    const C* B = core_ptr<C>(x, k);
+    DBuf Wn;
+    if (!chi) {
+      // W'[I, b1] = sum_{i, b0} W[I, b0] B[b0, i, b1]
+      TRY(Wn.alloc(c, (size_t)nc * b1 * sizeof(C)));
+      GemmDesc g;
+      g.bA = g.bB = g.bC = B0();
+      g.M = nc;
+      g.N = b1;
+      g.K = n * b0;
+      g.batch = 1;
+      g.mA = L1(nc, b0);
+      g.kA = L2(n, 0, b0, 1);
+      g.kB = L2(n, b1, b0, n * b1);
+      g.nB = L1(b1, 1);
+      g.mC = L1(nc, b1);
+      g.nC = L1(b1, 1);
+      g.conjA = g.conjB = 0;
+      TRY(gemm<R>(c, g, w, B, Wn.as<C>()));
+    } else {
+      // T[(I, a0), (i, b1)] = W[(I, a0), b0] B[b0, (i, b1)]; W'[I, a1, b1] = sum_{a0, i} conj(A[a0, i, a1]) T
+      const int64_t ra1 = chi->r[k];
+      DBuf Tm;
+      TRY(Tm.alloc(c, (size_t)nc * ra * n * b1 * sizeof(C)));
+      TRY(mm<R>(c, nc * ra, n * b1, b0, w, b0, 1, 0, B, n * b1, 1, 0, Tm.as<C>(), n * b1, 1));
+      TRY(Wn.alloc(c, (size_t)nc * ra1 * b1 * sizeof(C)));
+      GemmDesc g;
+      g.M = ra1;
+      g.N = b1;
+      g.K = ra * n;
+      g.batch = nc;
+      g.bA = L1(nc, 0);
+      g.mA = L1(ra1, 1);
+      g.kA = L1(ra * n, ra1);
+      g.bB = L1(nc, ra * n * b1);
+      g.kB = L1(ra * n, b1);
+      g.nB = L1(b1, 1);
+      g.bC = L1(nc, ra1 * b1);
+      g.mC = L1(ra1, b1);
+      g.nC = L1(b1, 1);
+      g.conjA = 1;
+      g.conjB = 0;
+      TRY(gemm<R>(c, g, core_ptr<C>(chi, k - 1), Tm.as<C>(), Wn.as<C>()));
+      ra = ra1;
+    }
+    W = std::move(Wn);
+    w = W.as<C>();
+  }
+  std::vector<C> h(nc);
+  TRY(sync_read(c, h.data(), w, (size_t)nc * sizeof(C)));
+  for (int i = 0; i < nc; ++i) {
+    out[2 * i] = (double)h[i].re;
+    out[2 * i + 1] = (double)h[i].im;
+  }
+  return QTT_OK;
+}
+template int control_sums<double>(qtt_ctx*, const qtt_tt*, const qtt_tt*, double*);
+template int control_sums<float>(qtt_ctx*, const qtt_tt*, const qtt_tt*, double*);
+
 // Frobenius norm: R factor sweep, then the norm of the centre.
 template <class R>
 int norm_dev(qtt_ctx* c, const qtt_tt* x, double* out) {
@@ -1672,32 +1770,22 @@ static int sketch_core(qtt_ctx* c, int T, const qtt_complex* coef, const qtt_mpo
                        qtt_tt** yout, double* dot_out) {
   const int d = S->d;
   typedef cplx<R> C;
-  // identity operators for terms without one
-  std::vector<qtt_mpo*> own(T, nullptr);
+  // Terms without an operator: shapes of the identity, no cores.  Where a core
+  // is the identity with bonds of 1, its contractions would copy U1 to U2 and
+  // T1 into Y, two of the term's five per core: they are skipped.
+  std::vector<qtt_mpo> own(T);
   std::vector<const qtt_mpo*> A(T);
-  struct Cleanup {
-    std::vector<qtt_mpo*>& v;
-    ~Cleanup() {
-      for (auto* p : v) mpo_free(p);
-    }
-  } cleanup{own};
   for (int t = 0; t < T; ++t) {
     if (xs[t]->d != d) return QTT_ERR_ARG;
     if (ops && ops[t]) {
       if (ops[t]->d != d) return QTT_ERR_ARG;
       A[t] = ops[t];
     } else {
-      int st;
-      std::vector<int> g(d + 1, 1);
-      own[t] = mpo_alloc(c, d, xs[t]->n, xs[t]->n, g, S->dtype, &st);
-      if (!own[t]) return st;
-      for (int k = 0; k < d; ++k) {
-        c->launches++;
-        TRY(qtt_identity_core<R>(1, xs[t]->n[k],
-                                 reinterpret_cast<C*>(static_cast<char*>(own[t]->data) + own[t]->off[k]), c->stream));
-        own[t]->diag[k] = 1;
-      }
-      A[t] = own[t];
+      own[t].d = d;
+      own[t].no = own[t].ni = xs[t]->n;
+      own[t].g.assign(d + 1, 1);
+      own[t].ident.assign(d, 1);
+      A[t] = &own[t];
     }
     for (int k = 0; k < d; ++k) {
       if (A[t]->ni[k] != xs[t]->n[k] || A[t]->no[k] != S->n[k]) return QTT_ERR_ARG;
@@ -1754,9 +1842,10 @@ static int sketch_core(qtt_ctx* c, int T, const qtt_complex* coef, const qtt_mpo
       }
       TRY(dbg_finite<R>(c, U1.as<C>(), g1 * a1 * no * l0, "sketch U1", k));
       // U2[a1, g0, j, l0] = sum_{i, g1} D[g0, i, j, g1] U1[g1, a1, i, l0]   (batch a1)
-      TRY(U2.alloc(c, (size_t)a1 * g0 * ni * l0 * sizeof(C)));
-      const bool dg = A[t]->diag[k] && ni == no;
-      if (dg) {
+      if (!A[t]->ident[k]) TRY(U2.alloc(c, (size_t)a1 * g0 * ni * l0 * sizeof(C)));
+      if (A[t]->ident[k]) {
+        U2 = std::move(U1);  // g0 = g1 = 1, j = i: the same array
+      } else if (A[t]->diag[k] && ni == no) {
         // diagonal core (D[g0, i, j, g1] = 0 for i != j): batch (a1, i),
         // U2[a1, g0, i, l0] = sum_g1 D[g0, i, i, g1] U1[g1, a1, i, l0]
         GemmDesc g;
@@ -1830,8 +1919,16 @@ static int sketch_core(qtt_ctx* c, int T, const qtt_complex* coef, const qtt_mpo
     return QTT_OK;
   }
   // ---- left-to-right projection
-  std::vector<DBuf> outc(d);
+  // its ranks follow from the sketch's, so the projected train is written in place
   std::vector<int> orank(d + 1, 1);
+  for (int k = 0; k + 1 < d; ++k)
+    orank[k + 1] = (int)std::min<int64_t>((int64_t)orank[k] * S->n[k], S->r[k + 1]);
+  int st;
+  struct Held {
+    qtt_tt* p;
+    ~Held() { tt_free(p); }
+  } P{tt_alloc(c, d, S->n, orank, S->dtype, &st)};
+  if (!P.p) return st;
   DBuf M;  // l_k x Bt_k
   {
     TRY(M.alloc(c, (size_t)T * sizeof(C)));
@@ -1848,6 +1945,24 @@ static int sketch_core(qtt_ctx* c, int T, const qtt_complex* coef, const qtt_mpo
     for (int t = 0; t < T; ++t) {
       const int64_t g0 = A[t]->g[k], g1 = A[t]->g[k + 1], ni = A[t]->ni[k];
       const int64_t a0 = xs[t]->r[k], a1 = xs[t]->r[k + 1];
+      if (A[t]->ident[k]) {
+        // Y[l, j, off' + a1] = sum_a0 M[l, off + a0] X[a0, j, a1], straight into its place
+        GemmDesc g;
+        g.bA = g.bB = g.bC = B0();
+        g.M = lk;
+        g.N = ni * a1;
+        g.K = a0;
+        g.batch = 1;
+        g.mA = L1(lk, Bt(k));
+        g.kA = L1(a0, 1);
+        g.kB = L1(a0, ni * a1);
+        g.nB = L1(g.N, 1);
+        g.mC = L1(lk, no * Bn);
+        g.nC = L2(ni, Bn, a1, 1);
+        g.conjA = g.conjB = 0;
+        TRY(gemm<R>(c, g, M.as<C>() + boff[k][t], Xk(t, k), Y.as<C>() + boff[k + 1][t]));
+        continue;
+      }
       // T1[l, g0, j, a1] = sum_a0 M[l, off + g0 a0 + a0] X[a0, j, a1]
       DBuf T1;
       TRY(T1.alloc(c, (size_t)lk * g0 * ni * a1 * sizeof(C)));
@@ -1907,44 +2022,35 @@ static int sketch_core(qtt_ctx* c, int T, const qtt_complex* coef, const qtt_mpo
       }
     }
     const int64_t l1 = S->r[k + 1];
-    // Z = Y (lk no x Bn) W_{k+1} (Bn x l1)
-    DBuf Z;
-    TRY(Z.alloc(c, (size_t)lk * no * l1 * sizeof(C)));
-    TRY(dbg_finite<R>(c, Y.as<C>(), lk * no * Bn, "left Y", k));
-    TRY(mm<R>(c, lk * no, l1, Bn, Y.as<C>(), Bn, 1, 0, W[k + 1].as<C>(), l1, 1, 0, Z.as<C>(), l1, 1));
-    TRY(dbg_finite<R>(c, Z.as<C>(), lk * no * l1, "left Z", k));
-    if (k == d - 1) {
-      outc[k] = std::move(Z);
-      break;
+    // Z = Y (lk no x Bn) W_{k+1} (Bn x l1); on the last core Z is the core
+    DBuf Zb;
+    C* core = core_ptr<C>(P.p, k);
+    C* Z = core;
+    if (k < d - 1) {
+      TRY(Zb.alloc(c, (size_t)lk * no * l1 * sizeof(C)));
+      Z = Zb.as<C>();
     }
+    TRY(dbg_finite<R>(c, Y.as<C>(), lk * no * Bn, "left Y", k));
+    TRY(mm<R>(c, lk * no, l1, Bn, Y.as<C>(), Bn, 1, 0, W[k + 1].as<C>(), l1, 1, 0, Z, l1, 1));
+    TRY(dbg_finite<R>(c, Z, lk * no * l1, "left Z", k));
+    if (k == d - 1) break;
     // Q of Z (lk no x l1): new core (lk, no, q)
     const int64_t m = lk * no, q = std::min(m, l1);
     DBuf Wq, tau;
-    TRY(outc[k].alloc(c, (size_t)m * q * sizeof(C)));
     TRY(Wq.alloc(c, qr_work(m, l1, 1) * sizeof(C)));
     TRY(tau.alloc(c, (size_t)2 * l1 * sizeof(C)));
-    TRY(qr_launch<R>(c, Z.as<C>(), B0(), L1(m, l1), L1(l1, 1), 0, m, l1, m, m, 1, Wq.as<C>(), nullptr, 0, 0,
-                     tau.as<C>(), outc[k].as<C>(), 0, q));
-    TRY(dbg_finite<R>(c, outc[k].as<C>(), m * q, "left Q", k));
-    orank[k + 1] = (int)q;
+    TRY(qr_launch<R>(c, Z, B0(), L1(m, l1), L1(l1, 1), 0, m, l1, m, m, 1, Wq.as<C>(), nullptr, 0, 0, tau.as<C>(), core,
+                     0, q));
+    TRY(dbg_finite<R>(c, core, m * q, "left Q", k));
     // M_{k+1} = Q^H Y  (q x Bn)
     DBuf Mn;
     TRY(Mn.alloc(c, (size_t)q * Bn * sizeof(C)));
-    TRY(mm<R>(c, q, Bn, m, outc[k].as<C>(), 1, q, 1, Y.as<C>(), Bn, 1, 0, Mn.as<C>(), Bn, 1));
+    TRY(mm<R>(c, q, Bn, m, core, 1, q, 1, Y.as<C>(), Bn, 1, 0, Mn.as<C>(), Bn, 1));
     M = std::move(Mn);
     lk = q;
   }
-  // assemble the projected train, then round it deterministically
-  int st;
-  qtt_tt* P = tt_alloc(c, d, S->n, orank, S->dtype, &st);
-  if (!P) return st;
-  for (int k = 0; k < d; ++k) {
-    size_t bytes = (size_t)orank[k] * S->n[k] * orank[k + 1] * sizeof(C);
-    cudaMemcpyAsync(static_cast<char*>(P->data) + P->off[k], outc[k].p, bytes, cudaMemcpyDeviceToDevice, c->stream);
-  }
-  int rs = round_det<R>(c, P, eps, max_rank, nullptr, info, yout, true);
-  tt_free(P);
-  return rs;
+  // round the projected train deterministically
+  return round_det<R>(c, P.p, eps, max_rank, nullptr, info, yout, true);
 }
 
 template <class R>

@@ -3,6 +3,7 @@
 
 #include <stdint.h>
 
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <unordered_map>
@@ -10,6 +11,7 @@
 
 #include "../../include/qtt.h"
 #include "common.cuh"
+#include "kernels.h"
 
 // Kernel classes for the built-in profiler (qtt_ctx_profile*).
 enum { PK_GEMM = 0, PK_QR = 1, PK_JACOBI = 2, PK_ELEM = 3, PK_N = 4 };
@@ -133,6 +135,7 @@ struct qtt_mpo {
   std::vector<int> no, ni, g;     // output modes, input modes, bond ranks (d + 1)
   std::vector<char> diag;         // per core: zero unless in == out index (a diagonal
                                   // operator core; the contractions then skip the zeros)
+  std::vector<char> ident;        // per core: the identity with bonds of 1 (its contractions are copies)
   qtt_dtype dtype = QTT_C128;
   void* data = nullptr;
   std::vector<size_t> off;
@@ -204,6 +207,21 @@ int gemm_ab(qtt_ctx* c, const GemmDesc& g, cplx<R> alpha, cplx<R> beta, const cp
             cplx<R>* C);
 
 // z = a x + b y (ranks add) and a synchronous host -> device copy (engine.cu)
+// cores of a train handed to a table kernel QTT_TABLE at a time: fn(first, count)
+template <class F>
+inline int each_table(int d, F fn) {
+  for (int k0 = 0; k0 < d; k0 += QTT_TABLE) {
+    const int st = fn(k0, std::min(QTT_TABLE, d - k0));
+    if (st != QTT_OK) return st;
+  }
+  return QTT_OK;
+}
+// (means of x and of chi x) per control index: sums over all spatial sites of
+// x(I, .) and, chi not null, of conj(chi(.)) x(I, .); out: 2 values (re, im) per
+// control index.  x: control core first; chi: the spatial sites only, x's dtype.
+template <class R>
+int control_sums(qtt_ctx* c, const qtt_tt* x, const qtt_tt* chi, double* out);
+
 template <class R>
 int add_dev(qtt_ctx* c, cplx<R> a, const qtt_tt* x, cplx<R> b, const qtt_tt* y, qtt_tt** out);
 int upload(qtt_ctx* c, void* dst, const void* src, size_t bytes);

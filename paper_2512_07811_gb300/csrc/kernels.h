@@ -93,6 +93,45 @@ int qtt_scale_rows(cplx<R>* x, int64_t rows, int64_t cols, int64_t ld, const R* 
 template <class R>
 int qtt_isfinite(const cplx<R>* x, int64_t count, int* flag, cudaStream_t s);
 
+// ---- one launch over the cores of a train (elem.cu): up to QTT_TABLE cores each
+#define QTT_TABLE 48
+struct CoreTable {
+  int n;
+  const void* src[QTT_TABLE];
+  void* dst[QTT_TABLE];
+  int64_t cnt[QTT_TABLE];
+};
+// what: 0 copy (elem bytes each, 8 or 16), 1 complex128 -> complex64, 2 complex64 -> complex128
+int qtt_cores_move(const CoreTable& t, int what, int elem, cudaStream_t s);
+// *flag = 1 if an element of the src cores is not finite
+template <class R>
+int qtt_cores_isfinite(const CoreTable& t, int* flag, cudaStream_t s);
+// sketch cores: the M x M identity where M > 0, else real Gaussian N(0, scale^2) from (seed, stream + core)
+struct SketchTable {
+  int n;
+  void* dst[QTT_TABLE];
+  int64_t cnt[QTT_TABLE], M[QTT_TABLE];
+  double scale[QTT_TABLE];
+  uint64_t seed, stream;
+};
+template <class R>
+int qtt_fill_sketch(const SketchTable& t, cudaStream_t s);
+// cores of a x + b y: blocks [x | y] on the bonds, zero elsewhere; xa, xb, ya, yb the bond sizes, first / last: the
+// train's end cores (bond 0 not stacked; scale on the first)
+template <class R>
+struct AddTable {
+  int n;
+  const cplx<R>* x[QTT_TABLE];
+  const cplx<R>* y[QTT_TABLE];
+  cplx<R>* z[QTT_TABLE];
+  int xa[QTT_TABLE], xb[QTT_TABLE], ya[QTT_TABLE], yb[QTT_TABLE], nk[QTT_TABLE];
+  int first, last;  // index of the first / last core in this table, or -1
+  cplx<R> a, b;
+  int ua, ub;  // a / b is exactly 1: the block is copied
+};
+template <class R>
+int qtt_add_cores(const AddTable<R>& t, int64_t max_count, cudaStream_t s);
+
 // ---- operator construction on the device (elem.cu)
 template <class R>
 int qtt_fill_qft_dense(cplx<R>* out, int n, double sign, cudaStream_t s);
