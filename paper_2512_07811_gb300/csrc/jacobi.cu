@@ -58,69 +58,125 @@ struct JacThreads {
   static constexpr int value = sizeof(R) == 8 ? 256 : 512;  // FP64 columns take twice the registers
 };
 
-template <class R>
-__device__ __forceinline__ cplx<R> wsum_c(cplx<R> w, int lane) {
+// sum over the LP lanes that share a pair (all lanes of the warp take part)
+template <int LP, class R>
+__device__ __forceinline__ R gsum(R v) {
+#pragma unroll
+  for (int o = LP / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+// FP64: half of the lanes sum the real part, half the imaginary one, one addition a level
+template <int LP, class R>
+__device__ __forceinline__ cplx<R> gsum_c(cplx<R> w, int lane) {
   if constexpr (sizeof(R) == 4) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
+    for (int o = LP / 2; o > 0; o >>= 1) {
       w.re += __shfl_xor_sync(0xffffffffu, w.re, o);
       w.im += __shfl_xor_sync(0xffffffffu, w.im, o);
     }
     return w;
   } else {
-    const bool up = lane & 16;
-    R v = (up ? w.im : w.re) + __shfl_xor_sync(0xffffffffu, up ? w.re : w.im, 16);
+    const bool up = lane & (LP / 2);
+    R v = (up ? w.im : w.re) + __shfl_xor_sync(0xffffffffu, up ? w.re : w.im, LP / 2);
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return cplx<R>(__shfl_sync(0xffffffffu, v, 0), __shfl_sync(0xffffffffu, v, 16));
+    for (int o = LP / 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    const R o = __shfl_xor_sync(0xffffffffu, v, LP / 2);
+    return up ? cplx<R>(o, v) : cplx<R>(v, o);
   }
 }
 
-// reciprocal square root that only steers a rotation angle
-__device__ __forceinline__ float rsqrt_fast(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double rsqrt_fast(double x) {
+// FP64 helpers without FP64 instructions
+__device__ __forceinline__ double rsqrt_seed(double x) {  // about 20 bits
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  return fma(0.5 * y, fma(-x * y, y, 1.0), y);
+  return y;
+}
+__device__ __forceinline__ double times2(double x, int k) {  // x 2^k, x normal
+  return __hiloint2double(__double2hiint(x) + (k << 20), __double2loint(x));
+}
+__device__ __forceinline__ int ilogb_c(double x) { return (__double2hiint(x) >> 20) - 1023; }  // x > 0 normal
+constexpr int kHiMin = 0x05e00000;  // squares of inner products below 1e-280 count as zero
+
+// whether a squared norm has dropped to less than about a sixteenth of its old value
+__device__ __forceinline__ bool dropped(float v, float old) { return !(v > 0.0625f * old); }
+__device__ __forceinline__ bool dropped(double v, double old) {
+  return __double2hiint(v) < __double2hiint(old) - (4 << 20);  // by the exponents: no FP64 instruction
 }
 
-template <class R, int RPL>
+template <int LP, class R, int RPL>
 __device__ __forceinline__ R col_norm2(const cplx<R> (&x)[RPL]) {
   R s = 0, s1 = 0;
 #pragma unroll
   for (int u = 0; u < RPL; ++u) {
     if (u & 1) s1 += abs2(x[u]); else s += abs2(x[u]);
   }
-  return dense::wsum(s + s1);
+  return gsum<LP>(s + s1);
 }
 
-// Rotates columns x, y (rows on the lanes) to orthogonality; al, be their
-// squared norms.  With g = x^H y, d = (be - al) / 2, h = sqrt(d^2 + |g|^2) and
-// w = |d| + h, the smaller root has tan = |g| / w and w^2 + |g|^2 = 2 h w, so
-// with r = 1 / sqrt(w^2 + |g|^2): cos = w r, sin e^{i arg g} = g r (signed by
-// d), and the norms change by |g|^2 / w = 2 |g|^2 h r^2.  cos^2 + sin^2 = 1 to
-// the accuracy of r, whatever h is.  Returns 0 (orthogonal to tol, or |g|^2
-// below the normal range), 1 (rotated), 3 (rotated, not small: |cos of the
-// angle between x and y| or the sine weighted by the norms' ratio above
-// sqrt(big2)).
-template <class R, int RPL>
+// Rotates columns x, y (rows on the LP lanes of a group) to orthogonality; al,
+// be their squared norms.  With g = x^H y, d = (be - al) / 2, h = sqrt(d^2 +
+// |g|^2) and w = |d| + h, the smaller root has tan = |g| / w and w^2 + |g|^2 =
+// 2 h w, so with r = 1 / sqrt(w^2 + |g|^2): cos = w r, sin e^{i arg g} = g r
+// (signed by d), and the norms change by |g|^2 / w = 2 |g|^2 h r^2.  cos^2 +
+// sin^2 = 1 to the accuracy of r, whatever h is.  Returns 0 (`act` false,
+// orthogonal to tol, or |g|^2 below the normal range), 1 (rotated) or 3 (rotated, not
+// small: the sine weighted by the norms' ratio above sqrt(big2); that weighted
+// sine is at least about half the cosine of the angle between x and y).
+template <int LP, class R, int RPL>
 __device__ __forceinline__ int rotate_pair(cplx<R> (&x)[RPL], cplx<R> (&y)[RPL], R& al, R& be, R tol2, R big2,
-                                           int lane) {
+                                           int lane, bool act) {
   cplx<R> g(0, 0), g1(0, 0);
 #pragma unroll
   for (int u = 0; u < RPL; ++u) {
     if (u & 1) cfma_conj(g1, x[u], y[u]); else cfma_conj(g, x[u], y[u]);
   }
-  g = wsum_c(g + g1, lane);
-  const R ag2 = abs2(g), ab = al * be;
-  if (!(ag2 > tol2 * ab) || !(ag2 >= Lim<R>::tiny)) return 0;
-  const R d = R(0.5) * (be - al), h2 = fma(d, d, ag2);
-  const R h = h2 * rsqrt_fast(h2), w = fabs(d) + h;
-  const R r = dense::rsqrt_nr(fma(w, w, ag2));
-  const R cs = w * r, sr = d >= R(0) ? r : -r;
-  const cplx<R> f(sr * g.re, sr * g.im);
-  const R s2 = ag2 * (r * r), dl = (h + h) * s2;
-  const int code = ag2 > big2 * ab || s2 * fmax(al, be) > big2 * fmin(al, be) ? 3 : 1;
+  g = gsum_c<LP>(g + g1, lane);
+  const R ag2 = abs2(g);
+  R cs, dl;
+  cplx<R> f;
+  int code;
+  bool rot, up;
+  if constexpr (sizeof(R) == 4) {
+    rot = act && ag2 > tol2 * (al * be) && ag2 >= FLT_MIN;
+    if (LP == 32 ? !rot : !__any_sync(0xffffffffu, rot)) return 0;
+    const R d = R(0.5) * (be - al), h2 = fma(d, d, ag2);
+    const R h = h2 * rsqrtf(h2), w = fabs(d) + h;
+    const R r = dense::rsqrt_nr(fma(w, w, ag2));
+    up = d >= R(0);  // be >= al
+    cs = w * r;
+    const R sr = up ? r : -r;
+    f = cplx<R>(sr * g.re, sr * g.im);
+    const R s2 = ag2 * (r * r);
+    dl = (h + h) * s2;
+    code = s2 * (up ? be : al) > big2 * (up ? al : be) ? 3 : 1;
+  } else {
+    // a warp instruction holds its quarter's FP64 unit for 64 cycles: comparisons
+    // by exponents (integer), factors of 2 and 4 by adding to them, h from the
+    // hardware's 20-bit reciprocal square root.  The threshold then lies between
+    // tol / sqrt(2) and 2 tol.
+    const int hg = __double2hiint(ag2), ea = __double2hiint(al) >> 20, eb = __double2hiint(be) >> 20;
+    rot = act && (hg >> 20) + 1023 > ea + eb + ilogb_c(tol2) && hg >= kHiMin && hg < 0x7ff00000;
+    if (LP == 32 ? !rot : !__any_sync(0xffffffffu, rot)) return 0;
+    const R D = be - al, q4 = times2(ag2, 2), h2 = fma(D, D, q4);
+    const R H = h2 * rsqrt_seed(h2), W = fabs(D) + H;  // 2 h, 2 w
+    const R x4 = fma(W, W, q4), y0 = rsqrt_seed(x4), er = fma(-x4 * y0, y0, 1.0);
+    const R r2 = fma(y0 * er, fma(0.375, er, 0.5), y0);  // r / 2, one third-order step from 20 bits
+    const R r = times2(r2, 1);
+    up = __double2hiint(D) >= 0;
+    cs = W * r2;
+    const R sr = up ? r : -r;
+    f = cplx<R>(sr * g.re, sr * g.im);
+    const R s2 = ag2 * (r * r);
+    dl = H * s2;
+    const int es = (__double2hiint(s2) >> 20) + (up ? eb - ea : ea - eb);
+    code = es >= ilogb_c(big2) + 1022 ? 3 : 1;
+  }
+  if (LP < 32 && !rot) {  // another group of the warp rotates
+    cs = R(1);
+    f = cplx<R>(0, 0);
+    dl = R(0);
+    code = 0;
+  }
 #pragma unroll
   for (int u = 0; u < RPL; ++u) {
     const cplx<R> a = x[u], b = y[u];
@@ -130,11 +186,15 @@ __device__ __forceinline__ int rotate_pair(cplx<R> (&x)[RPL], cplx<R> (&y)[RPL],
     y[u].im = fma(cs, b.im, fma(f.re, a.im, f.im * a.re));
   }
   const R al0 = al, be0 = be;
-  const R sd = d >= R(0) ? dl : -dl;
-  al = al0 - sd;
-  be = be0 + sd;
-  if (!(al > R(0.05) * al0)) al = col_norm2<R, RPL>(x);
-  if (!(be > R(0.05) * be0)) be = col_norm2<R, RPL>(y);
+  if (!up) dl = -dl;
+  al = al0 - dl;
+  be = be0 + dl;
+  const bool da = dropped(al, al0), db = dropped(be, be0);
+  if (LP == 32 ? da || db : __any_sync(0xffffffffu, da || db)) {
+    const R na = col_norm2<LP, R, RPL>(x), nb = col_norm2<LP, R, RPL>(y);
+    if (da) al = na;
+    if (db) be = nb;
+  }
   return code;
 }
 
@@ -143,15 +203,19 @@ __device__ __forceinline__ int jac_exponent(double a) { return a > 0 && a <= DBL
 __device__ __forceinline__ float jac_pow2(float, int e) { return ldexpf(1.f, e); }
 __device__ __forceinline__ double jac_pow2(double, int e) { return ldexp(1.0, e); }
 
-template <class R, int RPL>
+template <class R, int LP, int RPL>
 __global__ void __launch_bounds__(JacThreads<R>::value, 1)
 jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
   typedef cplx<R> C;
   cg::cluster_group cluster = cg::this_cluster();
   const int NC = (int)cluster.num_blocks(), NB = 2 * NC, rank = (int)cluster.block_rank();
   const int p = a.p, q = a.q, bs = a.bs, qp = NB * bs;
-  constexpr int LD = 32 * RPL;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nthr = blockDim.x;  // bs warps
+  constexpr int LD = LP * RPL;
+  const int lane = threadIdx.x & 31, nthr = blockDim.x;
+  // a pair is worked on by a group of LP lanes: group w of ng, lane gl of it
+  const int gl = lane % LP, w = threadIdx.x / LP, ng = nthr / LP;
+  const bool act = w < bs;       // this group has a column of either block
+  const int wc = act ? w : 0;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* slots = reinterpret_cast<C*>(smem_raw);                 // [4][bs][LD]
   double* scan = reinterpret_cast<double*>(slots + (size_t)4 * bs * LD);  // 2 of the truncation rule
@@ -182,10 +246,10 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-    if (lane == 0) sorted[w] = amax;
+    if (lane == 0) sorted[threadIdx.x >> 5] = amax;  // (2 NC bs values hold one per warp)
     __syncthreads();
-    if (w == 0) {
-      R t = lane < bs ? sorted[lane] : R(0);
+    if (threadIdx.x < 32) {
+      R t = lane < (nthr >> 5) ? sorted[lane] : R(0);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) t = fmax(t, __shfl_xor_sync(0xffffffffu, t, o));
       if (lane < NC) cluster.map_shared_rank(flags, lane)[32 + rank] = jac_exponent(t);
@@ -213,11 +277,11 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
   C x[RPL], y[RPL];
   auto load = [&](C(&v)[RPL], const C* s) {
 #pragma unroll
-    for (int u = 0; u < RPL; ++u) v[u] = s[lane + 32 * u];
+    for (int u = 0; u < RPL; ++u) v[u] = s[gl + LP * u];
   };
   auto store = [&](const C(&v)[RPL], C* s) {
 #pragma unroll
-    for (int u = 0; u < RPL; ++u) s[lane + 32 * u] = v[u];
+    for (int u = 0; u < RPL; ++u) s[gl + LP * u] = v[u];
   };
   const int posn[2] = {rank, NB - 1 - rank};
   int dst_cta[2], dst_top[2];
@@ -231,11 +295,11 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
   for (; sweep < a.max_sweeps; ++sweep) {
     int wf = 0;
     // fresh norms of both blocks
-    load(x, col(top, w));
-    load(y, col(bot, w));
+    load(x, col(top, wc));
+    load(y, col(bot, wc));
     {
-      const R na = col_norm2<R, RPL>(x), nb = col_norm2<R, RPL>(y);
-      if (lane == 0) {
+      const R na = col_norm2<LP, R, RPL>(x), nb = col_norm2<LP, R, RPL>(y);
+      if (gl == 0 && act) {
         nrm[top * bs + w] = na;
         nrm[bot * bs + w] = nb;
       }
@@ -244,21 +308,25 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
     // pairs inside each block (round-robin of bs columns, one bye if bs is odd)
     const int be_ = bs + (bs & 1), half = be_ / 2;
     for (int s = 0; s + 1 < be_; ++s) {
-      for (int kk = w; kk < 2 * half; kk += bs) {
+      for (int k0 = 0; k0 < 2 * half; k0 += ng) {
+        const int kk = min(k0 + w, 2 * half - 1);
         const int slot = kk < half ? top : bot, k = kk < half ? kk : kk - half;
         const int j0 = k == 0 ? 0 : 1 + (k - 1 + s) % (be_ - 1);
         const int k1 = be_ - 1 - k;
         const int j1 = 1 + (k1 - 1 + s) % (be_ - 1);
-        if (j0 >= bs || j1 >= bs) continue;
-        load(x, col(slot, j0));
-        load(y, col(slot, j1));
-        R al = nrm[slot * bs + j0], be = nrm[slot * bs + j1];
-        const int f = rotate_pair<R, RPL>(x, y, al, be, tol2, big2, lane);
+        const bool on = k0 + w < 2 * half && j0 < bs && j1 < bs;
+        const int i0 = on ? j0 : 0, i1 = on ? j1 : 0;
+        if (on) {
+          load(x, col(slot, i0));
+          load(y, col(slot, i1));
+        }
+        R al = nrm[slot * bs + i0], be = nrm[slot * bs + i1];
+        const int f = rotate_pair<LP, R, RPL>(x, y, al, be, tol2, big2, lane, on);
         if (f) {
           wf |= f;
           store(x, col(slot, j0));
           store(y, col(slot, j1));
-          if (lane == 0) {
+          if (gl == 0) {
             nrm[slot * bs + j0] = al;
             nrm[slot * bs + j1] = be;
           }
@@ -267,21 +335,22 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
       __syncthreads();
     }
     for (int br = 0; br < NB - 1; ++br) {
-      load(x, col(top, w));
-      R al = nrm[top * bs + w];
-      int c = w;
+      load(x, col(top, wc));
+      R al = nrm[top * bs + wc];
+      int c = wc;
       for (int s = 0; s < bs; ++s) {
-        load(y, col(bot, c));
+        if (act) load(y, col(bot, c));  // (an idle group's values are not used)
         R be = nrm[bot * bs + c];
-        const int f = rotate_pair<R, RPL>(x, y, al, be, tol2, big2, lane);
+        const int f = rotate_pair<LP, R, RPL>(x, y, al, be, tol2, big2, lane, act);
         wf |= f;
         if (s + 1 < bs) {
           if (f) {
             store(y, col(bot, c));
-            if (lane == 0) nrm[bot * bs + c] = be;
+            if (gl == 0) nrm[bot * bs + c] = be;
           }
           __syncthreads();
           c = c + 1 == bs ? 0 : c + 1;
+        } else if (!act) {
         } else if (NC > 1) {
           // both blocks to their next CTA, straight from the registers
           const int st = dst_top[0] ? in_top : in_bot, sb = dst_top[1] ? in_top : in_bot;
@@ -289,21 +358,21 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
           store(x, rs + ((size_t)st * bs + w) * LD);
           C* rb = cluster.map_shared_rank(slots, dst_cta[1]);
           store(y, rb + ((size_t)sb * bs + c) * LD);
-          if (lane == 0) {
+          if (gl == 0) {
             cluster.map_shared_rank(nrm, dst_cta[0])[st * bs + w] = al;
             cluster.map_shared_rank(nrm, dst_cta[1])[sb * bs + c] = be;
           }
         } else {
           store(x, col(top, w));
           store(y, col(bot, c));
-          if (lane == 0) {
+          if (gl == 0) {
             nrm[top * bs + w] = al;
             nrm[bot * bs + c] = be;
           }
         }
       }
       if (br == NB - 2) {
-        if (lane == 0 && wf) atomicOr(&s_int[0], wf);
+        if (gl == 0 && wf) atomicOr(&s_int[0], wf);
         __syncthreads();
         if (threadIdx.x < NC) cluster.map_shared_rank(flags, threadIdx.x)[(sweep & 1) * 16 + rank] = s_int[0];
       }
@@ -330,15 +399,16 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
   }
   if (bt == 0 && rank == 0 && threadIdx.x == 0 && a.sweeps) *a.sweeps = sweep;
   // column norms (whole columns are local), gathered in every CTA
-  load(x, col(top, w));
-  load(y, col(bot, w));
-  const R nx = sqrt(col_norm2<R, RPL>(x)), ny = sqrt(col_norm2<R, RPL>(y));
-  const int cx = rank * bs + w, cy = (NB - 1 - rank) * bs + w;
-  if (lane < NC) {
-    R* rn = cluster.map_shared_rank(norms, lane);
-    rn[cx] = nx;
-    rn[cy] = ny;
-  }
+  load(x, col(top, wc));
+  load(y, col(bot, wc));
+  const R nx = sqrt(col_norm2<LP, R, RPL>(x)), ny = sqrt(col_norm2<LP, R, RPL>(y));
+  const int cx = rank * bs + wc, cy = (NB - 1 - rank) * bs + wc;
+  if (act)
+    for (int i = gl; i < NC; i += LP) {
+      R* rn = cluster.map_shared_rank(norms, i);
+      rn[cx] = nx;
+      rn[cy] = ny;
+    }
   cluster.sync();
   // order by decreasing norm (ties by index; a NaN first, so that it stays a permutation)
   auto key = [&](int i) {
@@ -348,18 +418,16 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
   auto place = [&](int c) {
     const R v = key(c);
     int rk = 0;
-    for (int i = lane; i < q; i += 32) {
+    for (int i = gl; i < q; i += LP) {
       const R u = key(i);
       rk += (u > v) || (u == v && i < c);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) rk += __shfl_xor_sync(0xffffffffu, rk, o);
-    return rk;
+    return gsum<LP>(rk);
   };
   const R sb = jac_pow2(R(0), esc);
-  for (int c = w; c < q; c += nthr >> 5) {
-    const int rk = place(c);
-    if (lane == 0) sorted[rk] = norms[c] * sb;
+  for (int c0 = 0; c0 < q; c0 += ng) {
+    const int c = min(c0 + w, q - 1), rk = place(c);
+    if (gl == 0 && c0 + w < q) sorted[rk] = norms[c] * sb;
   }
   __syncthreads();
   if (a.sigma && rank == 0)
@@ -368,7 +436,7 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
   if (a.trunc) {
     // smallest t >= 1 with sqrt(sum_{j >= t} s_j^2) <= delta, sums in double
     // by a suffix scan over the lanes, 32 values at a time from the end
-    if (w == 0) {
+    if (threadIdx.x < 32) {
       const double delta = a.deltas ? a.deltas[bt] : a.delta;
       double tail = 0.0;
       int t = q;
@@ -417,14 +485,14 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int c = h == 0 ? cx : cy;
-    if (c >= q) continue;
-    const int rk = place(c);
+    const int rk = place(min(c, q - 1));
+    if (c >= q || !act) continue;
     const R v = h == 0 ? nx : ny;
     R f = v > Lim<R>::tiny * R(4) ? R(1) / v : R(0);
     if (a.mask && rk >= keep) f = 0;
 #pragma unroll
     for (int u = 0; u < RPL; ++u) {
-      const int i = lane + 32 * u;
+      const int i = gl + LP * u;
       if (i >= p) continue;
       const C g = h == 0 ? x[u] : y[u];
       C o(g.re * f, -g.im * f);
@@ -435,49 +503,90 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
 }
 
 struct JacPlan {
-  int nc, bs, rpl;
+  int nc, bs, lp, rpl, warps;
   size_t smem;
 };
 
-int jac_slices(int p) {
-  const int nu = (p + 31) / 32;
-  return nu <= 6 ? nu : nu <= 8 ? 8 : nu <= 12 ? 12 : 16;
+// instances: rows held by a group of lp lanes, rpl each
+template <class R>
+bool jac_rows(int p, int lp, int* rpl) {
+  const int need = (p + lp - 1) / lp;
+  auto first = [&](std::initializer_list<int> l) {
+    for (int v : l)
+      if (v >= need) {
+        *rpl = v;
+        return true;
+      }
+    return false;
+  };
+  if (sizeof(R) == 4) {
+    if (lp == 32) return first({1, 2, 3, 4, 5, 6, 8, 12, 16});
+    if (lp == 16) return first({1, 2, 4});
+    return false;
+  }
+  if (lp == 32) return first({1, 2, 3, 4, 5, 6, 8, 12, 16});
+  if (lp == 16) return first({1, 2, 4});
+  return first({1, 2});
 }
 
+// Cluster size, lanes per pair and column width, by the cost of a sweep in
+// cycles: (2 nc - 1) block-rounds of bs rounds and one exchange, bs rounds inside
+// the blocks.  A round costs its latency, or where that is more what its warps
+// queue for: FP32 the issue slots; FP64 the FP64 unit of their quarter of the
+// SM, which a warp instruction holds for 64 cycles (16 rows' worth per slice and
+// about 27 for the scalars), so that four pairs an SM, one per quarter, are
+// the most that run side by side.  An exchange costs a cluster barrier and two
+// blocks through distributed shared memory at about 17 bytes a clock.
+// Constants from clock readings inside the kernel (FP32 620 cycles a round at
+// 118 rows, 720 at 256).  Per sweep with powers of two of at most 8 columns a
+// block, and with this choice (us): 118 x 118 FP32 59.7 / 54.2, 256 x 136 FP32
+// 103.6 / 88.1, 128 x 72 FP32 39.9 / 32.8.
 template <class R>
 bool jac_plan(int p, int q, int batch, JacPlan* pl) {
   if (p < 1 || q < 1 || p > 512 || q > 512 || batch < 1 || batch > 65535) return false;
-  const int rpl = jac_slices(p), wmax = JacThreads<R>::value / 32;
   int ncmax = 16;
   while (ncmax > 1 && ncmax * batch > 160) ncmax /= 2;
-  int nc = 1;
-  if (sizeof(R) == 4) {
-    nc = q <= 16 ? 1 : q <= 32 ? 2 : q <= 64 ? 4 : q <= 128 ? 8 : 16;
-  } else {
-    nc = q <= 4 ? 1 : q <= 8 ? 2 : q <= 16 ? 4 : q <= 32 ? 8 : 16;
-  }
-  nc = std::min(nc, ncmax);
-  for (; nc <= 16; nc *= 2) {
-    const int bs = (q + 2 * nc - 1) / (2 * nc);
-    const size_t sm = (size_t)4 * bs * 32 * rpl * sizeof(cplx<R>) + 16 + (4 * bs + (size_t)4 * nc * bs) * sizeof(R) +
-                      (48 + 4) * sizeof(int) + 16;
-    if (bs <= wmax && sm <= 200 * 1024) {
-      *pl = JacPlan{nc, bs, rpl, sm};
-      return true;
+  const int wmax = JacThreads<R>::value / 32;
+  double best = 1e300;
+  for (int pass = 0; pass < 2 && best > 1e299; ++pass)  // second pass: whatever fits shared memory
+    for (int lp : {32, 16, 8}) {
+      int rpl;
+      if (!jac_rows<R>(p, lp, &rpl)) continue;
+      for (int nc = 1; nc <= (pass ? 16 : ncmax); ++nc) {
+        const int bs = (q + 2 * nc - 1) / (2 * nc), warps = (bs * lp + 31) / 32;
+        if (nc > 1 && (2 * nc - 2) * bs >= q) continue;  // a CTA less would hold them
+        const size_t sm = (size_t)4 * bs * lp * rpl * sizeof(cplx<R>) + 16 +
+                          (4 * bs + (size_t)std::max(4 * nc * bs, 64)) * sizeof(R) + (48 + 4) * sizeof(int) + 16;
+        if (warps > wmax || sm > 200 * 1024) continue;
+        const int lg = lp == 32 ? 5 : lp == 16 ? 4 : 3;
+        double c, e = nc > 1 ? 600.0 : 60.0;
+        if (sizeof(R) == 4) {
+          c = lp == 32 ? std::max(540.0 + 22.0 * rpl, (warps + 3) / 4 * (150.0 + 28.0 * rpl))
+                       : std::max(600.0 + 40.0 * rpl, (warps + 3) / 4 * (180.0 + 40.0 * rpl));
+          if (nc > 1) e += 100.0 + 30.0 * bs * lp * rpl / 32;
+        } else {
+          c = (warps + 3) / 4 * 64.0 * (16.0 * rpl + 22.0 + lg) + 300.0;
+          if (nc > 1) e += 60.0 * bs * lp * rpl / 32;
+        }
+        const double cost = (2 * nc - 1) * (bs * c + e) + (bs + (bs & 1)) * c;
+        if (cost < best) {
+          best = cost;
+          *pl = JacPlan{nc, bs, lp, rpl, warps, sm};
+        }
+      }
     }
-  }
-  return false;
+  return best < 1e299;
 }
 
-template <class R, int RPL>
+template <class R, int LP, int RPL>
 int launch(const JacArgs<R>& a, const JacPlan& pl, int batch, cudaStream_t s) {
-  const void* fn = (const void*)jacobi_cluster2_kernel<R, RPL>;
+  const void* fn = (const void*)jacobi_cluster2_kernel<R, LP, RPL>;
   if (qtt_allow_max_smem(fn) != QTT_OK) return QTT_ERR_CUDA;
   if (pl.nc > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
     return QTT_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)pl.nc, (unsigned)batch, 1);
-  cfg.blockDim = dim3(32 * pl.bs, 1, 1);
+  cfg.blockDim = dim3(32 * pl.warps, 1, 1);
   cfg.dynamicSmemBytes = pl.smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -487,7 +596,7 @@ int launch(const JacArgs<R>& a, const JacPlan& pl, int batch, cudaStream_t s) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, jacobi_cluster2_kernel<R, RPL>, a) == cudaSuccess ? QTT_OK : QTT_ERR_CUDA;
+  return cudaLaunchKernelEx(&cfg, jacobi_cluster2_kernel<R, LP, RPL>, a) == cudaSuccess ? QTT_OK : QTT_ERR_CUDA;
 }
 
 }  // namespace
@@ -504,17 +613,17 @@ int qtt_svd(const cplx<R>* G, const int* perm, cplx<R>* Vh, R* sigma, int* trunc
   JacPlan pl;
   if (!jac_plan<R>(p, q, batch, &pl)) return QTT_ERR_UNSUPPORTED;
   const JacArgs<R> a{G, perm, Vh, sigma, trunc, delta, deltas, max_rank, mask, p, q, pl.bs, max_sweeps, sweeps};
-  switch (pl.rpl) {
-    case 1: return launch<R, 1>(a, pl, batch, s);
-    case 2: return launch<R, 2>(a, pl, batch, s);
-    case 3: return launch<R, 3>(a, pl, batch, s);
-    case 4: return launch<R, 4>(a, pl, batch, s);
-    case 5: return launch<R, 5>(a, pl, batch, s);
-    case 6: return launch<R, 6>(a, pl, batch, s);
-    case 8: return launch<R, 8>(a, pl, batch, s);
-    case 12: return launch<R, 12>(a, pl, batch, s);
-    default: return launch<R, 16>(a, pl, batch, s);
+#define QTT_J(LP, RPL) \
+  if (pl.lp == LP && pl.rpl == RPL) return launch<R, LP, RPL>(a, pl, batch, s)
+  if constexpr (sizeof(R) == 4) {
+    QTT_J(32, 1); QTT_J(32, 2); QTT_J(32, 3); QTT_J(32, 4); QTT_J(32, 5); QTT_J(32, 6); QTT_J(32, 8); QTT_J(32, 12);
+    QTT_J(32, 16); QTT_J(16, 1); QTT_J(16, 2); QTT_J(16, 4);
+  } else {
+    QTT_J(32, 1); QTT_J(32, 2); QTT_J(32, 3); QTT_J(32, 4); QTT_J(32, 5); QTT_J(32, 6); QTT_J(32, 8); QTT_J(32, 12);
+    QTT_J(32, 16); QTT_J(16, 1); QTT_J(16, 2); QTT_J(16, 4); QTT_J(8, 1); QTT_J(8, 2);
   }
+#undef QTT_J
+  return QTT_ERR_UNSUPPORTED;
 }
 template bool qtt_svd_fits<float>(int, int, int);
 template bool qtt_svd_fits<double>(int, int, int);
