@@ -520,13 +520,10 @@ bool jac_rows(int p, int lp, int* rpl) {
     return false;
   };
   if (sizeof(R) == 4) {
-    if (lp == 32) return first({1, 2, 3, 4, 5, 6, 8, 12, 16});
-    if (lp == 16) return first({1, 2, 4});
-    return false;
+    return lp == 32 && first({1, 2, 3, 4, 5, 6, 8, 12, 16});
   }
   if (lp == 32) return first({1, 2, 3, 4, 5, 6, 8, 12, 16});
-  if (lp == 16) return first({1, 2, 4});
-  return first({1, 2});
+  return first({1, 2, 4});
 }
 
 // Cluster size, lanes per pair and column width, by the cost of a sweep in
@@ -538,9 +535,11 @@ bool jac_rows(int p, int lp, int* rpl) {
 // the most that run side by side.  An exchange costs a cluster barrier and two
 // blocks through distributed shared memory at about 17 bytes a clock.
 // Constants from clock readings inside the kernel (FP32 620 cycles a round at
-// 118 rows, 720 at 256).  Per sweep with powers of two of at most 8 columns a
-// block, and with this choice (us): 118 x 118 FP32 59.7 / 54.2, 256 x 136 FP32
-// 103.6 / 88.1, 128 x 72 FP32 39.9 / 32.8.
+// 118 rows, 720 at 256).  (FP32 gains nothing from two pairs a warp: 690 cycles
+// a round at 16 rows against 650.)  us per sweep with powers of two of at most 8
+// columns a block, and with this choice: 118 x 118 FP32 59.7 / 54.2, 256 x 136
+// FP32 103.6 / 88.1, 128 x 72 FP32 39.9 / 32.8; FP64, with the FP64 instructions
+// of the scalars cut from about 45 to 27, 68 x 68 376 / 224, 124 x 124 597 / 467.
 template <class R>
 bool jac_plan(int p, int q, int batch, JacPlan* pl) {
   if (p < 1 || q < 1 || p > 512 || q > 512 || batch < 1 || batch > 65535) return false;
@@ -549,7 +548,7 @@ bool jac_plan(int p, int q, int batch, JacPlan* pl) {
   const int wmax = JacThreads<R>::value / 32;
   double best = 1e300;
   for (int pass = 0; pass < 2 && best > 1e299; ++pass)  // second pass: whatever fits shared memory
-    for (int lp : {32, 16, 8}) {
+    for (int lp : {32, 16}) {
       int rpl;
       if (!jac_rows<R>(p, lp, &rpl)) continue;
       for (int nc = 1; nc <= (pass ? 16 : ncmax); ++nc) {
@@ -558,14 +557,12 @@ bool jac_plan(int p, int q, int batch, JacPlan* pl) {
         const size_t sm = (size_t)4 * bs * lp * rpl * sizeof(cplx<R>) + 16 +
                           (4 * bs + (size_t)std::max(4 * nc * bs, 64)) * sizeof(R) + (48 + 4) * sizeof(int) + 16;
         if (warps > wmax || sm > 200 * 1024) continue;
-        const int lg = lp == 32 ? 5 : lp == 16 ? 4 : 3;
         double c, e = nc > 1 ? 600.0 : 60.0;
         if (sizeof(R) == 4) {
-          c = lp == 32 ? std::max(540.0 + 22.0 * rpl, (warps + 3) / 4 * (150.0 + 28.0 * rpl))
-                       : std::max(600.0 + 40.0 * rpl, (warps + 3) / 4 * (180.0 + 40.0 * rpl));
+          c = std::max(540.0 + 22.0 * rpl, (warps + 3) / 4 * (150.0 + 28.0 * rpl));
           if (nc > 1) e += 100.0 + 30.0 * bs * lp * rpl / 32;
         } else {
-          c = (warps + 3) / 4 * 64.0 * (16.0 * rpl + 22.0 + lg) + 300.0;
+          c = (warps + 3) / 4 * 64.0 * (16.0 * rpl + 27.0) + 300.0;
           if (nc > 1) e += 60.0 * bs * lp * rpl / 32;
         }
         const double cost = (2 * nc - 1) * (bs * c + e) + (bs + (bs & 1)) * c;
@@ -617,10 +614,10 @@ int qtt_svd(const cplx<R>* G, const int* perm, cplx<R>* Vh, R* sigma, int* trunc
   if (pl.lp == LP && pl.rpl == RPL) return launch<R, LP, RPL>(a, pl, batch, s)
   if constexpr (sizeof(R) == 4) {
     QTT_J(32, 1); QTT_J(32, 2); QTT_J(32, 3); QTT_J(32, 4); QTT_J(32, 5); QTT_J(32, 6); QTT_J(32, 8); QTT_J(32, 12);
-    QTT_J(32, 16); QTT_J(16, 1); QTT_J(16, 2); QTT_J(16, 4);
+    QTT_J(32, 16);
   } else {
     QTT_J(32, 1); QTT_J(32, 2); QTT_J(32, 3); QTT_J(32, 4); QTT_J(32, 5); QTT_J(32, 6); QTT_J(32, 8); QTT_J(32, 12);
-    QTT_J(32, 16); QTT_J(16, 1); QTT_J(16, 2); QTT_J(16, 4); QTT_J(8, 1); QTT_J(8, 2);
+    QTT_J(32, 16); QTT_J(16, 1); QTT_J(16, 2); QTT_J(16, 4);
   }
 #undef QTT_J
   return QTT_ERR_UNSUPPORTED;
