@@ -591,6 +591,28 @@ int tsqr_r(qtt_ctx* c, const cplx<R>* in, MIdx rowI, MIdx colI, int conj_in, int
   return tsqr_r<R>(c, Rs.as<cplx<R>>(), L1(nch * n, n), L1(n, 1), 0, nch * n, n, Rout, rows_out, one_cta);
 }
 
+template <class R>
+static GemmDesc bgemm(int64_t B, int64_t M, int64_t N, int64_t K, int64_t bA, MIdx mA, MIdx kA, int64_t bB, MIdx kB,
+                      MIdx nB, int64_t bC, MIdx mC, MIdx nC, int conjA = 0, int conjB = 0) {
+  GemmDesc g;
+  g.M = M;
+  g.N = N;
+  g.K = K;
+  g.batch = B;
+  g.bA = L1(B, bA);
+  g.mA = mA;
+  g.kA = kA;
+  g.bB = L1(B, bB);
+  g.kB = kB;
+  g.nB = nB;
+  g.bC = L1(B, bC);
+  g.mC = mC;
+  g.nC = nC;
+  g.conjA = conjA;
+  g.conjB = conjB;
+  return g;
+}
+
 // ---------------------------------------------- SVD by sorted QR + Jacobi
 // Right singular vectors of `batch` m x n matrices C (element (i, j) of matrix
 // b at in[inB(b) + rowI(i) + colI(j)], conjugated if conj_in): C P = Q R with
@@ -639,10 +661,37 @@ static int svd_right(qtt_ctx* c, const cplx<R>* in, MIdx inB, MIdx rowI, MIdx co
                         perm.as<int>(), nullptr, 0, 0, c->stream));
   prof_end(c, ev, PK_QR, batch * qr_flops((double)m, (double)n, false), (double)batch * m * n * sizeof(cplx<R>) * 2.0);
   prof_shape(c, ev, m, n, 0, batch, 0);
+  DBuf V, V1, GV;
+  const cplx<R>* Gj = G.as<cplx<R>>();
+  if constexpr (sizeof(R) == 8) {
+    if (qtt_svd_pre_fits((int)n, (int)q, (int)batch)) {
+      const int64_t qq = q * q;
+      TRY(V.alloc(c, (size_t)batch * 3 * qq * sizeof(zc)));
+      TRY(V1.alloc(c, (size_t)batch * qq * sizeof(zc)));
+      TRY(GV.alloc(c, (size_t)batch * n * q * sizeof(zc)));
+      zc *v = V.as<zc>(), *e[2] = {v + batch * qq, v + 2 * batch * qq}, *v1 = V1.as<zc>();
+      c->launches++;
+      TRY(qtt_svd_pre(G.as<zc>(), v, (int)n, (int)q, (int)batch, nullptr, c->stream));
+      for (int it = 0; it < 2; ++it) {
+        // E = 3/2 - V^H V / 2, V <- V E (V stored transposed)
+        TRY(simt_gemm<double>(c, bgemm<double>(batch, q, q, q, qq, L1(q, q), L1(q, 1), qq, L1(q, 1), L1(q, q), qq,
+                                               L1(q, q), L1(q, 1), 1),
+                              zc(-0.5, 0), zc(1.5, 0), v, v, e[it]));
+        TRY(simt_gemm<double>(c, bgemm<double>(batch, q, q, q, qq, L1(q, 1), L1(q, q), qq, L1(q, q), L1(q, 1), qq,
+                                               L1(q, 1), L1(q, q)),
+                              zc(1, 0), zc(0, 0), v, e[it], v1));
+        std::swap(v, v1);
+      }
+      TRY(simt_gemm<double>(c, bgemm<double>(batch, n, q, q, n * q, L1(n, q), L1(q, 1), qq, L1(q, 1), L1(q, q), n * q,
+                                             L1(n, q), L1(q, 1)),
+                            zc(1, 0), zc(0, 0), G.as<zc>(), v, GV.as<zc>()));
+      Gj = GV.as<zc>();
+    }
+  }
   int idx;
   int* slot = prof_sweep_slot(c, &idx);
   ev = prof_begin(c);
-  TRY(qtt_svd<R>(G.as<cplx<R>>(), perm.as<int>(), Vh, sigma, trunc, delta, deltas, max_rank, mask, (int)n, (int)q,
+  TRY(qtt_svd<R>(Gj, perm.as<int>(), Vh, sigma, trunc, delta, deltas, max_rank, mask, (int)n, (int)q,
                  (int)batch, 60, slot, c->stream));
   prof_end(c, ev, PK_JACOBI, 0.0, (double)batch * n * q * sizeof(cplx<R>) * 2.0, idx,
            batch * jacobi_sweep_flops((double)n, (double)q));
@@ -1174,28 +1223,6 @@ template int round_det<float>(qtt_ctx*, const qtt_tt*, double, int, const int*, 
 // rows and columns stay exactly zero, and the outputs are cropped to each
 // train's ranks.  QTT_ERR_UNSUPPORTED for shapes it does not take (the
 // caller then rounds the trains one by one).
-template <class R>
-static GemmDesc bgemm(int64_t B, int64_t M, int64_t N, int64_t K, int64_t bA, MIdx mA, MIdx kA, int64_t bB, MIdx kB,
-                      MIdx nB, int64_t bC, MIdx mC, MIdx nC, int conjA = 0, int conjB = 0) {
-  GemmDesc g;
-  g.M = M;
-  g.N = N;
-  g.K = K;
-  g.batch = B;
-  g.bA = L1(B, bA);
-  g.mA = mA;
-  g.kA = kA;
-  g.bB = L1(B, bB);
-  g.kB = kB;
-  g.nB = nB;
-  g.bC = L1(B, bC);
-  g.mC = mC;
-  g.nC = nC;
-  g.conjA = conjA;
-  g.conjB = conjB;
-  return g;
-}
-
 template <class R>
 int round_det_batch(qtt_ctx* c, int B, const qtt_tt* const* xs, double eps, int max_rank, qtt_round_info* infos,
                     qtt_tt** ys) {

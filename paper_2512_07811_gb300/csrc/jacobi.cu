@@ -25,6 +25,17 @@
 //     would only confirm it (see `big2`).
 // The caller sorts and QR-factors the matrix first (jacobi on R^H), which cuts
 // the sweeps from 14-21 to 6-7 on the roundings' matrices.
+//
+// FP64 matrices get all but the last two or three sweeps in FP32 (PRE): a sweep
+// costs a fifth there (68 x 68: 45 us against 224 us).  The FP32 kernel rotates
+// an identity along and returns V; two Newton-Schulz steps make V unitary to
+// FP64 rounding, G V is formed in FP64, and the FP64 kernel goes on from there
+// to its own tolerance, so the result is as before: V only chooses a basis.
+// The columns of G V keep the accuracy of the small ones, since V is graded as
+// G is.  Clusters of values equal to FP32 still take the full number.  us of a
+// rounding with one such SVD (values over 12 decades) without / with it: 68 x 68
+// 2640 / 1627, 80 x 48 1682 / 1100, 256 x 128 9054 / 5167; errors against 64-bit
+// references unchanged.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -51,6 +62,10 @@ struct JacArgs {
   int mask;               // rows of Vh from the kept rank on are zeroed
   int p, q, bs, max_sweeps;
   int* sweeps;
+  // rotations only (PRE): the matrix in FP64, the accumulated rotations transposed (row j: the column of the j-th
+  // largest norm, q x q), followed by two identity matrices of that size
+  const zc* Gd;
+  zc* Vt;
 };
 
 template <class R>
@@ -103,8 +118,9 @@ __device__ __forceinline__ bool dropped(double v, double old) {
   return __double2hiint(v) < __double2hiint(old) - (4 << 20);  // by the exponents: no FP64 instruction
 }
 
-template <int LP, class R, int RPL>
-__device__ __forceinline__ R col_norm2(const cplx<R> (&x)[RPL]) {
+// (a column's first RPL slices are the matrix's, the other RT - RPL follow its rotations)
+template <int LP, int RPL, class R, int RT>
+__device__ __forceinline__ R col_norm2(const cplx<R> (&x)[RT]) {
   R s = 0, s1 = 0;
 #pragma unroll
   for (int u = 0; u < RPL; ++u) {
@@ -122,8 +138,11 @@ __device__ __forceinline__ R col_norm2(const cplx<R> (&x)[RPL]) {
 // orthogonal to tol, or |g|^2 below the normal range), 1 (rotated) or 3 (rotated, not
 // small: the sine weighted by the norms' ratio above sqrt(big2); that weighted
 // sine is at least about half the cosine of the angle between x and y).
-template <int LP, class R, int RPL>
-__device__ __forceinline__ int rotate_pair(cplx<R> (&x)[RPL], cplx<R> (&y)[RPL], R& al, R& be, R tol2, R big2,
+// FP32 rotations alone (RT > RPL): a pair's norms are brought to 2^40, so that the
+// noise columns of a rank-deficient matrix (1e-16 of the largest) are rotated
+// too: they take as many FP64 sweeps as the others.
+template <int LP, int RPL, class R, int RT>
+__device__ __forceinline__ int rotate_pair(cplx<R> (&x)[RT], cplx<R> (&y)[RT], R& al, R& be, R tol2, R big2,
                                            int lane, bool act) {
   cplx<R> g(0, 0), g1(0, 0);
 #pragma unroll
@@ -131,6 +150,16 @@ __device__ __forceinline__ int rotate_pair(cplx<R> (&x)[RPL], cplx<R> (&y)[RPL],
     if (u & 1) cfma_conj(g1, x[u], y[u]); else cfma_conj(g, x[u], y[u]);
   }
   g = gsum_c<LP>(g + g1, lane);
+  const R al0 = al, be0 = be;
+  R unscale = 1;
+  if constexpr (RT > RPL) {
+    const int e = max(__float_as_int(fmax(al, be)) >> 23, 60);
+    const R k = __int_as_float((294 - e) << 23);
+    g = k * g;
+    al *= k;
+    be *= k;
+    unscale = __int_as_float((e - 40) << 23);
+  }
   const R ag2 = abs2(g);
   R cs, dl;
   cplx<R> f;
@@ -138,7 +167,11 @@ __device__ __forceinline__ int rotate_pair(cplx<R> (&x)[RPL], cplx<R> (&y)[RPL],
   bool rot, up;
   if constexpr (sizeof(R) == 4) {
     rot = act && ag2 > tol2 * (al * be) && ag2 >= FLT_MIN;
-    if (LP == 32 ? !rot : !__any_sync(0xffffffffu, rot)) return 0;
+    if (LP == 32 ? !rot : !__any_sync(0xffffffffu, rot)) {
+      al = al0;
+      be = be0;
+      return 0;
+    }
     const R d = R(0.5) * (be - al), h2 = fma(d, d, ag2);
     const R h = h2 * rsqrtf(h2), w = fabs(d) + h;
     const R r = dense::rsqrt_nr(fma(w, w, ag2));
@@ -178,20 +211,20 @@ __device__ __forceinline__ int rotate_pair(cplx<R> (&x)[RPL], cplx<R> (&y)[RPL],
     code = 0;
   }
 #pragma unroll
-  for (int u = 0; u < RPL; ++u) {
+  for (int u = 0; u < RT; ++u) {
     const cplx<R> a = x[u], b = y[u];
     x[u].re = fma(cs, a.re, fma(-f.re, b.re, -f.im * b.im));
     x[u].im = fma(cs, a.im, fma(-f.re, b.im, f.im * b.re));
     y[u].re = fma(cs, b.re, fma(f.re, a.re, -f.im * a.im));
     y[u].im = fma(cs, b.im, fma(f.re, a.im, f.im * a.re));
   }
-  const R al0 = al, be0 = be;
+  if constexpr (RT > RPL) dl *= unscale;
   if (!up) dl = -dl;
   al = al0 - dl;
   be = be0 + dl;
   const bool da = dropped(al, al0), db = dropped(be, be0);
   if (LP == 32 ? da || db : __any_sync(0xffffffffu, da || db)) {
-    const R na = col_norm2<LP, R, RPL>(x), nb = col_norm2<LP, R, RPL>(y);
+    const R na = col_norm2<LP, RPL>(x), nb = col_norm2<LP, RPL>(y);
     if (da) al = na;
     if (db) be = nb;
   }
@@ -203,14 +236,14 @@ __device__ __forceinline__ int jac_exponent(double a) { return a > 0 && a <= DBL
 __device__ __forceinline__ float jac_pow2(float, int e) { return ldexpf(1.f, e); }
 __device__ __forceinline__ double jac_pow2(double, int e) { return ldexp(1.0, e); }
 
-template <class R, int LP, int RPL>
+template <class R, int LP, int RPL, bool PRE>
 __global__ void __launch_bounds__(JacThreads<R>::value, 1)
 jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
   typedef cplx<R> C;
   cg::cluster_group cluster = cg::this_cluster();
   const int NC = (int)cluster.num_blocks(), NB = 2 * NC, rank = (int)cluster.block_rank();
   const int p = a.p, q = a.q, bs = a.bs, qp = NB * bs;
-  constexpr int LD = LP * RPL;
+  constexpr int RT = PRE ? 2 * RPL : RPL, LD = LP * RT;
   const int lane = threadIdx.x & 31, nthr = blockDim.x;
   // a pair is worked on by a group of LP lanes: group w of ng, lane gl of it
   const int gl = lane % LP, w = threadIdx.x / LP, ng = nthr / LP;
@@ -225,7 +258,6 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
   int* flags = reinterpret_cast<int*>(sorted + qp);          // [2][NC] sweep flags, then [NC] exponents
   int* s_int = flags + 3 * 16;                               // [0] sweep flags of this CTA, [1] kept rank
   const int64_t bt = blockIdx.y;
-  const C* G = a.G + bt * (int64_t)p * q;
   auto col = [&](int slot, int j) { return slots + ((size_t)slot * bs + j) * LD; };
   int top = 0, bot = 1, in_top = 2, in_bot = 3;
   if (threadIdx.x == 0) s_int[0] = 0;
@@ -234,13 +266,49 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
   // brings the largest component near 1 (FP32: near 2^14, so that squares of
   // squared norms of columns down to 1e-14 of the largest stay normal)
   int esc;
-  {
+  if constexpr (PRE) {
+    const zc* G = a.Gd + bt * (int64_t)p * q;
+    double amax = 0;
+    for (int e = threadIdx.x; e < 2 * bs * p; e += nthr) {
+      const int i = e / (2 * bs), jj = e - i * 2 * bs, half = jj / bs, j = jj - half * bs;
+      const int c = (half == 0 ? rank : NB - 1 - rank) * bs + j;
+      if (c >= q) continue;
+      const zc v = G[(int64_t)i * q + c];
+      amax = fmax(amax, fmax(fabs(v.re), fabs(v.im)));
+    }
+    const int ex = __reduce_max_sync(0xffffffffu, jac_exponent(amax));
+    int* wex = reinterpret_cast<int*>(sorted);  // (2 NC bs values hold one per warp)
+    if (lane == 0) wex[threadIdx.x >> 5] = ex;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      const int t = __reduce_max_sync(0xffffffffu, lane < (nthr >> 5) ? wex[lane] : -1000);
+      if (lane < NC) cluster.map_shared_rank(flags, lane)[32 + rank] = t;
+    }
+    cluster.sync();
+    esc = flags[32];
+    for (int i = 1; i < NC; ++i) esc = max(esc, flags[32 + i]);
+    esc -= 14;
+    const double sg = jac_pow2(0.0, -esc);
+    for (int e = threadIdx.x; e < 2 * bs * LD; e += nthr) {
+      const int i = e / (2 * bs), jj = e - i * 2 * bs, half = jj / bs, j = jj - half * bs;
+      const int c = (half == 0 ? rank : NB - 1 - rank) * bs + j;
+      C v(0, 0);
+      if (c < q && i < p) {
+        const zc g = G[(int64_t)i * q + c];
+        v = C((R)(sg * g.re), (R)(sg * g.im));
+      } else if (c < q && i == LP * RPL + c) {
+        v = C(1, 0);
+      }
+      col(half == 0 ? top : bot, j)[i] = v;
+    }
+    __syncthreads();
+  } else {
     R amax = 0;
     for (int e = threadIdx.x; e < 2 * bs * LD; e += nthr) {
       const int i = e / (2 * bs), jj = e - i * 2 * bs, half = jj / bs, j = jj - half * bs;
       const int c = (half == 0 ? rank : NB - 1 - rank) * bs + j;
       C v(0, 0);
-      if (c < q && i < p) v = G[(int64_t)i * q + c];
+      if (c < q && i < p) v = a.G[bt * (int64_t)p * q + (int64_t)i * q + c];
       col(half == 0 ? top : bot, j)[i] = v;
       amax = fmax(amax, fmax(fabs(v.re), fabs(v.im)));
     }
@@ -267,21 +335,23 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
   // non-orthogonality, which the truncated train inherits once per bond (a
   // tolerance of eps sqrt(p) made it the largest error of a rounding, 1e-5 at
   // 128 columns).
-  const R tol = R(0.5) * Lim<R>::eps, tol2 = tol * tol;
+  // (Rotations alone stop where the FP64 sweeps after them take two: what they
+  // leave, about 1e-6, is squared by the first of them.)
+  const R tol = PRE ? R(4) * Lim<R>::eps : R(0.5) * Lim<R>::eps, tol2 = tol * tol;
   // Quadratic regime: a rotation by sin s_ij of a pair (i, j) puts back s_ij g_jk
   // into an annihilated g_ik.  With c the largest cosine and s the largest
   // sine weighted by the norms' ratio of a sweep, the cosines after it are at
   // most about sqrt(q) s c; with both at most sqrt(tol / sqrt(q)) they are at
   // most tol, and the next sweep would rotate nothing.
   const R big2 = tol / sqrt(R(q));
-  C x[RPL], y[RPL];
-  auto load = [&](C(&v)[RPL], const C* s) {
+  C x[RT], y[RT];
+  auto load = [&](C(&v)[RT], const C* s) {
 #pragma unroll
-    for (int u = 0; u < RPL; ++u) v[u] = s[gl + LP * u];
+    for (int u = 0; u < RT; ++u) v[u] = s[gl + LP * u];
   };
-  auto store = [&](const C(&v)[RPL], C* s) {
+  auto store = [&](const C(&v)[RT], C* s) {
 #pragma unroll
-    for (int u = 0; u < RPL; ++u) s[gl + LP * u] = v[u];
+    for (int u = 0; u < RT; ++u) s[gl + LP * u] = v[u];
   };
   const int posn[2] = {rank, NB - 1 - rank};
   int dst_cta[2], dst_top[2];
@@ -298,7 +368,7 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
     load(x, col(top, wc));
     load(y, col(bot, wc));
     {
-      const R na = col_norm2<LP, R, RPL>(x), nb = col_norm2<LP, R, RPL>(y);
+      const R na = col_norm2<LP, RPL>(x), nb = col_norm2<LP, RPL>(y);
       if (gl == 0 && act) {
         nrm[top * bs + w] = na;
         nrm[bot * bs + w] = nb;
@@ -321,7 +391,7 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
           load(y, col(slot, i1));
         }
         R al = nrm[slot * bs + i0], be = nrm[slot * bs + i1];
-        const int f = rotate_pair<LP, R, RPL>(x, y, al, be, tol2, big2, lane, on);
+        const int f = rotate_pair<LP, RPL>(x, y, al, be, tol2, big2, lane, on);
         if (f) {
           wf |= f;
           store(x, col(slot, j0));
@@ -341,7 +411,7 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
       for (int s = 0; s < bs; ++s) {
         if (act) load(y, col(bot, c));  // (an idle group's values are not used)
         R be = nrm[bot * bs + c];
-        const int f = rotate_pair<LP, R, RPL>(x, y, al, be, tol2, big2, lane, act);
+        const int f = rotate_pair<LP, RPL>(x, y, al, be, tol2, big2, lane, act);
         wf |= f;
         if (s + 1 < bs) {
           if (f) {
@@ -401,7 +471,7 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
   // column norms (whole columns are local), gathered in every CTA
   load(x, col(top, wc));
   load(y, col(bot, wc));
-  const R nx = sqrt(col_norm2<LP, R, RPL>(x)), ny = sqrt(col_norm2<LP, R, RPL>(y));
+  const R nx = sqrt(col_norm2<LP, RPL>(x)), ny = sqrt(col_norm2<LP, RPL>(y));
   const int cx = rank * bs + wc, cy = (NB - 1 - rank) * bs + wc;
   if (act)
     for (int i = gl; i < NC; i += LP) {
@@ -424,6 +494,26 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
     }
     return gsum<LP>(rk);
   };
+  if constexpr (PRE) {
+    zc* Vt = a.Vt + bt * (int64_t)q * q;
+    const int64_t eye = (int64_t)gridDim.y * q * q;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int c = h == 0 ? cx : cy;
+      const int rk = place(min(c, q - 1));
+      if (c >= q || !act) continue;
+#pragma unroll
+      for (int u = 0; u < RPL; ++u) {
+        const int i = gl + LP * u;
+        if (i >= q) continue;
+        const C g = h == 0 ? x[RPL + u] : y[RPL + u];
+        const int64_t o = (int64_t)rk * q + i;
+        Vt[o] = zc(g.re, g.im);
+        Vt[eye + o] = Vt[2 * eye + o] = zc(i == rk ? 1.0 : 0.0, 0.0);
+      }
+    }
+    return;
+  }
   const R sb = jac_pow2(R(0), esc);
   for (int c0 = 0; c0 < q; c0 += ng) {
     const int c = min(c0 + w, q - 1), rk = place(c);
@@ -505,6 +595,7 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
 struct JacPlan {
   int nc, bs, lp, rpl, warps;
   size_t smem;
+  double cost;  // cycles of a sweep
 };
 
 // instances: rows held by a group of lp lanes, rpl each
@@ -541,7 +632,7 @@ bool jac_rows(int p, int lp, int* rpl) {
 // FP32 103.6 / 88.1, 128 x 72 FP32 39.9 / 32.8; FP64, with the FP64 instructions
 // of the scalars cut from about 45 to 27, 68 x 68 376 / 224, 124 x 124 597 / 467.
 template <class R>
-bool jac_plan(int p, int q, int batch, JacPlan* pl) {
+bool jac_plan(int p, int q, int batch, JacPlan* pl, bool pre = false) {
   if (p < 1 || q < 1 || p > 512 || q > 512 || batch < 1 || batch > 65535) return false;
   int ncmax = 16;
   while (ncmax > 1 && ncmax * batch > 160) ncmax /= 2;
@@ -550,7 +641,8 @@ bool jac_plan(int p, int q, int batch, JacPlan* pl) {
   for (int pass = 0; pass < 2 && best > 1e299; ++pass)  // second pass: whatever fits shared memory
     for (int lp : {32, 16}) {
       int rpl;
-      if (!jac_rows<R>(p, lp, &rpl)) continue;
+      if (!jac_rows<R>(p, lp, &rpl) || (pre && rpl > 8)) continue;
+      if (pre) rpl *= 2;
       for (int nc = 1; nc <= (pass ? 16 : ncmax); ++nc) {
         const int bs = (q + 2 * nc - 1) / (2 * nc), warps = (bs * lp + 31) / 32;
         if (nc > 1 && (2 * nc - 2) * bs >= q) continue;  // a CTA less would hold them
@@ -568,16 +660,16 @@ bool jac_plan(int p, int q, int batch, JacPlan* pl) {
         const double cost = (2 * nc - 1) * (bs * c + e) + (bs + (bs & 1)) * c;
         if (cost < best) {
           best = cost;
-          *pl = JacPlan{nc, bs, lp, rpl, warps, sm};
+          *pl = JacPlan{nc, bs, lp, pre ? rpl / 2 : rpl, warps, sm, cost};
         }
       }
     }
   return best < 1e299;
 }
 
-template <class R, int LP, int RPL>
+template <class R, int LP, int RPL, bool PRE = false>
 int launch(const JacArgs<R>& a, const JacPlan& pl, int batch, cudaStream_t s) {
-  const void* fn = (const void*)jacobi_cluster2_kernel<R, LP, RPL>;
+  const void* fn = (const void*)jacobi_cluster2_kernel<R, LP, RPL, PRE>;
   if (qtt_allow_max_smem(fn) != QTT_OK) return QTT_ERR_CUDA;
   if (pl.nc > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
     return QTT_ERR_CUDA;
@@ -593,7 +685,7 @@ int launch(const JacArgs<R>& a, const JacPlan& pl, int batch, cudaStream_t s) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, jacobi_cluster2_kernel<R, LP, RPL>, a) == cudaSuccess ? QTT_OK : QTT_ERR_CUDA;
+  return cudaLaunchKernelEx(&cfg, jacobi_cluster2_kernel<R, LP, RPL, PRE>, a) == cudaSuccess ? QTT_OK : QTT_ERR_CUDA;
 }
 
 }  // namespace
@@ -609,7 +701,8 @@ int qtt_svd(const cplx<R>* G, const int* perm, cplx<R>* Vh, R* sigma, int* trunc
             int max_rank, int mask, int p, int q, int batch, int max_sweeps, int* sweeps, cudaStream_t s) {
   JacPlan pl;
   if (!jac_plan<R>(p, q, batch, &pl)) return QTT_ERR_UNSUPPORTED;
-  const JacArgs<R> a{G, perm, Vh, sigma, trunc, delta, deltas, max_rank, mask, p, q, pl.bs, max_sweeps, sweeps};
+  const JacArgs<R> a{G,    perm,  Vh, sigma,      trunc,  delta,   deltas, max_rank, mask,
+                     p,    q,     pl.bs, max_sweeps, sweeps, nullptr, nullptr};
 #define QTT_J(LP, RPL) \
   if (pl.lp == LP && pl.rpl == RPL) return launch<R, LP, RPL>(a, pl, batch, s)
   if constexpr (sizeof(R) == 4) {
@@ -622,6 +715,29 @@ int qtt_svd(const cplx<R>* G, const int* perm, cplx<R>* Vh, R* sigma, int* trunc
 #undef QTT_J
   return QTT_ERR_UNSUPPORTED;
 }
+
+// FP32 rotations first where seven FP32 sweeps and the five products (about 80
+// us at 70 columns) cost less than the 4.5 sweeps that they save; this is so from
+// about 16 columns on (us of a rounding, without / with: 24 x 24 602 / 518, 16 x
+// 16 378 / 349, 12 x 12 293 / 279, 16 x 8 212 / 224, 8 x 8 197 / 210).
+bool qtt_svd_pre_fits(int p, int q, int batch) {
+  JacPlan pd, pf;
+  if (p < q || !jac_plan<double>(p, q, batch, &pd) || !jac_plan<float>(p, q, batch, &pf, true)) return false;
+  return 4.5 * pd.cost > 7.0 * pf.cost + 1.5e5;
+}
+
+int qtt_svd_pre(const zc* G, zc* Vt, int p, int q, int batch, int* sweeps, cudaStream_t s) {
+  JacPlan pl;
+  if (p < q || !jac_plan<float>(p, q, batch, &pl, true)) return QTT_ERR_UNSUPPORTED;
+  const JacArgs<float> a{nullptr, nullptr, nullptr, nullptr, nullptr, 0.0,    nullptr, 0, 0,
+                         p,       q,       pl.bs,   30,      sweeps,  G, Vt};
+#define QTT_J(RPL) \
+  if (pl.rpl == RPL) return launch<float, 32, RPL, true>(a, pl, batch, s)
+  QTT_J(1); QTT_J(2); QTT_J(3); QTT_J(4); QTT_J(5); QTT_J(6); QTT_J(8);
+#undef QTT_J
+  return QTT_ERR_UNSUPPORTED;
+}
+
 template bool qtt_svd_fits<float>(int, int, int);
 template bool qtt_svd_fits<double>(int, int, int);
 template int qtt_svd<float>(const cc*, const int*, cc*, float*, int*, double, const double*, int, int, int, int, int, int,

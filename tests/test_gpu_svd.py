@@ -1,0 +1,91 @@
+"""The SVD step of a rounding (sorted QR, FP64 column rotations started in FP32,
+cluster Jacobi; csrc/jacobi.cu) at the edges of its plans: rows next to a
+16- or 32-row slice and to the instances' limits, one to many columns per block,
+square and tall, and the spectra on which it can go wrong.
+
+A two-core train (U diag(s), W^H) of p modes and rank q has the SVD of its
+p x q matrix taken; U, s and W are known.
+
+Tolerances: the backward error of the QR and of the rotations is about
+sqrt(k) u ||A|| in practice (k = p + q, u = 2^-24 or 2^-53), as is what rounding
+adds to the cosines of the vectors, which the rotations bring below 2 u:
+20 sqrt(k) u bounds the entries of the Gram matrix, 40 sqrt(k) u the norm of
+the reconstruction's error (two cores) beyond the tail that is cut."""
+import math
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def Q():
+    from paper_2512_07811_gb300 import qtt
+    return qtt
+
+
+@pytest.fixture(scope="module")
+def ctx(Q):
+    return Q.Context(0)
+
+
+def _unitary(rng, m, n):
+    q, r = np.linalg.qr(rng.standard_normal((m, n)) + 1j * rng.standard_normal((m, n)))
+    return q * (np.diag(r) / abs(np.diag(r)))
+
+
+def _spectrum(kind, q, fp32):
+    """values, the tolerance to round to, the rank that is left (the others are below a tenth of it in all)"""
+    if kind == "graded":  # all kept
+        return np.logspace(0, -3 if fp32 else -9, q), 0.0, q
+    k = (q + 1) // 2
+    s = np.full(q, (1e-6 if fp32 else 1e-12) / math.sqrt(q))
+    if kind == "noise":
+        s[:k] = np.logspace(0, -1 if fp32 else -4, k)
+    elif kind == "equal":  # one value many times: any basis of its space is as good
+        s[:k] = 1.0
+    else:  # pairs that single precision cannot tell apart
+        s[:k] = np.repeat(np.logspace(0, -1, (k + 1) // 2), 2)[:k] * (1 + 1e-9 * (np.arange(k) % 2))
+    return s, 1e-4 if fp32 else 1e-8, k
+
+
+SHAPES = [(1, 1), (2, 2), (5, 3), (16, 16), (17, 15), (32, 32), (33, 31), (64, 33), (65, 64), (96, 48), (97, 97),
+          (128, 16), (129, 65), (160, 129), (193, 100), (255, 33), (256, 128), (257, 40), (300, 7)]
+
+
+@pytest.mark.parametrize("p,q", SHAPES)
+@pytest.mark.parametrize("kind", ["graded", "noise", "equal", "pairs"])
+@pytest.mark.parametrize("fp32", [False, True])
+def test_svd_of_a_two_core_train(Q, ctx, p, q, kind, fp32):
+    rng = np.random.default_rng(p * 1000 + q)
+    s, eps, rank = _spectrum(kind, q, fp32)
+    x = [(_unitary(rng, q, q) * s)[None], _unitary(rng, p, q).conj().T[:, :, None]]
+    y, info = Q.tt_round(ctx, Q.TT.from_cores(ctx, x, Q.C64 if fp32 else Q.C128), eps)
+    assert y.ranks[1] == rank
+    a, b = [c.astype(np.complex128) for c in y.cores()]
+    b = b[:, :, 0]
+    u, tol = (2.0 ** -24 if fp32 else 2.0 ** -53), math.sqrt(p + q)
+    assert abs(b @ b.conj().T - np.eye(rank)).max() <= 20 * tol * u
+    err = np.linalg.norm(a[0] @ b - x[0][0] @ x[1][:, :, 0])
+    assert err <= np.linalg.norm(s[rank:]) + 40 * tol * u * np.linalg.norm(s)
+
+
+@pytest.mark.parametrize("p,q", [(17, 15), (64, 33), (128, 72)])
+@pytest.mark.parametrize("fp32", [False, True])
+def test_batch_with_a_rank_per_train(Q, ctx, p, q, fp32):
+    """Trains rounded together keep their own ranks; rows beyond them are cropped."""
+    rng = np.random.default_rng(p * 1000 + q + 1)
+    dt, xs = Q.C64 if fp32 else Q.C128, []
+    ranks = [1, q // 2, q]
+    for k in ranks:
+        s = np.full(q, (1e-6 if fp32 else 1e-12) / math.sqrt(q))
+        s[:k] = np.logspace(0, -1, k)
+        xs.append([(_unitary(rng, q, q) * s)[None], _unitary(rng, p, q).conj().T[:, :, None]])
+    ys, _ = Q.tt_round_batch(ctx, [Q.TT.from_cores(ctx, x, dt) for x in xs], 1e-4 if fp32 else 1e-8)
+    u, tol = (2.0 ** -24 if fp32 else 2.0 ** -53), math.sqrt(p + q)
+    for k, x, y in zip(ranks, xs, ys):
+        assert y.ranks[1] == k
+        a, b = [c.astype(np.complex128) for c in y.cores()]
+        ref = x[0][0] @ x[1][:, :, 0]
+        assert np.linalg.norm(a[0] @ b[:, :, 0] - ref) <= (1e-6 if fp32 else 1e-12) + 40 * tol * u * np.linalg.norm(ref)
