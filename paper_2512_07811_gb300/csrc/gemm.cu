@@ -168,48 +168,64 @@ gemm_midx_kernel(GemmDesc g, cplx<R> alpha, cplx<R> beta,
   }
 }
 
-// FP64 kernel: one output per thread, BM x BN outputs per CTA.  An SM issues two
-// FP64 FMAs a clock, so one warp's complex multiply-add holds its pipe for 64
-// cycles and the shared-memory traffic of one output per thread is hidden
-// under it; what counts is how many SMs work and how much of a tile is
-// padding.  With 32 x 32 tiles (the only choice below 38 tiles of 64 x 64)
-// 64 x 148 x 74 ran on 10 SMs in 94 us and 256 x 4 x 310, batch 144, spent seven
-// eighths of 2560 us on padding; see f64_tile() for the choice.  Sums run over
-// k in order, as in gemm_midx_kernel.
-template <int BM, int BN>
-__global__ void __launch_bounds__(BM * BN)
+// FP64 kernel: BM x BN outputs per CTA of 256 threads, KG threads per output that
+// take KD of every BK = KG KD values of k each.  An SM issues two FP64 FMAs a
+// clock, and each of its quarters holds its FP64 unit for 64 cycles per warp
+// instruction, so a warp's complex multiply-add takes 256 cycles whatever else
+// happens (the shared-memory traffic of one output per thread is hidden
+// under it): what counts is that every quarter of every SM has its share of
+// the work, and how much of a tile is padding.  Hence tiles from 16 x 16 down to
+// 4 x 4, always with eight warps; see f64_tile() for the choice.  The KG partial
+// sums are added pairwise in a fixed order.
+template <int BM, int BN, int KG, int BK>
+__global__ void __launch_bounds__(256)
 gemm_f64_kernel(GemmDesc g, zc alpha, zc beta, const zc* __restrict__ A, const zc* __restrict__ B, zc* __restrict__ C,
                 int splits, int64_t kchunk, zc* __restrict__ P) {
-  constexpr int NT = BM * BN, BK = 16;
-  __shared__ zc As[BK][BM + 1], Bs[BK][BN + 1];
+  constexpr int NT = 256, NO = BM * BN, KD = BK / KG;
+  static_assert(NO * KG == NT && KD * KG == BK, "tile shape");
+  __shared__ zc As[BK][BM + 1], Bs[BK][BN + 1], red[KG > 1 ? NT / 2 : 1];
   const int64_t b = blockIdx.z / splits;
   const int split = blockIdx.z - (int)(b * splits);
   const int64_t kbeg = (int64_t)split * kchunk, kend = min(g.K, kbeg + kchunk);
-  const int64_t m0 = (int64_t)blockIdx.y * BM, n0 = (int64_t)blockIdx.x * BN;
-  const int tid = threadIdx.x, tn = tid % BN, tm = tid / BN;
+  const unsigned ntn = (unsigned)((g.N + BN - 1) / BN), row = blockIdx.x / ntn;
+  const int64_t m0 = (int64_t)row * BM, n0 = (int64_t)(blockIdx.x - row * ntn) * BN;
+  const int tid = threadIdx.x, o = tid % NO, kg = tid / NO, tn = o % BN, tm = o / BN;
+  const int64_t m = m0 + tm, n = n0 + tn;
+  const bool in = m < g.M && n < g.N;
   const zc* Ab = A + midx_off(g.bA, b);
   const zc* Bb = B + midx_off(g.bB, b);
   const bool a_kfast = midx_unit_inner(g.kA) && !midx_unit_inner(g.mA);
   const bool b_kfast = midx_unit_inner(g.kB) && !midx_unit_inner(g.nB);
   constexpr int LA = (BM * BK + NT - 1) / NT, LB = (BN * BK + NT - 1) / NT;
   zc ra[LA], rb[LB];
+  int64_t oa[LA], ob[LB];  // offsets of the rows and columns this thread loads, -1 beyond the matrix
+#pragma unroll
+  for (int l = 0; l < LA; ++l) {
+    const int e = tid + l * NT, mm = a_kfast ? e / BK : e % BM;
+    oa[l] = e < BM * BK && m0 + mm < g.M ? midx_off(g.mA, m0 + mm) : -1;
+  }
+#pragma unroll
+  for (int l = 0; l < LB; ++l) {
+    const int e = tid + l * NT, nn = b_kfast ? e / BK : e % BN;
+    ob[l] = e < BN * BK && n0 + nn < g.N ? midx_off(g.nB, n0 + nn) : -1;
+  }
   auto fetch = [&](int64_t k0) {
 #pragma unroll
     for (int l = 0; l < LA; ++l) {
-      const int e = tid + l * NT, mm = a_kfast ? e / BK : e % BM, kk = a_kfast ? e % BK : e / BM;
+      const int e = tid + l * NT, kk = a_kfast ? e % BK : e / BM;
       zc v(0, 0);
-      if (e < BM * BK && m0 + mm < g.M && k0 + kk < kend) {
-        v = Ab[midx_off(g.mA, m0 + mm) + midx_off(g.kA, k0 + kk)];
+      if (oa[l] >= 0 && k0 + kk < kend) {
+        v = Ab[oa[l] + midx_off(g.kA, k0 + kk)];
         if (g.conjA) v.im = -v.im;
       }
       ra[l] = v;
     }
 #pragma unroll
     for (int l = 0; l < LB; ++l) {
-      const int e = tid + l * NT, nn = b_kfast ? e / BK : e % BN, kk = b_kfast ? e % BK : e / BN;
+      const int e = tid + l * NT, kk = b_kfast ? e % BK : e / BN;
       zc v(0, 0);
-      if (e < BN * BK && n0 + nn < g.N && k0 + kk < kend) {
-        v = Bb[midx_off(g.nB, n0 + nn) + midx_off(g.kB, k0 + kk)];
+      if (ob[l] >= 0 && k0 + kk < kend) {
+        v = Bb[ob[l] + midx_off(g.kB, k0 + kk)];
         if (g.conjB) v.im = -v.im;
       }
       rb[l] = v;
@@ -230,25 +246,33 @@ gemm_f64_kernel(GemmDesc g, zc alpha, zc beta, const zc* __restrict__ A, const z
     }
     __syncthreads();
     if (k0 + BK < kend) fetch(k0 + BK);
-    const int kn = (int)min((int64_t)BK, kend - k0);
-    if (kn == BK) {
+    if (in) {  // (a warp of padding alone costs no FP64 time)
+      const int kb = kg * KD, kn = (int)min((int64_t)KD, kend - k0 - kb);
+      if (kn == KD) {
 #pragma unroll
-      for (int kk = 0; kk < BK; ++kk) cfma(acc, As[kk][tm], Bs[kk][tn]);
-    } else {
-      for (int kk = 0; kk < kn; ++kk) cfma(acc, As[kk][tm], Bs[kk][tn]);
+        for (int kk = 0; kk < KD; ++kk) cfma(acc, As[kb + kk][tm], Bs[kb + kk][tn]);
+      } else {
+        for (int kk = 0; kk < kn; ++kk) cfma(acc, As[kb + kk][tm], Bs[kb + kk][tn]);
+      }
     }
     __syncthreads();
   }
-  const int64_t m = m0 + tm, n = n0 + tn;
-  if (m >= g.M || n >= g.N) return;
+#pragma unroll
+  for (int s = KG / 2; s > 0; s /= 2) {
+    if (kg >= s && kg < 2 * s) red[(kg - s) * NO + o] = acc;
+    __syncthreads();
+    if (kg < s) acc = acc + red[kg * NO + o];
+    __syncthreads();
+  }
+  if (kg > 0 || !in) return;
   if (splits > 1) {
     P[(((int64_t)split * g.batch + b) * g.M + m) * g.N + n] = acc;
     return;
   }
-  const int64_t o = midx_off(g.bC, b) + midx_off(g.mC, m) + midx_off(g.nC, n);
+  const int64_t oc = midx_off(g.bC, b) + midx_off(g.mC, m) + midx_off(g.nC, n);
   zc v = alpha * acc;
-  if (beta.re != 0.0 || beta.im != 0.0) v = v + beta * C[o];
-  C[o] = v;
+  if (beta.re != 0.0 || beta.im != 0.0) v = v + beta * C[oc];
+  C[oc] = v;
 }
 
 // C[b][m][n] = alpha sum_s P[s][b][m][n] + beta C[b][m][n], summed in split order
@@ -271,69 +295,75 @@ __global__ void splitk_reduce_kernel(GemmDesc g, cplx<R> alpha, cplx<R> beta, co
 
 }  // namespace
 
-// FP64 tile (BM, BN): 64 x 64 outputs (gemm_midx_kernel) where that makes two
-// waves of CTAs; else one output per thread, 256 per CTA where that fills the
-// SMs and 64 where not, the tile four wide in a dimension of at most four.
-static void f64_tile(const GemmDesc& g, int* bm, int* bn) {
+// FP32 tile edge: 64, or 32 for thin shapes and for grids of
+// 64 x 64 tiles that would not fill a quarter of the SMs.
+static int64_t gemm_tile(const GemmDesc& g) {
+  if (g.M <= 32 || g.N <= 32) return 32;
   const int64_t t64 = ((g.M + 63) / 64) * ((g.N + 63) / 64) * g.batch;
-  if (g.M > 32 && g.N > 32 && t64 >= 304) {
-    *bm = *bn = 64;
-    return;
+  return t64 < 38 ? 32 : 64;
+}
+
+// FP64 tile of a contraction: the one with the least time on the busiest SM, in
+// cycles: two FP64 FMAs a clock for the tile's 4 K BM BN (a few per cent less in the
+// 64-wide ones), and 350 per level of the KG sums for each CTA beyond the three
+// that hide one another's start.  us of one tile against another: 128 x 124 x 124
+// 16 x 16 41, 8 x 8 23, 4 x 4 27; 512 x 64 x 64 23, 25, 31; 74 x 68 x 74 27, 12, 10; 1024 x
+// 1024 x 1024 7220, 7550 (64 x 64, no longer there, 8330); 256 x 4 x 310, batch 144, 16 x 4
+// 367, 64 x 4 395, 4 x 4 410; 70000 x 3 x 2 64 x 4 20, 16 x 4 35.  Before this rule (8 x 8 by
+// two warps, 16 x 16 or 64 x 64 by the number of outputs) and with it: 144 x 4 x 72
+// 20.6 / 8.3, 74 x 68 x 74 22.6 / 12.3, 96 x 48 x 520 70 / 29, 144 x 72 x 1240 287 / 131, 310 x
+// 72 x 256, batch 8, 428 / 358 (floor 316).
+struct F64Tile {
+  int bm, bn, levels;
+  double work;
+};
+static const F64Tile kF64Tiles[] = {{16, 16, 0, 2.0}, {8, 8, 2, 2.0},  {4, 4, 4, 2.0}, {16, 4, 2, 2.0},
+                                    {4, 16, 2, 2.0},  {64, 4, 0, 2.1}, {4, 64, 0, 2.1}};
+
+static int64_t f64_tiles(const GemmDesc& g, int bm, int bn) {
+  return ((g.M + bm - 1) / bm) * ((g.N + bn - 1) / bn) * g.batch;
+}
+
+static const F64Tile& f64_tile(const GemmDesc& g) {
+  const F64Tile* best = kF64Tiles;
+  double cost = 1e300;
+  for (const F64Tile& t : kF64Tiles) {
+    const double ctas = (double)((f64_tiles(g, t.bm, t.bn) + 151) / 152);  // on the busiest SM
+    const double c = ctas * t.work * t.bm * t.bn * g.K + t.levels * (200.0 + 350.0 * std::max(0.0, ctas - 3));
+    if (c < cost) {
+      cost = c;
+      best = &t;
+    }
   }
-  const bool big = (g.M * g.N * g.batch) / 256 >= 152;
-  if (g.N <= 4) {
-    *bm = big ? 64 : 16;
-    *bn = 4;
-  } else if (g.M <= 4) {
-    *bm = 4;
-    *bn = big ? 64 : 16;
-  } else {
-    *bm = *bn = big && g.M > 8 && g.N > 8 ? 16 : 8;
-  }
+  return *best;
 }
 
 // K splits of an FP64 contraction: about one CTA per SM, at least 64 of K each
 int qtt_gemm_splits_f64(const GemmDesc& g) {
-  int bm, bn;
-  f64_tile(g, &bm, &bn);
-  const int64_t tiles = ((g.M + bm - 1) / bm) * ((g.N + bn - 1) / bn) * g.batch;
+  const F64Tile& t = f64_tile(g);
+  const int64_t tiles = f64_tiles(g, t.bm, t.bn);
   if (tiles >= 76 || g.K < 128) return 1;
   return (int)std::min<int64_t>(32, std::min<int64_t>((g.K + 63) / 64, std::max<int64_t>(1, 152 / tiles)));
 }
 
 static int launch_f64(const GemmDesc& g, zc alpha, zc beta, const zc* A, const zc* B, zc* C, int splits,
                       int64_t kchunk, zc* P, cudaStream_t s) {
-  int bm, bn;
-  f64_tile(g, &bm, &bn);
-  // a grid has at most 65535 tiles along m: taller ones take the wide tile
-  if ((g.M + bm - 1) / bm > 65535) bm = bn = 64;
-  const dim3 grid((unsigned)((g.N + bn - 1) / bn), (unsigned)((g.M + bm - 1) / bm), (unsigned)(g.batch * splits));
-  if (grid.y > 65535) return QTT_ERR_ARG;
-#define QTT_F64(X, Y) gemm_f64_kernel<X, Y><<<grid, X * Y, 0, s>>>(g, alpha, beta, A, B, C, splits, kchunk, P)
-  if (bm == 64 && bn == 64)
-    gemm_midx_kernel<double, 64, 64, 8, 4, 4><<<grid, 256, 0, s>>>(g, alpha, beta, A, B, C, splits, kchunk, P);
-  else if (bm == 16 && bn == 16)
-    QTT_F64(16, 16);
-  else if (bm == 8)
-    QTT_F64(8, 8);
-  else if (bm == 64)
-    QTT_F64(64, 4);
-  else if (bm == 16)
-    QTT_F64(16, 4);
-  else if (bn == 64)
-    QTT_F64(4, 64);
-  else
-    QTT_F64(4, 16);
+  const F64Tile& t = f64_tile(g);
+  const int64_t edge = gemm_tile(g);
+  if ((g.M + edge - 1) / edge > 65535 || g.batch * splits > 65535) return QTT_ERR_ARG;  // the sizes that FP32 takes
+  const dim3 grid((unsigned)(f64_tiles(g, t.bm, t.bn) / g.batch), 1, (unsigned)(g.batch * splits));
+#define QTT_F64(X, Y, KG, BK)    \
+  if (t.bm == X && t.bn == Y) \
+    gemm_f64_kernel<X, Y, KG, BK><<<grid, 256, 0, s>>>(g, alpha, beta, A, B, C, splits, kchunk, P)
+  QTT_F64(16, 16, 1, 16);
+  QTT_F64(8, 8, 4, 32);
+  QTT_F64(4, 4, 16, 64);
+  QTT_F64(16, 4, 4, 32);
+  QTT_F64(4, 16, 4, 32);
+  QTT_F64(64, 4, 1, 16);
+  QTT_F64(4, 64, 1, 16);
 #undef QTT_F64
   return QTT_OK;
-}
-
-// Tile edge of qtt_gemm_ex: 64, or 32 for thin shapes and for grids of
-// 64 x 64 tiles that would not fill a quarter of the SMs.
-static int64_t gemm_tile(const GemmDesc& g) {
-  if (g.M <= 32 || g.N <= 32) return 32;
-  const int64_t t64 = ((g.M + 63) / 64) * ((g.N + 63) / 64) * g.batch;
-  return t64 < 38 ? 32 : 64;
 }
 
 // Number of K splits worth using for this shape (1 = no split): GEMMs whose
@@ -353,8 +383,8 @@ int qtt_gemm_ex(const GemmDesc& g, cplx<R> alpha, cplx<R> beta, const cplx<R>* A
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return QTT_OK;
   if (splits < 1 || (splits > 1 && !P)) return QTT_ERR_ARG;
   const int64_t kchunk = splits > 1 ? (g.K + splits - 1) / splits : std::max<int64_t>(g.K, 1);
-  const bool thin = (tile ? tile : gemm_tile(g)) == 32;
-  constexpr int BK = sizeof(R) == 8 ? 8 : 16;
+  [[maybe_unused]] const bool thin = (tile ? tile : gemm_tile(g)) == 32;  // (FP64 chooses its own tiles)
+  constexpr int BK = 16;
   const int64_t zdim = g.batch * splits;
   if (zdim > 65535) return QTT_ERR_ARG;
   if constexpr (sizeof(R) == 8) {
@@ -392,17 +422,7 @@ int qtt_gemm_splits_for(const GemmDesc& g, int tile) {
 template <class R>
 int qtt_gemm(const GemmDesc& g, cplx<R> alpha, cplx<R> beta, const cplx<R>* A,
              const cplx<R>* B, cplx<R>* C, cudaStream_t s) {
-  if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return QTT_OK;
-  if (g.K <= 0) {
-    // C = beta * C; scale through the kernel with K = 0 (loop body skipped)
-  }
-  constexpr int BM = 64, BN = 64, TM = 4, TN = 4;
-  constexpr int BK = sizeof(R) == 8 ? 8 : 16;
-  dim3 grid((unsigned)((g.N + BN - 1) / BN), (unsigned)((g.M + BM - 1) / BM), (unsigned)g.batch);
-  if (grid.y > 65535 || grid.z > 65535) return QTT_ERR_ARG;
-  gemm_midx_kernel<R, BM, BN, BK, TM, TN><<<grid, (BM / TM) * (BN / TN), 0, s>>>(g, alpha, beta, A, B, C, 1,
-                                                                                std::max<int64_t>(g.K, 1), nullptr);
-  return cudaGetLastError() == cudaSuccess ? QTT_OK : QTT_ERR_CUDA;
+  return qtt_gemm_ex<R>(g, alpha, beta, A, B, C, 1, nullptr, s, 64);
 }
 
 template int qtt_gemm<double>(const GemmDesc&, zc, zc, const zc*, const zc*, zc*, cudaStream_t);
