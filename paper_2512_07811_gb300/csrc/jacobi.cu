@@ -39,6 +39,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "dense.cuh"
@@ -60,7 +61,7 @@ struct JacArgs {
   const double* deltas;   // per matrix instead of delta, or null
   int max_rank;           // 0: no cap
   int mask;               // rows of Vh from the kept rank on are zeroed
-  int p, q, bs, max_sweeps;
+  int p, q, bs, bsx, adapt, max_sweeps;  // bsx: the most columns a block may get; adapt: columns may be left out
   int* sweeps;
   // rotations only (PRE): the matrix in FP64, the accumulated rotations transposed (row j: the column of the j-th
   // largest norm, q x q), followed by two identity matrices of that size
@@ -68,10 +69,29 @@ struct JacArgs {
   zc* Vt;
 };
 
-template <class R>
+// most threads of a CTA: 256 where a pair's two columns take more than the 128
+// registers that 512 leave (up to 256 rows or columns, which sixteen CTAs of
+// eight warps hold)
+template <class R, int RT, bool PRE>
 struct JacThreads {
-  static constexpr int value = sizeof(R) == 8 ? 256 : 512;  // FP64 columns take twice the registers
+  static constexpr int value = sizeof(R) == 8 || PRE || (RT > 4 && RT <= 8) ? 256 : 512;
 };
+
+// cycles of a sweep, see jac_plan
+template <class R>
+__host__ __device__ inline float jac_cost(int nc, int bs, int lp, int rows) {
+  const int queue = ((bs * lp + 31) / 32 + 3) / 4;
+  float c, e = nc > 1 ? 600.f : 60.f;
+  if (sizeof(R) == 4) {
+    const float lat = 540.f + 22.f * rows, issue = queue * (150.f + 28.f * rows);
+    c = lat > issue ? lat : issue;
+    if (nc > 1) e += 100.f + 30.f * bs * lp * rows / 32;
+  } else {
+    c = queue * 64.f * (16.f * rows + 27.f) + 300.f;
+    if (nc > 1) e += 60.f * bs * lp * rows / 32;
+  }
+  return (2 * nc - 1) * (bs * c + e) + (bs + (bs & 1)) * c;
+}
 
 // sum over the LP lanes that share a pair (all lanes of the warp take part)
 template <int LP, class R>
@@ -237,97 +257,187 @@ __device__ __forceinline__ float jac_pow2(float, int e) { return ldexpf(1.f, e);
 __device__ __forceinline__ double jac_pow2(double, int e) { return ldexp(1.0, e); }
 
 template <class R, int LP, int RPL, bool PRE>
-__global__ void __launch_bounds__(JacThreads<R>::value, 1)
+__global__ void __launch_bounds__(JacThreads<R, RPL, PRE>::value, 1)
 jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
   typedef cplx<R> C;
   cg::cluster_group cluster = cg::this_cluster();
-  const int NC = (int)cluster.num_blocks(), NB = 2 * NC, rank = (int)cluster.block_rank();
-  const int p = a.p, q = a.q, bs = a.bs, qp = NB * bs;
+  typedef typename std::conditional<PRE, double, R>::type S;  // type of the matrix
+  const int rank = (int)cluster.block_rank(), p = a.p, q = a.q;
+  // active CTAs of the cluster, columns of a block, columns worked on
+  int NC = (int)cluster.num_blocks(), bs = a.bs, qa = q;
   constexpr int RT = PRE ? 2 * RPL : RPL, LD = LP * RT;
-  const int lane = threadIdx.x & 31, nthr = blockDim.x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int nthr = blockDim.x;
   // a pair is worked on by a group of LP lanes: group w of ng, lane gl of it
-  const int gl = lane % LP, w = threadIdx.x / LP, ng = nthr / LP;
-  const bool act = w < bs;       // this group has a column of either block
-  const int wc = act ? w : 0;
+  const int gl = lane % LP, w = threadIdx.x / LP;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* slots = reinterpret_cast<C*>(smem_raw);                 // [4][bs][LD]
-  double* scan = reinterpret_cast<double*>(slots + (size_t)4 * bs * LD);  // 2 of the truncation rule
+  double* scan = reinterpret_cast<double*>(slots + (size_t)4 * a.bsx * LD);  // [0] squared norm of the dropped columns
   R* nrm = reinterpret_cast<R*>(scan + 2);                   // [4][bs] squared norms
-  R* norms = nrm + 4 * bs;                                   // [qp] final norms
-  R* sorted = norms + qp;                                    // [qp]
-  int* flags = reinterpret_cast<int*>(sorted + qp);          // [2][NC] sweep flags, then [NC] exponents
-  int* s_int = flags + 3 * 16;                               // [0] sweep flags of this CTA, [1] kept rank
+  R* norms = nrm + 4 * a.bsx;                                // [qp] final norms
+  R* sorted = norms + q + 64;                                // [qp]
+  int* flags = reinterpret_cast<int*>(sorted + q + 64);      // [2][NC] sweep flags, then [NC] exponents
+  int* s_int = flags + 3 * 16;                               // [0] sweep flags of this CTA, [1] kept rank, [2..4] plan
   const int64_t bt = blockIdx.y;
-  auto col = [&](int slot, int j) { return slots + ((size_t)slot * bs + j) * LD; };
+  auto col = [&](int slot, int j) { return slots + (slot * a.bsx + j) * LD; };
   int top = 0, bot = 1, in_top = 2, in_bot = 3;
   if (threadIdx.x == 0) s_int[0] = 0;
   cluster.sync();
-  // initial blocks (rank on top, NB-1-rank below), and the power of two that
-  // brings the largest component near 1 (FP32: near 2^14, so that squares of
-  // squared norms of columns down to 1e-14 of the largest stay normal)
-  int esc;
-  if constexpr (PRE) {
-    const zc* G = a.Gd + bt * (int64_t)p * q;
-    double amax = 0;
-    for (int e = threadIdx.x; e < 2 * bs * p; e += nthr) {
+  const cplx<S>* G;
+  if constexpr (PRE) G = a.Gd; else G = a.G;
+  G += bt * (int64_t)p * q;
+  // blocks of this CTA: rank on top, 2 NC - 1 - rank below
+  auto blocks = [&](auto&& f) {
+    for (int e = threadIdx.x; e < 2 * bs * LD; e += nthr) {
       const int i = e / (2 * bs), jj = e - i * 2 * bs, half = jj / bs, j = jj - half * bs;
-      const int c = (half == 0 ? rank : NB - 1 - rank) * bs + j;
-      if (c >= q) continue;
-      const zc v = G[(int64_t)i * q + c];
-      amax = fmax(amax, fmax(fabs(v.re), fabs(v.im)));
+      const int c = (half == 0 ? rank : 2 * NC - 1 - rank) * bs + j;
+      f(c, i, col(half == 0 ? top : bot, j) + i);
     }
+  };
+  // the power of two that brings the largest component near 1 (FP32: near
+  // 2^14, so that squares of squared norms of columns down to 1e-14 of the
+  // largest stay normal)
+  const bool whole = PRE || a.adapt;  // the matrix is read before its columns are dealt out
+  S amax = 0;
+  // (rows dealt to the CTAs, a CTA's rows to groups of qg threads)
+  const int qg = min((q + 31) & ~31, nthr), ngr = nthr / qg, grp = threadIdx.x / qg, c0 = threadIdx.x - grp * qg;
+  if (whole) {
+    if (grp < ngr)
+      for (int c = c0; c < q; c += qg) {
+#pragma unroll 8
+        for (int i = rank + NC * grp; i < p; i += NC * ngr) {
+          const cplx<S> v = G[(int64_t)i * q + c];
+          amax = fmax(amax, fmax(fabs(v.re), fabs(v.im)));
+        }
+      }
+  } else if constexpr (!PRE) {
+    blocks([&](int c, int i, C* d) {
+      C v(0, 0);
+      if (c < q && i < p) v = G[(int64_t)i * q + c];
+      *d = v;
+      amax = fmax(amax, fmax(fabs(v.re), fabs(v.im)));
+    });
+  }
+  {
     const int ex = __reduce_max_sync(0xffffffffu, jac_exponent(amax));
-    int* wex = reinterpret_cast<int*>(sorted);  // (2 NC bs values hold one per warp)
-    if (lane == 0) wex[threadIdx.x >> 5] = ex;
+    int* wex = reinterpret_cast<int*>(sorted);
+    if (lane == 0) wex[warp] = ex;
     __syncthreads();
-    if (threadIdx.x < 32) {
+    if (warp == 0) {
       const int t = __reduce_max_sync(0xffffffffu, lane < (nthr >> 5) ? wex[lane] : -1000);
       if (lane < NC) cluster.map_shared_rank(flags, lane)[32 + rank] = t;
     }
     cluster.sync();
-    esc = flags[32];
-    for (int i = 1; i < NC; ++i) esc = max(esc, flags[32 + i]);
-    esc -= 14;
-    const double sg = jac_pow2(0.0, -esc);
-    for (int e = threadIdx.x; e < 2 * bs * LD; e += nthr) {
-      const int i = e / (2 * bs), jj = e - i * 2 * bs, half = jj / bs, j = jj - half * bs;
-      const int c = (half == 0 ? rank : NB - 1 - rank) * bs + j;
-      C v(0, 0);
-      if (c < q && i < p) {
-        const zc g = G[(int64_t)i * q + c];
-        v = C((R)(sg * g.re), (R)(sg * g.im));
-      } else if (c < q && i == LP * RPL + c) {
-        v = C(1, 0);
+  }
+  int esc = flags[32];
+  for (int i = 1; i < NC; ++i) esc = max(esc, flags[32 + i]);
+  if (sizeof(R) == 4) esc -= 14;
+  const S sg = jac_pow2(S(0), -esc);
+  if (a.adapt) {
+    // Trailing columns whose whole norm is at most eps ||G|| (one rounding of G)
+    // and a quarter of the truncation threshold are left out: in a rounding
+    // of a train with superfluous rank they are the noise of the QR, half of
+    // the columns.  Their norm counts as discarded, so the tail's bound holds.
+    // us without / with: 118 x 118 of rank 59 453 / 227, 172 x 172 of rank 85 852 /
+    // 412, FP64 68 x 68 of rank 33 475 / 356; where all columns stay 5 more.
+    R* parts = reinterpret_cast<R*>(slots);  // [NC][q] partial sums of the CTAs' rows, then [q] squared norms
+    R* cn = parts + NC * q;
+    R* own = cn + q;  // [ngr][q]
+    if (grp < ngr)
+      for (int c = c0; c < q; c += qg) {
+        R t = 0;
+#pragma unroll 8
+        for (int i = rank + NC * grp; i < p; i += NC * ngr) {
+          const cplx<S> v = G[(int64_t)i * q + c];
+          t += abs2(C((R)(sg * v.re), (R)(sg * v.im)));
+        }
+        own[grp * q + c] = t;
       }
-      col(half == 0 ? top : bot, j)[i] = v;
-    }
     __syncthreads();
-  } else {
-    R amax = 0;
-    for (int e = threadIdx.x; e < 2 * bs * LD; e += nthr) {
-      const int i = e / (2 * bs), jj = e - i * 2 * bs, half = jj / bs, j = jj - half * bs;
-      const int c = (half == 0 ? rank : NB - 1 - rank) * bs + j;
-      C v(0, 0);
-      if (c < q && i < p) v = a.G[bt * (int64_t)p * q + (int64_t)i * q + c];
-      col(half == 0 ? top : bot, j)[i] = v;
-      amax = fmax(amax, fmax(fabs(v.re), fabs(v.im)));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-    if (lane == 0) sorted[threadIdx.x >> 5] = amax;  // (2 NC bs values hold one per warp)
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      R t = lane < (nthr >> 5) ? sorted[lane] : R(0);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t = fmax(t, __shfl_xor_sync(0xffffffffu, t, o));
-      if (lane < NC) cluster.map_shared_rank(flags, lane)[32 + rank] = jac_exponent(t);
+    for (int c = threadIdx.x; c < q; c += nthr) {
+      R t = 0;
+      for (int g = 0; g < ngr; ++g) t += own[g * q + c];
+      for (int k = 0; k < NC; ++k) cluster.map_shared_rank(parts, k)[rank * q + c] = t;
     }
     cluster.sync();
-    esc = flags[32];
-    for (int i = 1; i < NC; ++i) esc = max(esc, flags[32 + i]);
-    if (sizeof(R) == 4) esc -= 14;
-    const R sg = jac_pow2(R(0), -esc);
-    for (int e = threadIdx.x; e < 2 * bs * LD; e += nthr) slots[e] = sg * slots[e];
+    for (int c = threadIdx.x; c < q; c += nthr) {
+      R t = 0;
+      for (int k = 0; k < NC; ++k) t += parts[k * q + c];
+      cn[c] = t;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      double tot = 0;
+      for (int j = lane; j < q; j += 32) tot += (double)cn[j];
+      tot = dense::wsum(tot);
+      constexpr double eps = sizeof(S) == 4 ? (double)FLT_EPSILON : DBL_EPSILON;
+      const double ds = 0.25 * (a.deltas ? a.deltas[bt] : a.delta) * jac_pow2(0.0, -esc);
+      double thr2 = eps * eps * tot;
+      if (!(ds * ds >= thr2)) thr2 = ds * ds;  // (a NaN drops nothing)
+      double out = 0;
+      int t = q;
+      for (int hi = q; hi > 1; hi -= 32) {
+        const int j = hi - 1 - lane;
+        double v = j >= 1 ? (double)cn[j] : 0.0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const double u = __shfl_up_sync(0xffffffffu, v, o);
+          if (lane >= o) v += u;
+        }
+        v += out;
+        const unsigned ok = __ballot_sync(0xffffffffu, j >= 1 && v <= thr2);
+        const int n = __ffs(~ok) - 1, cnt = n < 0 ? 32 : n;  // leading lanes that may go
+        t -= cnt;
+        if (cnt > 0) out = __shfl_sync(0xffffffffu, v, cnt - 1);
+        if (cnt < 32) break;
+      }
+      // the cheapest tournament of t columns on at most NC CTAs
+      const int nc = lane + 1, b = (t + 2 * nc - 1) / (2 * nc);
+      float cost = FLT_MAX;
+      if (nc <= NC && b <= a.bsx && (nc == 1 || (2 * nc - 2) * b < t)) cost = jac_cost<R>(nc, b, LP, RT);
+      int best = nc;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const float oc = __shfl_xor_sync(0xffffffffu, cost, o);
+        const int on = __shfl_xor_sync(0xffffffffu, best, o);
+        if (oc < cost || (oc == cost && on < best)) {
+          cost = oc;
+          best = on;
+        }
+      }
+      if (lane == 0) {
+        scan[0] = out;
+        s_int[2] = best;
+        s_int[3] = (t + 2 * best - 1) / (2 * best);
+        s_int[4] = t;
+      }
+    }
+    __syncthreads();
+    NC = s_int[2];
+    bs = s_int[3];
+    qa = s_int[4];
+    nthr = (bs * LP + 31) & ~31;
+    if (rank >= NC || threadIdx.x >= nthr) return;  // (the barriers wait for the threads that are left)
+  }
+  const int ng = nthr / LP;
+  const int NB = 2 * NC;
+  const bool act = w < bs;       // this group has a column of either block
+  const int wc = act ? w : 0;
+  if (whole) {
+    blocks([&](int c, int i, C* d) {
+      C v(0, 0);
+      if (c < qa && i < p) {
+        const cplx<S> g = G[(int64_t)i * q + c];
+        v = C((R)(sg * g.re), (R)(sg * g.im));
+      } else if (PRE && c < qa && i == LP * RPL + c) {
+        v = C(1, 0);
+      }
+      *d = v;
+    });
+    // (the partial sums lay where another CTA's columns arrive)
+    if (NC > 1) cluster.sync(); else __syncthreads();
+  } else {
+    for (int e = threadIdx.x; e < 2 * bs * LD; e += nthr) slots[e] = (R)sg * slots[e];  // (bsx = bs)
     __syncthreads();
   }
   // Pairs are rotated down to a cosine of eps / 2 (the inner product's own
@@ -341,9 +451,9 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
   // Quadratic regime: a rotation by sin s_ij of a pair (i, j) puts back s_ij g_jk
   // into an annihilated g_ik.  With c the largest cosine and s the largest
   // sine weighted by the norms' ratio of a sweep, the cosines after it are at
-  // most about sqrt(q) s c; with both at most sqrt(tol / sqrt(q)) they are at
+  // most about sqrt(qa) s c; with both at most sqrt(tol / sqrt(qa)) they are at
   // most tol, and the next sweep would rotate nothing.
-  const R big2 = tol / sqrt(R(q));
+  const R big2 = tol / sqrt(R(qa));
   C x[RT], y[RT];
   auto load = [&](C(&v)[RT], const C* s) {
 #pragma unroll
@@ -370,8 +480,8 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
     {
       const R na = col_norm2<LP, RPL>(x), nb = col_norm2<LP, RPL>(y);
       if (gl == 0 && act) {
-        nrm[top * bs + w] = na;
-        nrm[bot * bs + w] = nb;
+        nrm[top * a.bsx + w] = na;
+        nrm[bot * a.bsx + w] = nb;
       }
     }
     __syncthreads();
@@ -390,15 +500,15 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
           load(x, col(slot, i0));
           load(y, col(slot, i1));
         }
-        R al = nrm[slot * bs + i0], be = nrm[slot * bs + i1];
+        R al = nrm[slot * a.bsx + i0], be = nrm[slot * a.bsx + i1];
         const int f = rotate_pair<LP, RPL>(x, y, al, be, tol2, big2, lane, on);
         if (f) {
           wf |= f;
           store(x, col(slot, j0));
           store(y, col(slot, j1));
           if (gl == 0) {
-            nrm[slot * bs + j0] = al;
-            nrm[slot * bs + j1] = be;
+            nrm[slot * a.bsx + j0] = al;
+            nrm[slot * a.bsx + j1] = be;
           }
         }
       }
@@ -406,17 +516,17 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
     }
     for (int br = 0; br < NB - 1; ++br) {
       load(x, col(top, wc));
-      R al = nrm[top * bs + wc];
+      R al = nrm[top * a.bsx + wc];
       int c = wc;
       for (int s = 0; s < bs; ++s) {
         if (act) load(y, col(bot, c));  // (an idle group's values are not used)
-        R be = nrm[bot * bs + c];
+        R be = nrm[bot * a.bsx + c];
         const int f = rotate_pair<LP, RPL>(x, y, al, be, tol2, big2, lane, act);
         wf |= f;
         if (s + 1 < bs) {
           if (f) {
             store(y, col(bot, c));
-            if (gl == 0) nrm[bot * bs + c] = be;
+            if (gl == 0) nrm[bot * a.bsx + c] = be;
           }
           __syncthreads();
           c = c + 1 == bs ? 0 : c + 1;
@@ -425,19 +535,19 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
           // both blocks to their next CTA, straight from the registers
           const int st = dst_top[0] ? in_top : in_bot, sb = dst_top[1] ? in_top : in_bot;
           C* rs = cluster.map_shared_rank(slots, dst_cta[0]);
-          store(x, rs + ((size_t)st * bs + w) * LD);
+          store(x, rs + (st * a.bsx + w) * LD);
           C* rb = cluster.map_shared_rank(slots, dst_cta[1]);
-          store(y, rb + ((size_t)sb * bs + c) * LD);
+          store(y, rb + (sb * a.bsx + c) * LD);
           if (gl == 0) {
-            cluster.map_shared_rank(nrm, dst_cta[0])[st * bs + w] = al;
-            cluster.map_shared_rank(nrm, dst_cta[1])[sb * bs + c] = be;
+            cluster.map_shared_rank(nrm, dst_cta[0])[st * a.bsx + w] = al;
+            cluster.map_shared_rank(nrm, dst_cta[1])[sb * a.bsx + c] = be;
           }
         } else {
           store(x, col(top, w));
           store(y, col(bot, c));
           if (gl == 0) {
-            nrm[top * bs + w] = al;
-            nrm[bot * bs + c] = be;
+            nrm[top * a.bsx + w] = al;
+            nrm[bot * a.bsx + c] = be;
           }
         }
       }
@@ -488,7 +598,7 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
   auto place = [&](int c) {
     const R v = key(c);
     int rk = 0;
-    for (int i = gl; i < q; i += LP) {
+    for (int i = gl; i < qa; i += LP) {
       const R u = key(i);
       rk += (u > v) || (u == v && i < c);
     }
@@ -500,8 +610,8 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int c = h == 0 ? cx : cy;
-      const int rk = place(min(c, q - 1));
-      if (c >= q || !act) continue;
+      const int rk = place(min(c, qa - 1));
+      if (c >= qa || !act) continue;
 #pragma unroll
       for (int u = 0; u < RPL; ++u) {
         const int i = gl + LP * u;
@@ -512,26 +622,31 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
         Vt[eye + o] = Vt[2 * eye + o] = zc(i == rk ? 1.0 : 0.0, 0.0);
       }
     }
+    for (int e = rank * nthr + threadIdx.x; e < (q - qa) * q; e += NC * nthr) {  // dropped columns stay
+      const int64_t o = (int64_t)qa * q + e;
+      Vt[o] = Vt[eye + o] = Vt[2 * eye + o] = zc(o / q == o % q ? 1.0 : 0.0, 0.0);
+    }
     return;
   }
   const R sb = jac_pow2(R(0), esc);
-  for (int c0 = 0; c0 < q; c0 += ng) {
-    const int c = min(c0 + w, q - 1), rk = place(c);
-    if (gl == 0 && c0 + w < q) sorted[rk] = norms[c] * sb;
+  for (int k0 = 0; k0 < qa; k0 += ng) {
+    const int c = min(k0 + w, qa - 1), rk = place(c);
+    if (gl == 0 && k0 + w < qa) sorted[rk] = norms[c] * sb;
   }
   __syncthreads();
   if (a.sigma && rank == 0)
     for (int i = threadIdx.x; i < q; i += nthr) a.sigma[bt * q + i] = sorted[i];
-  int keep = q;
+  int keep = qa;
   if (a.trunc) {
     // smallest t >= 1 with sqrt(sum_{j >= t} s_j^2) <= delta, sums in double
     // by a suffix scan over the lanes, 32 values at a time from the end
     if (threadIdx.x < 32) {
       const double delta = a.deltas ? a.deltas[bt] : a.delta;
-      double tail = 0.0;
-      int t = q;
+      const double sq = jac_pow2(0.0, esc);
+      double tail = qa < q ? scan[0] * sq * sq : 0.0;
+      int t = qa;
       bool stop = false;
-      for (int hi = q; hi > 1 && !stop; hi -= 32) {
+      for (int hi = qa; hi > 1 && !stop; hi -= 32) {
         const int j = hi - 1 - lane;  // lane 0 the last value
         const double v = j >= 1 ? (double)sorted[j] : 0.0;
         double s = v * v;
@@ -575,8 +690,8 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int c = h == 0 ? cx : cy;
-    const int rk = place(min(c, q - 1));
-    if (c >= q || !act) continue;
+    const int rk = place(min(c, qa - 1));
+    if (c >= qa || !act) continue;
     const R v = h == 0 ? nx : ny;
     R f = v > Lim<R>::tiny * R(4) ? R(1) / v : R(0);
     if (a.mask && rk >= keep) f = 0;
@@ -590,10 +705,11 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
       Vh[(int64_t)rk * p + (perm ? perm[i] : i)] = o;
     }
   }
+  for (int e = rank * nthr + threadIdx.x; e < (q - qa) * p; e += NC * nthr) Vh[(int64_t)qa * p + e] = C(0, 0);
 }
 
 struct JacPlan {
-  int nc, bs, lp, rpl, warps;
+  int nc, bs, lp, rpl, warps, bsx, adapt;
   size_t smem;
   double cost;  // cycles of a sweep
 };
@@ -617,6 +733,11 @@ bool jac_rows(int p, int lp, int* rpl) {
   return first({1, 2, 4});
 }
 
+template <class R>
+size_t jac_smem(int q, int bs, int ld) {
+  return (size_t)4 * bs * ld * sizeof(cplx<R>) + 16 + (4 * bs + (size_t)2 * (q + 64)) * sizeof(R) + 56 * sizeof(int) + 16;
+}
+
 // Cluster size, lanes per pair and column width, by the cost of a sweep in
 // cycles: (2 nc - 1) block-rounds of bs rounds and one exchange, bs rounds inside
 // the blocks.  A round costs its latency, or where that is more what its warps
@@ -636,35 +757,44 @@ bool jac_plan(int p, int q, int batch, JacPlan* pl, bool pre = false) {
   if (p < 1 || q < 1 || p > 512 || q > 512 || batch < 1 || batch > 65535) return false;
   int ncmax = 16;
   while (ncmax > 1 && ncmax * batch > 160) ncmax /= 2;
-  const int wmax = JacThreads<R>::value / 32;
   double best = 1e300;
   for (int pass = 0; pass < 2 && best > 1e299; ++pass)  // second pass: whatever fits shared memory
     for (int lp : {32, 16}) {
       int rpl;
       if (!jac_rows<R>(p, lp, &rpl) || (pre && rpl > 8)) continue;
+      const int wmax = sizeof(R) == 8 || pre || (rpl > 4 && rpl <= 8) ? 8 : 16;
       if (pre) rpl *= 2;
       for (int nc = 1; nc <= (pass ? 16 : ncmax); ++nc) {
         const int bs = (q + 2 * nc - 1) / (2 * nc), warps = (bs * lp + 31) / 32;
         if (nc > 1 && (2 * nc - 2) * bs >= q) continue;  // a CTA less would hold them
-        const size_t sm = (size_t)4 * bs * lp * rpl * sizeof(cplx<R>) + 16 +
-                          (4 * bs + (size_t)std::max(4 * nc * bs, 64)) * sizeof(R) + (48 + 4) * sizeof(int) + 16;
+        const size_t sm = jac_smem<R>(q, bs, lp * rpl);
         if (warps > wmax || sm > 200 * 1024) continue;
-        double c, e = nc > 1 ? 600.0 : 60.0;
-        if (sizeof(R) == 4) {
-          c = std::max(540.0 + 22.0 * rpl, (warps + 3) / 4 * (150.0 + 28.0 * rpl));
-          if (nc > 1) e += 100.0 + 30.0 * bs * lp * rpl / 32;
-        } else {
-          c = (warps + 3) / 4 * 64.0 * (16.0 * rpl + 27.0) + 300.0;
-          if (nc > 1) e += 60.0 * bs * lp * rpl / 32;
-        }
-        const double cost = (2 * nc - 1) * (bs * c + e) + (bs + (bs & 1)) * c;
+        const double cost = jac_cost<R>(nc, bs, lp, rpl);
         if (cost < best) {
           best = cost;
-          *pl = JacPlan{nc, bs, lp, pre ? rpl / 2 : rpl, warps, sm, cost};
+          *pl = JacPlan{nc, bs, lp, pre ? rpl / 2 : rpl, warps, bs, 0, sm, cost};
         }
       }
     }
   return best < 1e299;
+}
+
+// Columns may be left out (see the kernel) where that can save more than the 5 us
+// it takes to look for them (a sweep of 48 FP32 columns takes 19 us); a block may then be wider, since fewer CTAs can be
+// quicker for fewer columns.
+template <class R>
+void jac_adapt(JacPlan* pl, int q, bool pre) {
+  if (q < (sizeof(R) == 4 && !pre ? 48 : 24)) return;
+  const int ld = pl->lp * pl->rpl * (pre ? 2 : 1), b = std::max(pl->bs, sizeof(R) == 4 ? 8 : 4);
+  const size_t sm = jac_smem<R>(q, b, ld);
+  const int threads = (b * pl->lp + 31) / 32 * 32;  // (a partial sum each, or per column)
+  if (sm > 200 * 1024 ||
+      ((size_t)(pl->nc + 1) * q + std::max(threads, q)) * sizeof(R) > (size_t)4 * b * ld * sizeof(cplx<R>))
+    return;
+  pl->bsx = b;
+  pl->adapt = 1;
+  pl->smem = sm;
+  pl->warps = (b * pl->lp + 31) / 32;
 }
 
 template <class R, int LP, int RPL, bool PRE = false>
@@ -701,8 +831,9 @@ int qtt_svd(const cplx<R>* G, const int* perm, cplx<R>* Vh, R* sigma, int* trunc
             int max_rank, int mask, int p, int q, int batch, int max_sweeps, int* sweeps, cudaStream_t s) {
   JacPlan pl;
   if (!jac_plan<R>(p, q, batch, &pl)) return QTT_ERR_UNSUPPORTED;
-  const JacArgs<R> a{G,    perm,  Vh, sigma,      trunc,  delta,   deltas, max_rank, mask,
-                     p,    q,     pl.bs, max_sweeps, sweeps, nullptr, nullptr};
+  if (trunc && !sigma) jac_adapt<R>(&pl, q, false);
+  const JacArgs<R> a{G, perm,  Vh,     sigma,    trunc,      delta,  deltas,  max_rank, mask,
+                     p, q,     pl.bs,  pl.bsx,   pl.adapt,   max_sweeps, sweeps, nullptr, nullptr};
 #define QTT_J(LP, RPL) \
   if (pl.lp == LP && pl.rpl == RPL) return launch<R, LP, RPL>(a, pl, batch, s)
   if constexpr (sizeof(R) == 4) {
@@ -726,11 +857,13 @@ bool qtt_svd_pre_fits(int p, int q, int batch) {
   return 4.5 * pd.cost > 7.0 * pf.cost + 1.5e5;
 }
 
-int qtt_svd_pre(const zc* G, zc* Vt, int p, int q, int batch, int* sweeps, cudaStream_t s) {
+int qtt_svd_pre(const zc* G, zc* Vt, bool trunc, double delta, const double* deltas, int p, int q, int batch,
+                int* sweeps, cudaStream_t s) {
   JacPlan pl;
   if (p < q || !jac_plan<float>(p, q, batch, &pl, true)) return QTT_ERR_UNSUPPORTED;
-  const JacArgs<float> a{nullptr, nullptr, nullptr, nullptr, nullptr, 0.0,    nullptr, 0, 0,
-                         p,       q,       pl.bs,   30,      sweeps,  G, Vt};
+  if (trunc) jac_adapt<float>(&pl, q, true);
+  const JacArgs<float> a{nullptr, nullptr, nullptr, nullptr, nullptr,  delta, deltas, 0, 0,
+                         p,       q,       pl.bs,   pl.bsx,  pl.adapt, 30,    sweeps, G, Vt};
 #define QTT_J(RPL) \
   if (pl.rpl == RPL) return launch<float, 32, RPL, true>(a, pl, batch, s)
   QTT_J(1); QTT_J(2); QTT_J(3); QTT_J(4); QTT_J(5); QTT_J(6); QTT_J(8);

@@ -49,7 +49,9 @@ int qtt_svd(const cplx<R>* G, const int* perm, cplx<R>* Vh, R* sigma, int* trunc
 // Column rotations of an FP64 matrix computed in FP32: V with the columns of G V orthogonal to about 1e-6, V itself
 // unitary to FP32 rounding.  Vt (3 batch q^2 elements): V transposed, then two identity matrices per matrix.
 bool qtt_svd_pre_fits(int p, int q, int batch);  // where that and the FP64 products are cheaper than the sweeps saved
-int qtt_svd_pre(const zc* G, zc* Vt, int p, int q, int batch, int* sweeps, cudaStream_t s);
+// (trunc: the vectors are truncated at delta, deltas[b] if not null, as by qtt_svd)
+int qtt_svd_pre(const zc* G, zc* Vt, bool trunc, double delta, const double* deltas, int p, int q, int batch,
+                int* sweeps, cudaStream_t s);
 // whether qtt_qr_cluster takes the shape with sorted columns
 template <class R>
 bool qtt_qr_cluster_fits(int64_t m, int64_t n, int64_t batch);

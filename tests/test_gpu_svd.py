@@ -39,6 +39,11 @@ def _spectrum(kind, q, fp32):
     """values, the tolerance to round to, the rank that is left (the others are below a tenth of it in all)"""
     if kind == "graded":  # all kept
         return np.logspace(0, -3 if fp32 else -9, q), 0.0, q
+    if kind == "deficient":  # columns of rounding noise, which may be left out
+        k = q // 3 + 1
+        s = np.zeros(q)
+        s[:k] = np.logspace(0, -1 if fp32 else -4, k)
+        return s, 1e-4 if fp32 else 1e-8, k
     k = (q + 1) // 2
     s = np.full(q, (1e-6 if fp32 else 1e-12) / math.sqrt(q))
     if kind == "noise":
@@ -51,11 +56,11 @@ def _spectrum(kind, q, fp32):
 
 
 SHAPES = [(1, 1), (2, 2), (5, 3), (16, 16), (17, 15), (32, 32), (33, 31), (64, 33), (65, 64), (96, 48), (97, 97),
-          (128, 16), (129, 65), (160, 129), (193, 100), (255, 33), (256, 128), (257, 40), (300, 7)]
+          (128, 16), (129, 65), (160, 129), (193, 100), (200, 24), (255, 33), (256, 128), (257, 40), (300, 7)]
 
 
 @pytest.mark.parametrize("p,q", SHAPES)
-@pytest.mark.parametrize("kind", ["graded", "noise", "equal", "pairs"])
+@pytest.mark.parametrize("kind", ["graded", "noise", "equal", "pairs", "deficient"])
 @pytest.mark.parametrize("fp32", [False, True])
 def test_svd_of_a_two_core_train(Q, ctx, p, q, kind, fp32):
     rng = np.random.default_rng(p * 1000 + q)
