@@ -117,17 +117,6 @@ __global__ void sumsq_kernel(const cplx<R>* __restrict__ x, int64_t count, doubl
   }
 }
 
-__global__ void z2c_kernel(const zc* __restrict__ in, cc* __restrict__ out, int64_t count) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < count;
-       e += (int64_t)gridDim.x * blockDim.x)
-    out[e] = cc((float)in[e].re, (float)in[e].im);
-}
-__global__ void c2z_kernel(const cc* __restrict__ in, zc* __restrict__ out, int64_t count) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < count;
-       e += (int64_t)gridDim.x * blockDim.x)
-    out[e] = zc((double)in[e].re, (double)in[e].im);
-}
-
 template <class R>
 __global__ void copy_strided_kernel(const cplx<R>* __restrict__ in, MIdx rows, MIdx cols, int64_t nrows,
                                     int64_t ncols, int conj_in, cplx<R>* __restrict__ out, int64_t ldo) {
@@ -526,16 +515,6 @@ int qtt_scale(cplx<R>* x, int64_t count, cplx<R> sc, cudaStream_t s) {
 template <class R>
 int qtt_sumsq(const cplx<R>* x, int64_t count, double* out, cudaStream_t s) {
   sumsq_kernel<R><<<1, 1024, 0, s>>>(x, count, out);
-  CHECK_LAUNCH();
-}
-int qtt_convert_z2c(const zc* in, cc* out, int64_t count, cudaStream_t s) {
-  if (count <= 0) return QTT_OK;
-  z2c_kernel<<<nblocks(count), TPB, 0, s>>>(in, out, count);
-  CHECK_LAUNCH();
-}
-int qtt_convert_c2z(const cc* in, zc* out, int64_t count, cudaStream_t s) {
-  if (count <= 0) return QTT_OK;
-  c2z_kernel<<<nblocks(count), TPB, 0, s>>>(in, out, count);
   CHECK_LAUNCH();
 }
 template <class R>

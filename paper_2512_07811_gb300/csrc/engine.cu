@@ -671,7 +671,7 @@ static int svd_right(qtt_ctx* c, const cplx<R>* in, MIdx inB, MIdx rowI, MIdx co
       TRY(GV.alloc(c, (size_t)batch * n * q * sizeof(zc)));
       zc *v = V.as<zc>(), *e[2] = {v + batch * qq, v + 2 * batch * qq}, *v1 = V1.as<zc>();
       c->launches++;
-      TRY(qtt_svd_pre(G.as<zc>(), v, trunc && !sigma, delta, deltas, (int)n, (int)q, (int)batch, nullptr, c->stream));
+      TRY(qtt_svd_pre(G.as<zc>(), v, delta, deltas, (int)n, (int)q, (int)batch, nullptr, c->stream));
       for (int it = 0; it < 2; ++it) {
         // E = 3/2 - V^H V / 2, V <- V E (V stored transposed)
         TRY(simt_gemm<double>(c, bgemm<double>(batch, q, q, q, qq, L1(q, q), L1(q, 1), qq, L1(q, 1), L1(q, q), qq,
@@ -704,7 +704,9 @@ static int svd_right(qtt_ctx* c, const cplx<R>* in, MIdx inB, MIdx rowI, MIdx co
 // got = min(rows, cols)), then one-sided Jacobi on R^H (rows x got), whose
 // normalised rotated columns are the left singular vectors of C (no rotation
 // accumulation).  U: rows x got, row-major (leading dimension got), columns
-// by decreasing singular value; sigma: got values; *nsv = got.  `sampling`
+// by decreasing singular value; sigma: got values; *nsv = got.  The caller
+// truncates at a tail of `cut`, if that is not negative: values that are
+// rounding noise may then come as one value and zeros.  `sampling`
 // (TT-cross) keeps the one-CTA QR kernels: the samples of a 0/1 geometry have
 // many equal singular values, so the pivots, and with them what a run of the
 // cross finds, hang on the rounding of the factorisation (on the 64^3 sphere
@@ -712,13 +714,13 @@ static int svd_right(qtt_ctx* c, const cplx<R>* in, MIdx inB, MIdx rowI, MIdx co
 // 113, the one-CTA kernels' 1).
 template <class R>
 int left_svd(qtt_ctx* c, const cplx<R>* Cm, int64_t rows, int64_t cols, int64_t ld, cplx<R>* U, R* sigma,
-             int64_t* nsv, bool sampling) {
+             int64_t* nsv, bool sampling, double cut) {
   const int64_t p = std::min(rows, cols);
   if (!sampling && svd_right_fits<R>(cols, rows, 1, L1(cols, 1))) {
     // right vectors of C^H; U is the adjoint of what svd_right returns
     DBuf Vh;
     TRY(Vh.alloc(c, (size_t)p * rows * sizeof(cplx<R>)));
-    TRY(svd_right<R>(c, Cm, B0(), L1(cols, 1), L1(rows, ld), 1, cols, rows, 1, Vh.as<cplx<R>>(), sigma, nullptr, 0.0,
+    TRY(svd_right<R>(c, Cm, B0(), L1(cols, 1), L1(rows, ld), 1, cols, rows, 1, Vh.as<cplx<R>>(), sigma, nullptr, cut,
                      nullptr, 0, 0));
     c->launches++;
     TRY(qtt_copy_strided<R>(Vh.as<cplx<R>>(), L1(rows, 1), L1(p, rows), rows, p, 1, U, p, c->stream));
@@ -1602,7 +1604,7 @@ int tt_svd_dev(qtt_ctx* c, int d, const std::vector<int>& modes, const cplx<R>* 
     TRY(U.alloc(c, (size_t)m * m * sizeof(cplx<R>)));
     TRY(sig.alloc(c, (size_t)m * sizeof(R)));
     int64_t nsv = 0;
-    TRY(left_svd<R>(c, C, m, rest, rest, U.as<cplx<R>>(), sig.as<R>(), &nsv));
+    TRY(left_svd<R>(c, C, m, rest, rest, U.as<cplx<R>>(), sig.as<R>(), &nsv, false, delta));
     c->launches++;
     TRY(qtt_trunc_rank<R>(sig.as<R>(), (int)nsv, delta, max_rank, dint, dscal + 1, c->stream));
     int hv[2];
@@ -1636,8 +1638,8 @@ int tt_svd_dev(qtt_ctx* c, int d, const std::vector<int>& modes, const cplx<R>* 
 
 template int tt_svd_dev<double>(qtt_ctx*, int, const std::vector<int>&, const zc*, double, int, qtt_dtype, qtt_tt**);
 template int tt_svd_dev<float>(qtt_ctx*, int, const std::vector<int>&, const cc*, double, int, qtt_dtype, qtt_tt**);
-template int left_svd<double>(qtt_ctx*, const zc*, int64_t, int64_t, int64_t, zc*, double*, int64_t*, bool);
-template int left_svd<float>(qtt_ctx*, const cc*, int64_t, int64_t, int64_t, cc*, float*, int64_t*, bool);
+template int left_svd<double>(qtt_ctx*, const zc*, int64_t, int64_t, int64_t, zc*, double*, int64_t*, bool, double);
+template int left_svd<float>(qtt_ctx*, const cc*, int64_t, int64_t, int64_t, cc*, float*, int64_t*, bool, double);
 
 // ----------------------------------------------------------- inner product
 template <class R>

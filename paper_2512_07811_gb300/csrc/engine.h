@@ -251,7 +251,7 @@ int amen_mv_dev(qtt_ctx* c, const qtt_mpo* A, const qtt_tt* x, const qtt_tt* y0,
 // (leading dimension ld); *nsv = min(rows, cols).
 template <class R>
 int left_svd(qtt_ctx* c, const cplx<R>* Cm, int64_t rows, int64_t cols, int64_t ld, cplx<R>* U, R* sigma,
-             int64_t* nsv, bool sampling = false);
+             int64_t* nsv, bool sampling = false, double cut = -1.0);
 
 template <class T>
 inline T* core_ptr(const qtt_tt* x, int k) {

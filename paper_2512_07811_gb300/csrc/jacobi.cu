@@ -635,7 +635,8 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
   }
   __syncthreads();
   if (a.sigma && rank == 0)
-    for (int i = threadIdx.x; i < q; i += nthr) a.sigma[bt * q + i] = sorted[i];
+    for (int i = threadIdx.x; i < q; i += nthr)  // (the dropped columns' norm as one value)
+      a.sigma[bt * q + i] = i < qa ? sorted[i] : i == qa ? (R)(sqrt(scan[0]) * jac_pow2(0.0, esc)) : R(0);
   int keep = qa;
   if (a.trunc) {
     // smallest t >= 1 with sqrt(sum_{j >= t} s_j^2) <= delta, sums in double
@@ -831,7 +832,7 @@ int qtt_svd(const cplx<R>* G, const int* perm, cplx<R>* Vh, R* sigma, int* trunc
             int max_rank, int mask, int p, int q, int batch, int max_sweeps, int* sweeps, cudaStream_t s) {
   JacPlan pl;
   if (!jac_plan<R>(p, q, batch, &pl)) return QTT_ERR_UNSUPPORTED;
-  if (trunc && !sigma) jac_adapt<R>(&pl, q, false);
+  if (deltas || delta >= 0) jac_adapt<R>(&pl, q, false);
   const JacArgs<R> a{G, perm,  Vh,     sigma,    trunc,      delta,  deltas,  max_rank, mask,
                      p, q,     pl.bs,  pl.bsx,   pl.adapt,   max_sweeps, sweeps, nullptr, nullptr};
 #define QTT_J(LP, RPL) \
@@ -857,11 +858,11 @@ bool qtt_svd_pre_fits(int p, int q, int batch) {
   return 4.5 * pd.cost > 7.0 * pf.cost + 1.5e5;
 }
 
-int qtt_svd_pre(const zc* G, zc* Vt, bool trunc, double delta, const double* deltas, int p, int q, int batch,
+int qtt_svd_pre(const zc* G, zc* Vt, double delta, const double* deltas, int p, int q, int batch,
                 int* sweeps, cudaStream_t s) {
   JacPlan pl;
   if (p < q || !jac_plan<float>(p, q, batch, &pl, true)) return QTT_ERR_UNSUPPORTED;
-  if (trunc) jac_adapt<float>(&pl, q, true);
+  if (deltas || delta >= 0) jac_adapt<float>(&pl, q, true);
   const JacArgs<float> a{nullptr, nullptr, nullptr, nullptr, nullptr,  delta, deltas, 0, 0,
                          p,       q,       pl.bs,   pl.bsx,  pl.adapt, 30,    sweeps, G, Vt};
 #define QTT_J(RPL) \

@@ -40,7 +40,9 @@ int qtt_qr_cluster(const cplx<R>* in, MIdx inB, MIdx rowI, MIdx colI, int conj_i
 // p*q apart), conjugated, one per row of Vh (q x p) by decreasing singular value, component i of G's rows at perm[i]
 // (p per matrix; null: i).  sigma (q, or null); trunc (4 ints per matrix, or null): the rank that the tail threshold
 // delta (deltas[b] if not null) and max_rank (0: no cap) keep, 1 if the cap cut it, the discarded tail as a double;
-// mask: rows of Vh from that rank on are zeroed.  QTT_ERR_UNSUPPORTED where qtt_svd_fits is false.
+// mask: rows of Vh from that rank on are zeroed.  Where delta is not negative the caller truncates at that tail, and
+// trailing columns of rounding noise may be left out: their rows of Vh are zero, and sigma holds their norm as one value
+// and zeros.  QTT_ERR_UNSUPPORTED where qtt_svd_fits is false.
 template <class R>
 bool qtt_svd_fits(int p, int q, int batch);
 template <class R>
@@ -49,8 +51,8 @@ int qtt_svd(const cplx<R>* G, const int* perm, cplx<R>* Vh, R* sigma, int* trunc
 // Column rotations of an FP64 matrix computed in FP32: V with the columns of G V orthogonal to about 1e-6, V itself
 // unitary to FP32 rounding.  Vt (3 batch q^2 elements): V transposed, then two identity matrices per matrix.
 bool qtt_svd_pre_fits(int p, int q, int batch);  // where that and the FP64 products are cheaper than the sweeps saved
-// (trunc: the vectors are truncated at delta, deltas[b] if not null, as by qtt_svd)
-int qtt_svd_pre(const zc* G, zc* Vt, bool trunc, double delta, const double* deltas, int p, int q, int batch,
+// (delta, deltas as in qtt_svd)
+int qtt_svd_pre(const zc* G, zc* Vt, double delta, const double* deltas, int p, int q, int batch,
                 int* sweeps, cudaStream_t s);
 // whether qtt_qr_cluster takes the shape with sorted columns
 template <class R>
@@ -88,8 +90,6 @@ template <class R>
 int qtt_scale(cplx<R>* x, int64_t count, cplx<R> scale, cudaStream_t s);
 template <class R>
 int qtt_sumsq(const cplx<R>* x, int64_t count, double* out, cudaStream_t s);
-int qtt_convert_z2c(const zc* in, cc* out, int64_t count, cudaStream_t s);
-int qtt_convert_c2z(const cc* in, zc* out, int64_t count, cudaStream_t s);
 template <class R>
 int qtt_copy_strided(const cplx<R>* in, MIdx rows, MIdx cols, int64_t nrows, int64_t ncols, int conj_in,
                      cplx<R>* out, int64_t ldo, cudaStream_t s);

@@ -94,3 +94,31 @@ def test_batch_with_a_rank_per_train(Q, ctx, p, q, fp32):
         a, b = [c.astype(np.complex128) for c in y.cores()]
         ref = x[0][0] @ x[1][:, :, 0]
         assert np.linalg.norm(a[0] @ b[:, :, 0] - ref) <= (1e-6 if fp32 else 1e-12) + 40 * tol * u * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("m,n", [(23, 40), (30, 24), (64, 64), (100, 130), (130, 70)])
+@pytest.mark.parametrize("kind", ["graded", "noise", "deficient"])
+def test_svd_of_a_dense_matrix(Q, ctx, m, n, kind):
+    """TT-SVD of an m x n array: left vectors and the values they are cut by."""
+    torch = pytest.importorskip("torch")
+    rng = np.random.default_rng(m * 1000 + n + 2)
+    q = min(m, n)
+    s, eps, rank = _spectrum(kind, q, False)
+    A = _unitary(rng, m, q) * s @ _unitary(rng, n, q).conj().T
+    d = torch.tensor(A, device="cuda")
+    y = Q.tt_from_dense(ctx, d.data_ptr(), [m, n], eps)
+    assert y.ranks[1] == rank
+    a, b = y.cores()
+    tol = math.sqrt(m + n) * 2.0 ** -53
+    assert abs(a[0].conj().T @ a[0] - np.eye(rank)).max() <= 20 * tol
+    assert np.linalg.norm(a[0] @ b[:, :, 0] - A) <= np.linalg.norm(s[rank:]) + 40 * tol * np.linalg.norm(s)
+
+
+def test_zero_tolerance(Q, ctx):
+    """No noise is left out at a zero tolerance."""
+    rng = np.random.default_rng(5)
+    s = np.zeros(60)
+    s[:20] = np.logspace(0, -3, 20)
+    x = [(_unitary(rng, 60, 60) * s)[None], _unitary(rng, 80, 60).conj().T[:, :, None]]
+    y, info = Q.tt_round(ctx, Q.TT.from_cores(ctx, x, Q.C128), 0.0)
+    assert y.ranks[1] >= 20 and info.tail == 0.0
