@@ -1873,6 +1873,7 @@ static int sketch_core(qtt_ctx* c, int T, const qtt_complex* coef, const qtt_mpo
       // U2[a1, g0, j, l0] = sum_{i, g1} D[g0, i, j, g1] U1[g1, a1, i, l0]   (batch a1)
       if (!A[t]->ident[k]) TRY(U2.alloc(c, (size_t)a1 * g0 * ni * l0 * sizeof(C)));
       if (A[t]->ident[k]) {
+        if (a1 * ni > 65535) return QTT_ERR_ARG;  // the sizes that an operator's core takes
         U2 = std::move(U1);  // g0 = g1 = 1, j = i: the same array
       } else if (A[t]->diag[k] && ni == no) {
         // diagonal core (D[g0, i, j, g1] = 0 for i != j): batch (a1, i),
@@ -1975,6 +1976,7 @@ static int sketch_core(qtt_ctx* c, int T, const qtt_complex* coef, const qtt_mpo
       const int64_t g0 = A[t]->g[k], g1 = A[t]->g[k + 1], ni = A[t]->ni[k];
       const int64_t a0 = xs[t]->r[k], a1 = xs[t]->r[k + 1];
       if (A[t]->ident[k]) {
+        if (lk * no > 65535) return QTT_ERR_ARG;
         // Y[l, j, off' + a1] = sum_a0 M[l, off + a0] X[a0, j, a1], straight into its place
         GemmDesc g;
         g.bA = g.bB = g.bC = B0();
