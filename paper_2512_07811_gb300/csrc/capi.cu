@@ -1742,32 +1742,75 @@ int ms_solve(qtt_ctx* c, const qtt_rve* rve, const double* C1h, const double* C2
 template <class R>
 static int tt_full_dev(qtt_ctx* c, const qtt_tt* x, DBuf* out) {
   typedef cplx<R> C;
-  int64_t P = x->n[0];
-  DBuf V;
-  TRY(V.alloc(c, (size_t)P * x->r[1] * sizeof(C)));
-  if (cudaMemcpyAsync(V.p, core_ptr<const C>(x, 0), (size_t)P * x->r[1] * sizeof(C), cudaMemcpyDeviceToDevice,
-                      c->stream) != cudaSuccess)
-    return QTT_ERR_CUDA;
-  for (int k = 1; k < x->d; ++k) {
-    const int64_t rk = x->r[k], nk = x->n[k], r1 = x->r[k + 1];
+  const int d = x->d;
+  // The first and the last cores, as far as their products are small, are
+  // multiplied up by one launch; the last bond then has up to 32 values (8 in
+  // FP64), which also replaces the contractions of 2, 4, 8 columns by one (us for
+  // 20 sites complex64: 250 / 60).
+  constexpr int64_t cap = QTT_ENDS / sizeof(R), last = sizeof(R) == 8 ? 8 : 32;
+  int a = 0, b = d;  // cores 0 .. a-1 and b .. d-1
+  {
+    int64_t w = 1, big = 0;
+    for (int k = 0; k < d; ++k) {  // (the largest sizes that one contraction per core takes)
+      if (k > 0) {
+        const int64_t N = (int64_t)x->n[k] * x->r[k + 1], edge = w <= 32 || N <= 32 ? 32 : 64;
+        big = std::max(big, (w + edge - 1) / edge);
+      }
+      w *= x->n[k];
+    }
+    if (big > 65535) return QTT_ERR_ARG;
+    w = 1;
+    while (a < d - 1 && a < 16 && w * x->n[a] * x->r[a + 1] <= cap) w *= x->n[a++];
+    w = 1;
+    while (b > a && b > 1 && d - b < 16 && w * x->n[b - 1] * x->r[b - 1] <= cap && x->r[b - 1] <= last) w *= x->n[--b];
+  }
+  if (a == 0) a = 1, b = d;  // (a first core beyond the cap: core by core)
+  int64_t P = 1, S = 1;
+  for (int k = 0; k < a; ++k) P *= x->n[k];
+  for (int k = b; k < d; ++k) S *= x->n[k];
+  DBuf V, Sd;
+  TRY(V.alloc(c, (size_t)P * x->r[a] * sizeof(C)));
+  if (a == 1 && b == d) {
+    if (cudaMemcpyAsync(V.p, core_ptr<const C>(x, 0), (size_t)P * x->r[1] * sizeof(C), cudaMemcpyDeviceToDevice,
+                        c->stream) != cudaSuccess)
+      return QTT_ERR_CUDA;
+  } else {
+    EndsTable t{};
+    t.n[0] = a;
+    t.n[1] = d - b;
+    for (int k = 0; k < d; ++k) {
+      if (k >= a && k < b) continue;
+      const int e = k < a ? 0 : 1, f = e ? k - b : k;
+      t.core[e][f] = core_ptr<const C>(x, k);
+      t.r0[e][f] = x->r[k];
+      t.m[e][f] = x->n[k];
+      t.r1[e][f] = x->r[k + 1];
+    }
+    if (b < d) TRY(Sd.alloc(c, (size_t)S * x->r[b] * sizeof(C)));
+    c->launches++;
+    TRY(qtt_train_ends<R>(t, V.as<C>(), Sd.as<C>(), c->stream));
+  }
+  for (int k = a; k <= b && k < d; ++k) {
+    const bool join = k == b;  // the last cores' product
+    const int64_t rk = x->r[k], N = join ? S : (int64_t)x->n[k] * x->r[k + 1];
     DBuf W;
-    TRY(W.alloc(c, (size_t)P * nk * r1 * sizeof(C)));
+    TRY(W.alloc(c, (size_t)P * N * sizeof(C)));
     GemmDesc g;
     g.bA = g.bB = g.bC = MIdx{1, 1, 0, 0};
     g.M = P;
-    g.N = nk * r1;
+    g.N = N;
     g.K = rk;
     g.batch = 1;
     g.mA = MIdx{P, 1, rk, 0};
     g.kA = MIdx{rk, 1, 1, 0};
-    g.kB = MIdx{rk, 1, nk * r1, 0};
-    g.nB = MIdx{nk * r1, 1, 1, 0};
-    g.mC = MIdx{P, 1, nk * r1, 0};
-    g.nC = MIdx{nk * r1, 1, 1, 0};
+    g.kB = MIdx{rk, 1, N, 0};
+    g.nB = MIdx{N, 1, 1, 0};
+    g.mC = MIdx{P, 1, N, 0};
+    g.nC = MIdx{N, 1, 1, 0};
     g.conjA = g.conjB = 0;
-    TRY(gemm_ab<R>(c, g, C(1, 0), C(0, 0), V.as<C>(), core_ptr<const C>(x, k), W.as<C>()));
+    TRY(gemm_ab<R>(c, g, C(1, 0), C(0, 0), V.as<C>(), join ? Sd.as<const C>() : core_ptr<const C>(x, k), W.as<C>()));
     V = std::move(W);
-    P *= nk;
+    P *= join ? S : x->n[k];
   }
   *out = std::move(V);
   return QTT_OK;

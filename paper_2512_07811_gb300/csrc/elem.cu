@@ -117,6 +117,47 @@ __global__ void sumsq_kernel(const cplx<R>* __restrict__ x, int64_t count, doubl
   }
 }
 
+// The first or the last cores of a train multiplied up in shared memory, one CTA
+// per end: their contractions are of a few values each and cost a launch (4 us)
+// apiece on their own.
+template <class R>
+__global__ void __launch_bounds__(256) train_ends_kernel(const __grid_constant__ EndsTable t, cplx<R>* __restrict__ P,
+                                                         cplx<R>* __restrict__ S) {
+  typedef cplx<R> C;
+  constexpr int CAP = QTT_ENDS / sizeof(R);
+  __shared__ C buf[2][CAP];
+  const int e = blockIdx.x, nc = t.n[e];
+  if (nc == 0) return;
+  C* out = e == 0 ? P : S;
+  int f = e == 0 ? 0 : nc - 1, cur = 0;
+  int w = e == 0 ? t.m[0][0] : t.m[1][f];  // values of the modes so far
+  const C* c0 = static_cast<const C*>(t.core[e][f]);
+  for (int i = threadIdx.x; i < t.r0[e][f] * t.m[e][f] * t.r1[e][f]; i += 256) buf[0][i] = c0[i];
+  __syncthreads();
+  for (int k = 1; k < nc; ++k) {
+    f = e == 0 ? k : nc - 1 - k;
+    const C* core = static_cast<const C*>(t.core[e][f]);
+    const int r0 = t.r0[e][f], m = t.m[e][f], r1 = t.r1[e][f];
+    const C* x = buf[cur];
+    C* y = buf[cur ^ 1];
+    // (w x r0)(r0 x m r1), or (r0 m x r1)(r1 x w)
+    const int rows = e == 0 ? w : r0 * m, cols = e == 0 ? m * r1 : w, kk = e == 0 ? r0 : r1;
+    const C* A = e == 0 ? x : core;
+    const C* B = e == 0 ? core : x;
+    for (int i = threadIdx.x; i < rows * cols; i += 256) {
+      const int a = i / cols, b = i - a * cols;
+      C v(0, 0);
+      for (int l = 0; l < kk; ++l) cfma(v, A[a * kk + l], B[l * cols + b]);
+      y[i] = v;
+    }
+    w *= m;
+    cur ^= 1;
+    __syncthreads();
+  }
+  const int total = w * (e == 0 ? t.r1[0][nc - 1] : t.r0[1][0]);
+  for (int i = threadIdx.x; i < total; i += 256) out[i] = buf[cur][i];
+}
+
 template <class R>
 __global__ void copy_strided_kernel(const cplx<R>* __restrict__ in, MIdx rows, MIdx cols, int64_t nrows,
                                     int64_t ncols, int conj_in, cplx<R>* __restrict__ out, int64_t ldo) {
@@ -517,6 +558,13 @@ int qtt_sumsq(const cplx<R>* x, int64_t count, double* out, cudaStream_t s) {
   sumsq_kernel<R><<<1, 1024, 0, s>>>(x, count, out);
   CHECK_LAUNCH();
 }
+template <class R>
+int qtt_train_ends(const EndsTable& t, cplx<R>* P, cplx<R>* S, cudaStream_t s) {
+  train_ends_kernel<R><<<2, 256, 0, s>>>(t, P, S);
+  CHECK_LAUNCH();
+}
+template int qtt_train_ends<double>(const EndsTable&, zc*, zc*, cudaStream_t);
+template int qtt_train_ends<float>(const EndsTable&, cc*, cc*, cudaStream_t);
 template <class R>
 int qtt_copy_strided(const cplx<R>* in, MIdx rows, MIdx cols, int64_t nrows, int64_t ncols, int conj_in,
                      cplx<R>* out, int64_t ldo, cudaStream_t s) {

@@ -109,6 +109,16 @@ struct CoreTable {
 };
 // what: 0 copy (elem bytes each, 8 or 16), 1 complex128 -> complex64, 2 complex64 -> complex128
 int qtt_cores_move(const CoreTable& t, int what, int elem, cudaStream_t s);
+// Products of a train's first cores (p x r row-major to P) and of its last ones (r x q to S), each partial product at
+// most QTT_ENDS / sizeof(R) elements: one CTA each
+#define QTT_ENDS 4096
+struct EndsTable {
+  int n[2];                 // cores of either end, at most 16
+  const void* core[2][16];  // in train order
+  int r0[2][16], m[2][16], r1[2][16];
+};
+template <class R>
+int qtt_train_ends(const EndsTable& t, cplx<R>* P, cplx<R>* S, cudaStream_t s);
 // *flag = 1 if an element of the src cores is not finite
 template <class R>
 int qtt_cores_isfinite(const CoreTable& t, int* flag, cudaStream_t s);

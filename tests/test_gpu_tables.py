@@ -77,3 +77,28 @@ def test_kept_blocks_are_bounded_and_given_back(Q):
     ctx.close()
     torch.cuda.synchronize()
     assert torch.cuda.mem_get_info()[0] >= free0 - (64 << 20)
+
+
+@pytest.mark.parametrize("d,r,ctrl", [(1, 1, 0), (1, 2, 3), (2, 2, 0), (3, 40, 0), (5, 3, 6), (6, 33, 0), (9, 8, 1), (12, 9, 0),
+                                      (14, 32, 0), (11, 40, 6), (4, 600, 0), (13, 1, 0)])
+@pytest.mark.parametrize("fp32", [False, True])
+def test_read_out_of_a_whole_train(Q, ctx, d, r, ctrl, fp32):
+    """Every entry of a train of d bits along one axis: the first and last cores
+    are multiplied up on their own, up to bonds of 8 or 32 values."""
+    rng = np.random.default_rng(d * 100 + r)
+    modes = ([ctrl] if ctrl else []) + [2] * d
+    rk = [1] + [r] * (len(modes) - 1) + [1]
+    x = [rng.standard_normal((rk[k], n, rk[k + 1])) + 1j * rng.standard_normal((rk[k], n, rk[k + 1]))
+         for k, n in enumerate(modes)]
+    x = [a / np.linalg.norm(a) * r ** 0.5 for a in x]
+    if fp32:
+        x = [a.astype(np.complex64) for a in x]
+    v = Q.contract_voxels(ctx, Q.TT.from_cores(ctx, x, Q.C64 if fp32 else Q.C128), [d, 0, 0])
+    full = np.ones((1, 1), dtype=np.complex128)
+    for a in x:
+        full = (full @ a.astype(np.complex128).reshape(a.shape[0], -1)).reshape(-1, a.shape[2])
+    u = 2.0 ** -24 if fp32 else 2.0 ** -53
+    err = np.linalg.norm(v.reshape(-1) - full[:, 0])
+    # sums of r products per core, relative to the product of the cores' norms (largest singular value times sqrt(r))
+    scale = np.prod([np.linalg.norm(a.astype(np.complex128)) / (r ** 0.5 if k else 1) for k, a in enumerate(x)])
+    assert err <= 20 * len(modes) * max(r, 2) ** 0.5 * u * max(np.linalg.norm(full), scale)
