@@ -54,8 +54,8 @@ E2E_OP_TOL = 1e-6   # the float path's operators in float (ms_setup)
 # dominant kernel class, from the one-kernel ncu captures summarised in
 # profiles/ (file named in the line); None where no current capture exists.
 TRAFFIC = {
-    "jacobi_block_kernel": {"bytes": 316.16e3, "profile": "profiles/jacobi_block_kernel_sphere32.md"},
-    "qr_blocked_kernel": {"bytes": None, "profile": None},
+    "jacobi_cluster2_kernel": {"bytes": 368.64e3, "profile": "profiles/jacobi_cluster2_kernel_sphere32.md"},
+    "qr_cluster_kernel": {"bytes": 372.48e3, "profile": "profiles/qr_cluster_kernel_sphere32.md"},
     "gemm_midx_kernel": {"bytes": 554.496e3, "profile": "profiles/gemm_midx_kernel_sphere32.md"},
 }
 
@@ -647,7 +647,7 @@ def run_ours(args, world, local_rank):
                 green_rank=green_rank, phase_rank=phase_rank, setup_ms=setup_ms)
 
 
-SMS_USED = {"gemm": None, "qr": 1, "jacobi": 8}
+SMS_USED = {"gemm": None, "qr": 16, "jacobi": 10}
 
 
 def roofline(prof, repp, peaks, mpeaks):
@@ -655,11 +655,11 @@ def roofline(prof, repp, peaks, mpeaks):
     (CUDA events around each launch, load cases one after another so that no
     launch shares the GPU with another solve's).  achieved = the class's
     model flops / summed duration, against the measured FP32 FMA peak of the
-    whole GPU and of the SMs one launch occupies (one CTA per QR, one 8-CTA
-    cluster per Jacobi SVD)."""
+    whole GPU and of the SMs one launch occupies (one cluster per matrix: 16
+    CTAs for the 272 x 136 QR, 10 for the 256 x 136 Jacobi SVD)."""
     dom = max(["gemm", "qr", "jacobi"], key=lambda k: prof[k]["ms"])
     p = prof[dom]
-    kernel = {"gemm": "gemm_midx_kernel", "qr": "qr_blocked_kernel", "jacobi": "jacobi_block_kernel"}[dom]
+    kernel = {"gemm": "gemm_midx_kernel", "qr": "qr_cluster_kernel", "jacobi": "jacobi_cluster2_kernel"}[dom]
     roof = {"bound": "alu", "kernel": kernel, "unit": "TFLOP/s",
             "achieved": p["flops"] / (p["ms"] * 1e-3) / 1e12 if p["ms"] else 0.0,
             "peak": peaks["fp32_tflops"],

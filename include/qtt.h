@@ -116,8 +116,8 @@ QTT_API int qtt_ctx_profile_read(qtt_ctx* ctx, int kclass, double* total_ms, int
  * to `max_rows` rows of 8 doubles to `rows` (host, caller-owned, 8 *
  * max_rows), by decreasing total time: d0, d1, d2, batch, variant, launches,
  * total ms, model flops -- GEMM: M, N, K, batch and variant = tile edge x 100
- * + split-K count (tile edge 128: the tensor-core kernel, + its TF32
- * passes); QR: m, n, 0, batch, variant 1 when the explicit Q was formed;
+ * + split-K count (the FP32 tile's edge, the FP64 kernel has smaller ones;
+ * tile edge 128: the tensor-core kernel, + its TF32 passes); QR: m, n, 0, batch, variant 1 when the explicit Q was formed;
  * Jacobi: rows p, columns q, 0, batch, 0.  *n_rows = the number of distinct
  * shapes (may exceed max_rows).  Synchronises the stream.  QTT_ERR_ARG on a
  * bad class or null pointers. */

@@ -621,7 +621,8 @@ static GemmDesc bgemm(int64_t B, int64_t M, int64_t N, int64_t K, int64_t bA, MI
 // C P.  The sort is what pays: R^H then has its large columns first and is
 // close to diagonal already, and Jacobi takes 6-7 sweeps where C^H itself, or
 // an unsorted R^H, takes 14-21 (rounding matrices of 64 to 128 columns with
-// singular values over six decades).  Vh: min(m, n) x n per matrix, rows by
+// singular values over six decades).  FP64: most sweeps are done in FP32 first
+// (qtt_svd_pre), V made unitary by two Newton-Schulz steps.  Vh: min(m, n) x n per matrix, rows by
 // decreasing singular value; trunc, delta(s), max_rank, mask as in qtt_svd.
 // fits: whether the two cluster kernels take the shape (m beyond 512 rows is
 // first reduced by a TSQR, single matrices only).
@@ -1217,8 +1218,8 @@ template int round_det<float>(qtt_ctx*, const qtt_tt*, double, int, const int*, 
 // ------------------------------------------------ batched deterministic round
 // B trains of one shape (same modes and ranks) rounded in lockstep by the
 // algorithm of round_det: every step of either sweep is one launch per kernel
-// for the whole batch -- batched GEMMs, one QR CTA per train, one Jacobi
-// cluster per train -- and the truncation sweep needs one host
+// for the whole batch -- batched GEMMs, one QR and one Jacobi cluster per
+// train -- and the truncation sweep needs one host
 // synchronisation per core for all trains.  Each train keeps its own
 // truncation: a bond is carried at the largest rank of the batch, the
 // singular vectors beyond a train's own rank are zeroed, so that its padded
