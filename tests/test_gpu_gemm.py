@@ -42,3 +42,18 @@ def test_dot_of_two_core_trains(Q, ctx, r, s, n, fp32):
     scale = math.prod(float(np.linalg.norm(c.astype(np.complex128))) for c in x + y)
     u = 2.0 ** -24 if fp32 else 2.0 ** -53
     assert abs(v - np.vdot(full[0], full[1])) <= 20 * math.sqrt(r + s + n) * u * scale
+
+
+@pytest.mark.parametrize("K", [8, 40, 256, 1000, 4096])
+@pytest.mark.parametrize("value", [0.7, 1.1])
+def test_long_sums_of_one_sign(Q, ctx, K, value):
+    """A sum of K equal values, whose roundings all go the same way: runs of 8 and the sum of the runs
+    round by at most (8 + K / 8) u; one chain is off by 41, 167, 680 u at K = 256, 1000, 4096."""
+    import torch
+    M, N = 70, 66
+    a = torch.full((M, K), value, dtype=torch.complex64, device="cuda")
+    b = torch.ones(K, N, dtype=torch.complex64, device="cuda")
+    c = torch.empty(M, N, dtype=torch.complex64, device="cuda")
+    Q.qtt_cgemm(ctx, M, N, K, a.data_ptr(), b.data_ptr(), c.data_ptr(), engine=0)
+    ref = K * float(np.float32(value))
+    assert float((c.to(torch.complex128) - ref).abs().max()) <= (8 + K / 8) * 2.0 ** -24 * ref
