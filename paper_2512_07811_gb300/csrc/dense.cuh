@@ -63,5 +63,32 @@ __device__ __forceinline__ void add_comp(R& hi, R& lo, R t) {
   lo += (hi - (s - bb)) + (t - bb);
   hi = s;
 }
+// the lanes' compensated sums added up, in every lane
+template <class R>
+__device__ __forceinline__ void wsum_comp(R& hi, R& lo) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const R ohi = __shfl_xor_sync(0xffffffffu, hi, o), olo = __shfl_xor_sync(0xffffffffu, lo, o);
+    lo += olo;
+    add_comp(hi, lo, ohi);
+  }
+}
+
+// Brings a vector whose norm is 1 to single precision (entries on the lanes, N each)
+// to the norm 1 that its stored entries allow: x += x (1 - |x|^2) / 2.  The sum of
+// squares is compensated.  A rounding's vectors and reflections are used as
+// exactly orthonormal, bond after bond, and a norm that is off scales
+// everything: left as the factorisations leave them (1e-7) they were half of
+// what a complex64 solve's error owed to them.
+template <int N>
+__device__ __forceinline__ void unit_norm(cplx<float> (&x)[N]) {
+  float hi = 0, lo = 0;
+#pragma unroll
+  for (int u = 0; u < N; ++u) add_comp(hi, lo, abs2(x[u]));
+  wsum_comp(hi, lo);
+  const float k = -0.5f * ((hi - 1.0f) + lo);
+#pragma unroll
+  for (int u = 0; u < N; ++u) x[u] = cplx<float>(fmaf(x[u].re, k, x[u].re), fmaf(x[u].im, k, x[u].im));
+}
 
 }  // namespace dense

@@ -696,14 +696,17 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
     const R v = h == 0 ? nx : ny;
     R f = v > Lim<R>::tiny * R(4) ? R(1) / v : R(0);
     if (a.mask && rk >= keep) f = 0;
+    C o[RPL];
+#pragma unroll
+    for (int u = 0; u < RPL; ++u) {
+      const C g = h == 0 ? x[u] : y[u];
+      o[u] = f == R(0) ? C(0, 0) : C(g.re * f, -g.im * f);
+    }
+    if constexpr (sizeof(R) == 4) dense::unit_norm(o);
 #pragma unroll
     for (int u = 0; u < RPL; ++u) {
       const int i = gl + LP * u;
-      if (i >= p) continue;
-      const C g = h == 0 ? x[u] : y[u];
-      C o(g.re * f, -g.im * f);
-      if (f == R(0)) o = C(0, 0);
-      Vh[(int64_t)rk * p + (perm ? perm[i] : i)] = o;
+      if (i < p) Vh[(int64_t)rk * p + (perm ? perm[i] : i)] = o[u];
     }
   }
   for (int e = rank * nthr + threadIdx.x; e < (q - qa) * p; e += NC * nthr) Vh[(int64_t)qa * p + e] = C(0, 0);

@@ -147,12 +147,7 @@ __device__ __forceinline__ R reflector_scalars(cplx<R> (&x)[RPL], int j, R zero2
   if constexpr (sizeof(R) == 4) {
     lo += lo1;
     dense::add_comp(hi, lo, hi1);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const R ohi = __shfl_xor_sync(0xffffffffu, hi, o), olo = __shfl_xor_sync(0xffffffffu, lo, o);
-      lo += olo;
-      dense::add_comp(hi, lo, ohi);
-    }
+    dense::wsum_comp(hi, lo);
     hi += lo;
   } else {
     hi = dense::wsum(hi + hi1);
@@ -462,6 +457,7 @@ qr_cluster_kernel(const __grid_constant__ QrArgs<R> a) {
         }
     }
     if (c < kmax) {
+      if constexpr (sizeof(R) == 4) dense::unit_norm(x);
 #pragma unroll
       for (int u = 0; u < RPL; ++u) {
         const int i = lane + 32 * u;

@@ -122,3 +122,29 @@ def test_zero_tolerance(Q, ctx):
     x = [(_unitary(rng, 60, 60) * s)[None], _unitary(rng, 80, 60).conj().T[:, :, None]]
     y, info = Q.tt_round(ctx, Q.TT.from_cores(ctx, x, Q.C128), 0.0)
     assert y.ranks[1] >= 20 and info.tail == 0.0
+
+
+@pytest.mark.parametrize("sketched", [False, True])
+def test_norms_of_rounded_cores_fp32(Q, ctx, sketched):
+    """Cores 2..d of a complex64 rounding have rows of norm 1 to what storing their entries allows.  What storing
+    leaves is taken from the rows themselves (normalised in FP64, rounded); forming the sum of squares adds the
+    rounding of each square, 0.5 u rms where one entry makes up the row, independent of it."""
+    rng = np.random.default_rng(5)
+    r = [1] + [min(40, 2 ** k, 2 ** (14 - k)) for k in range(1, 14)] + [1]
+    x = [rng.standard_normal((r[k], 2, r[k + 1])) + 1j * rng.standard_normal((r[k], 2, r[k + 1])) for k in range(14)]
+    x = Q.TT.from_cores(ctx, [(c / np.linalg.norm(c)).astype(np.complex64) for c in x], Q.C64)
+    if sketched:
+        w = [1] + [min(48, 2 ** k, 2 ** (14 - k)) for k in range(1, 14)] + [1]
+        S = Q.TT.from_cores(ctx, [rng.standard_normal((w[k], 2, w[k + 1])).astype(np.complex64) for k in range(14)],
+                            Q.C64)
+        y, _ = Q.tt_round_sketched(ctx, [(1.0, None, x)], S, 1e-6)
+    else:
+        y, _ = Q.tt_round(ctx, x, 1e-6)
+    norm2 = lambda m: (abs(m.astype(np.complex128)) ** 2).sum(1) - 1  # noqa: E731
+    off, stored = [], []
+    for c in y.cores()[1:]:
+        m = c.astype(np.complex128).reshape(c.shape[0], -1)
+        off.append(norm2(m))
+        stored.append(norm2((m / np.linalg.norm(m, axis=1, keepdims=True)).astype(np.complex64)))
+    rms = lambda v: math.sqrt((np.concatenate(v) ** 2).mean())  # noqa: E731
+    assert rms(off) <= math.hypot(rms(stored), 0.5 * 2.0 ** -24)
