@@ -172,6 +172,20 @@ __global__ void copy_strided_kernel(const cplx<R>* __restrict__ in, MIdx rows, M
 }
 
 // x[i, :] *= sv[i]  (or /= sv[i] when invert; rows with sv[i] == 0 are zeroed)
+// U += D diag(1 / sv): rows of ldu and ldd elements
+template <class R>
+__global__ void add_scaled_cols_kernel(cplx<R>* __restrict__ U, int64_t ldu, const cplx<R>* __restrict__ D, int64_t ldd,
+                                       int64_t rows, int64_t cols, const R* __restrict__ sv) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < rows * cols;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = e / cols, j = e - i * cols;
+    const R f = R(1) / sv[j];
+    cplx<R>& u = U[i * ldu + j];
+    const cplx<R> v = D[i * ldd + j];
+    u = cplx<R>(u.re + f * v.re, u.im + f * v.im);
+  }
+}
+
 template <class R>
 __global__ void scale_rows_kernel(cplx<R>* x, int64_t rows, int64_t cols, int64_t ld, const R* sv, int invert) {
   const int64_t total = rows * cols;
@@ -573,6 +587,14 @@ int qtt_copy_strided(const cplx<R>* in, MIdx rows, MIdx cols, int64_t nrows, int
   copy_strided_kernel<R><<<nblocks(total), TPB, 0, s>>>(in, rows, cols, nrows, ncols, conj_in, out, ldo);
   CHECK_LAUNCH();
 }
+template <class R>
+int qtt_add_scaled_cols(cplx<R>* U, int64_t ldu, const cplx<R>* D, int64_t ldd, int64_t rows, int64_t cols, const R* sv,
+                        cudaStream_t s) {
+  if (rows * cols <= 0) return QTT_OK;
+  add_scaled_cols_kernel<R><<<nblocks(rows * cols), TPB, 0, s>>>(U, ldu, D, ldd, rows, cols, sv);
+  CHECK_LAUNCH();
+}
+template int qtt_add_scaled_cols<float>(cc*, int64_t, const cc*, int64_t, int64_t, int64_t, const float*, cudaStream_t);
 template <class R>
 int qtt_scale_rows(cplx<R>* x, int64_t rows, int64_t cols, int64_t ld, const R* sv, int invert, cudaStream_t s) {
   int64_t total = rows * cols;

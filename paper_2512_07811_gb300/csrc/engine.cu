@@ -1576,6 +1576,57 @@ int upload(qtt_ctx* c, void* dst, const void* src, size_t bytes) {
 }
 
 // ------------------------------------------------------------------- TT-SVD
+// Left vectors U (m x t, leading dimension ldu) of C (m x rest) and B = U^H C (t x
+// rest) set right to first order, in single precision.
+//   * Jacobi's rotated columns have taken about sqrt(columns x sweeps) roundings each,
+//     so a vector leans out of the range of C by up to 1e-6, and what of C it no
+//     longer covers is lost: 1e-6 ||C|| a bond, from the largest vectors.  One step
+//     of subspace iteration on the leaning alone: D = (I - U U^H) C B^H diag(sigma^-2), U
+//     += D, for the vectors with sigma_j >= sigma_0 / 32 (the products' own error is about
+//     1e-7 sigma_0 / sigma_j, a smaller vector would not gain).  D is orthogonal to
+//     U, so U stays orthonormal to |D|^2.
+//   * The vectors are orthogonal to 2e-8 a pair, 2e-7 of C a bond: B gets the
+//     correction of the least-squares problem, B += U^H (C - U B).
+// Columns of C in slabs, so that the extra buffers stay below 32 MiB or so.
+static int straighten_vectors(qtt_ctx* c, const cc* C, int64_t m, int64_t rest, cc* U, int64_t ldu, int64_t t,
+                              const float* sig, cc* B) {
+  std::vector<float> s(t);
+  TRY(sync_read(c, s.data(), sig, (size_t)t * sizeof(float)));
+  if (!(s[0] >= 1e-30f)) return QTT_OK;  // (so small that 1 / sigma would overflow)
+  int64_t t1 = 1;
+  while (t1 < t && s[t1] >= s[0] / 32) ++t1;
+  const int64_t w = std::min(rest, std::max<int64_t>(1024, ((int64_t)1 << 22) / m));
+  DBuf W, Y, S;
+  TRY(W.alloc(c, (size_t)m * w * sizeof(cc)));
+  TRY(Y.alloc(c, (size_t)m * t1 * sizeof(cc)));
+  TRY(S.alloc(c, (size_t)t * t1 * sizeof(cc)));
+  cc *wk = W.as<cc>(), *y = Y.as<cc>();
+  const cc one(1, 0), neg(-1, 0);
+  auto slab = [&](const cc* src, int64_t rows, int64_t n) {
+    return cudaMemcpy2DAsync(wk, n * sizeof(cc), src, rest * sizeof(cc), n * sizeof(cc), rows, cudaMemcpyDeviceToDevice,
+                             c->stream) == cudaSuccess ? QTT_OK : QTT_ERR_CUDA;
+  };
+  for (int64_t k = 0; k < rest; k += w) {
+    const int64_t n = std::min(w, rest - k);
+    TRY(slab(B + k, t1, n));
+    c->launches++;
+    TRY(qtt_scale_rows<float>(wk, t1, n, n, sig, 1, c->stream));
+    TRY(mm<float>(c, m, t1, n, C + k, rest, 1, 0, wk, 1, n, 1, y, t1, 1, one, k > 0 ? one : cc(0, 0)));
+  }
+  TRY(mm<float>(c, t, t1, m, U, 1, ldu, 1, y, t1, 1, 0, S.as<cc>(), t1, 1));
+  TRY(mm<float>(c, m, t1, t, U, ldu, 1, 0, S.as<cc>(), t1, 1, 0, y, t1, 1, neg, one));
+  c->launches++;
+  TRY(qtt_add_scaled_cols<float>(U, ldu, y, t1, m, t1, sig, c->stream));
+  TRY(mm<float>(c, t1, rest, m, U, 1, ldu, 1, C, rest, 1, 0, B, rest, 1));
+  for (int64_t k = 0; k < rest; k += w) {
+    const int64_t n = std::min(w, rest - k);
+    TRY(slab(C + k, m, n));
+    TRY(mm<float>(c, m, n, t, U, ldu, 1, 0, B + k, rest, 1, 0, wk, n, 1, neg, one));
+    TRY(mm<float>(c, t, n, m, U, 1, ldu, 1, wk, n, 1, 0, B + k, rest, 1, one, one));
+  }
+  return QTT_OK;
+}
+
 template <class R>
 int tt_svd_dev(qtt_ctx* c, int d, const std::vector<int>& modes, const cplx<R>* dense, double eps, int max_rank,
                qtt_dtype dt, qtt_tt** out) {
@@ -1612,14 +1663,16 @@ int tt_svd_dev(qtt_ctx* c, int d, const std::vector<int>& modes, const cplx<R>* 
     TRY(sync_read(c, hv, dint, sizeof(hv)));
     const int t = hv[0];
     ranks[k + 1] = t;
-    // core k = U[:, :t] as (rprev, n_k, t)
-    TRY(cores[k].alloc(c, (size_t)m * t * sizeof(cplx<R>)));
-    c->launches++;
-    TRY(qtt_copy_strided<R>(U.as<cplx<R>>(), L1(m, nsv), L1(t, 1), m, t, 0, cores[k].as<cplx<R>>(), t, c->stream));
     // next C = U_t^H C  (t x rest)
     DBuf Cn;
     TRY(Cn.alloc(c, (size_t)t * rest * sizeof(cplx<R>)));
     TRY(mm<R>(c, t, rest, m, U.as<cplx<R>>(), 1, nsv, 1, C, rest, 1, 0, Cn.as<cplx<R>>(), rest, 1));
+    if constexpr (sizeof(R) == 4)
+      TRY(straighten_vectors(c, C, m, rest, U.as<cc>(), nsv, t, sig.as<float>(), Cn.as<cc>()));
+    // core k = U[:, :t] as (rprev, n_k, t)
+    TRY(cores[k].alloc(c, (size_t)m * t * sizeof(cplx<R>)));
+    c->launches++;
+    TRY(qtt_copy_strided<R>(U.as<cplx<R>>(), L1(m, nsv), L1(t, 1), m, t, 0, cores[k].as<cplx<R>>(), t, c->stream));
     Cown = std::move(Cn);
     C = Cown.as<cplx<R>>();
     rprev = t;

@@ -93,6 +93,10 @@ int qtt_sumsq(const cplx<R>* x, int64_t count, double* out, cudaStream_t s);
 template <class R>
 int qtt_copy_strided(const cplx<R>* in, MIdx rows, MIdx cols, int64_t nrows, int64_t ncols, int conj_in,
                      cplx<R>* out, int64_t ldo, cudaStream_t s);
+// U += D diag(1 / sv) (row-major, leading dimensions ldu, ldd)
+template <class R>
+int qtt_add_scaled_cols(cplx<R>* U, int64_t ldu, const cplx<R>* D, int64_t ldd, int64_t rows, int64_t cols, const R* sv,
+                        cudaStream_t s);
 template <class R>
 int qtt_scale_rows(cplx<R>* x, int64_t rows, int64_t cols, int64_t ld, const R* sv, int invert,
                    cudaStream_t s);
