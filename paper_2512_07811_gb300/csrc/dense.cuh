@@ -22,27 +22,42 @@ __device__ __forceinline__ R wsum(R v) {
   return v;
 }
 
-// 1 / sqrt(x) and 1 / x to within a few units in the last place for normal x.
-// FP64 divisions and square roots of the CUDA library take tens of FP64
-// instructions each, and one FP64 warp instruction holds this part's FP64
-// pipe for 16 cycles; a hardware approximation (about 20 bits) corrected by
-// Newton steps takes about ten.  Arguments near the ends of the range (where
-// the approximation flushes or an intermediate could leave the normal range)
-// go to the library's functions.
+// 1 / sqrt(x) and 1 / x by Newton's method from an approximation that the
+// hardware gives (rsqrt.approx, rcp.approx of the PTX ISA; about 20 bits in FP64).
+// One FP64 warp instruction holds this part's FP64 pipe for 16 cycles and a
+// dependent one takes 75, so that the accuracy is bought no further than
+// needed and the chain kept short.
+//
+// Newton's method on f(y) = 1 / y^2 - x: with e = 1 - x y^2 the root is y (1 - e)^(-1/2) =
+// y (1 + e / 2 + 3 e^2 / 8 + 5 e^3 / 16 + ...), the step y + y e / 2 keeps the first
+// two terms and leaves 3 e^2 / 8: from |e| <= 2^-19 to 2^-39, then 2^-78.  The
+// rounding of the last step leaves e good to 2^-53 and y to 2 units in the last
+// place.  Newton's method on f(y) = 1 / y - x: e = 1 - x y, the root is y / (1 - e) =
+// y (1 + e + ...), the step y + y e leaves e^2 (2^-40, then 2^-80); here e is exact but
+// for its own last place: 1 unit.
+// The third-order step (the same series with its third term: Householder's
+// iteration of that order) goes from 2^-19 to 5 e^3 / 16 = 2^-58 at once: 2 units.
+// Arguments near the ends of the range, where the approximation flushes
+// subnormal values to zero, go to the library's functions.
 __device__ __forceinline__ float rsqrt_nr(float x) {
   // the correction is added (y + y e / 2): multiplying by 1.5 - x y^2 / 2 rounds
   // next to 1, where the spacing changes, and leaves a bias of -1.7e-8
   const float y = rsqrtf(x);
   return fmaf(0.5f * y, fmaf(-x * y, y, 1.0f), y);
 }
-__device__ __forceinline__ double rsqrt_nr(double x) {
-  if (!(x > 1e-290 && x < 1e290)) return 1.0 / sqrt(x);
+__device__ __forceinline__ double rsqrt_approx(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  double e = fma(-x * y, y, 1.0);            // third-order step: 20 -> 60 bits
-  y = fma(y * e, fma(0.375, e, 0.5), y);
-  e = fma(-x * y, y, 1.0);                   // rounding of the first step
-  return fma(0.5 * y, e, y);
+  return y;
+}
+__device__ __forceinline__ double rsqrt_newton(double x, double y) { return fma(0.5 * y, fma(-x * y, y, 1.0), y); }
+__device__ __forceinline__ double rsqrt_third_order(double x, double y) {
+  const double e = fma(-x * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+__device__ __forceinline__ double rsqrt_nr(double x) {
+  if (!(x > 1e-290 && x < 1e290)) return 1.0 / sqrt(x);
+  return rsqrt_newton(x, rsqrt_newton(x, rsqrt_approx(x)));
 }
 __device__ __forceinline__ float rcp_nr(float x) { return 1.0f / x; }
 __device__ __forceinline__ double rcp_nr(double x) {
@@ -50,10 +65,8 @@ __device__ __forceinline__ double rcp_nr(double x) {
   if (!(ax > 1e-290 && ax < 1e290)) return 1.0 / x;
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  double e = fma(-x, y, 1.0);
-  y = fma(y, fma(e, e, e), y);
-  e = fma(-x, y, 1.0);
-  return fma(y, e, y);
+  y = fma(y, fma(-x, y, 1.0), y);
+  return fma(y, fma(-x, y, 1.0), y);
 }
 
 // Compensated accumulation (Knuth's TwoSum): hi + lo += t.

@@ -121,11 +121,6 @@ __device__ __forceinline__ cplx<R> gsum_c(cplx<R> w, int lane) {
 }
 
 // FP64 helpers without FP64 instructions
-__device__ __forceinline__ double rsqrt_seed(double x) {  // about 20 bits
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  return y;
-}
 __device__ __forceinline__ double times2(double x, int k) {  // x 2^k, x normal
   return __hiloint2double(__double2hiint(x) + (k << 20), __double2loint(x));
 }
@@ -211,9 +206,9 @@ __device__ __forceinline__ int rotate_pair(cplx<R> (&x)[RT], cplx<R> (&y)[RT], R
     rot = act && (hg >> 20) + 1023 > ea + eb + ilogb_c(tol2) && hg >= kHiMin && hg < 0x7ff00000;
     if (LP == 32 ? !rot : !__any_sync(0xffffffffu, rot)) return 0;
     const R D = be - al, q4 = times2(ag2, 2), h2 = fma(D, D, q4);
-    const R H = h2 * rsqrt_seed(h2), W = fabs(D) + H;  // 2 h, 2 w
-    const R x4 = fma(W, W, q4), y0 = rsqrt_seed(x4), er = fma(-x4 * y0, y0, 1.0);
-    const R r2 = fma(y0 * er, fma(0.375, er, 0.5), y0);  // r / 2, one third-order step from 20 bits
+    const R H = h2 * dense::rsqrt_approx(h2), W = fabs(D) + H;  // 2 h, 2 w
+    const R x4 = fma(W, W, q4);
+    const R r2 = dense::rsqrt_third_order(x4, dense::rsqrt_approx(x4));  // r / 2
     const R r = times2(r2, 1);
     up = __double2hiint(D) >= 0;
     cs = W * r2;
