@@ -201,7 +201,7 @@ __device__ __forceinline__ int rotate_pair(cplx<R> (&x)[RT], cplx<R> (&y)[RT], R
     // a warp instruction holds its quarter's FP64 unit for 64 cycles: comparisons
     // by exponents (integer), factors of 2 and 4 by adding to them, h from the
     // hardware's 20-bit reciprocal square root.  The threshold then lies between
-    // tol / sqrt(2) and 2 tol.
+    // tol / sqrt(2) and sqrt(2) tol.
     const int hg = __double2hiint(ag2), ea = __double2hiint(al) >> 20, eb = __double2hiint(be) >> 20;
     rot = act && (hg >> 20) + 1023 > ea + eb + ilogb_c(tol2) && hg >= kHiMin && hg < 0x7ff00000;
     if (LP == 32 ? !rot : !__any_sync(0xffffffffu, rot)) return 0;
@@ -435,7 +435,7 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
     for (int e = threadIdx.x; e < 2 * bs * LD; e += nthr) slots[e] = (R)sg * slots[e];  // (bsx = bs)
     __syncthreads();
   }
-  // Pairs are rotated down to a cosine of eps / 2 (the inner product's own
+  // Pairs are rotated down to a cosine of eps / 2, in FP64 at most 0.7 eps (the inner product's own
   // rounding is below that): what is left of the cosines is the vectors'
   // non-orthogonality, which the truncated train inherits once per bond (a
   // tolerance of eps sqrt(p) made it the largest error of a rounding, 1e-5 at
@@ -448,7 +448,11 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
   // sine weighted by the norms' ratio of a sweep, the cosines after it are at
   // most about sqrt(qa) s c; with both at most sqrt(tol / sqrt(qa)) they are at
   // most tol, and the next sweep would rotate nothing.
-  const R big2 = tol / sqrt(R(qa));
+  // FP64 takes its angles from a square root good to 2^-20, so that a rotation also
+  // leaves 2^-21 of the cosine it removes (half of h's error goes into w); c is at
+  // most about 2 s, and s at most 2^19 tol keeps that below tol / 2.
+  R big2 = tol / sqrt(R(qa));
+  if constexpr (sizeof(R) == 8) big2 = fmin(big2, tol2 * R(1ll << 38));
   C x[RT], y[RT];
   auto load = [&](C(&v)[RT], const C* s) {
 #pragma unroll

@@ -148,3 +148,22 @@ def test_norms_of_rounded_cores_fp32(Q, ctx, sketched):
         stored.append(norm2((m / np.linalg.norm(m, axis=1, keepdims=True)).astype(np.complex64)))
     rms = lambda v: math.sqrt((np.concatenate(v) ** 2).mean())  # noqa: E731
     assert rms(off) <= math.hypot(rms(stored), 0.5 * 2.0 ** -24)
+
+
+def test_cosines_left_by_the_last_sweep(Q, ctx):
+    """Two columns whose cosine is 6e-9: small enough for the quadratic regime, large enough that a rotation
+    from a 20-bit angle alone would leave up to 3e-15.  Rotations stop below 2 u (a threshold by exponents); the
+    two stored vectors' entries, each good to 2 u (scaled, rounded), add 4 u at most: 6 u."""
+    rng = np.random.default_rng(11)
+    worst = 0.0
+    for ratio in np.linspace(0.2, 0.6, 60):
+        # the first column is the largest and parallel to e_1, so that the QR leaves the rows as they are
+        c = _unitary(rng, 7, 2).conj().T * np.array([[0.3], [1.0]])
+        c[1] += 6e-9 / 0.3 * c[0] / 0.3
+        c = np.concatenate([[[0.95], [0.0]], c], axis=1)
+        c = c / np.linalg.norm(c, axis=1, keepdims=True) * np.array([[1.0], [ratio]])
+        y, _ = Q.tt_round(ctx, Q.TT.from_cores(ctx, [np.eye(2)[None], c[:, :, None]], Q.C128), 0.0)
+        b = y.cores()[1][:, :, 0].astype(np.clongdouble)
+        assert b.shape == (2, 8)
+        worst = max(worst, float(abs((b[0].conj() * b[1]).sum())))
+    assert worst <= 6 * 2.0 ** -53
