@@ -313,7 +313,7 @@ int qtt_ctx_create(int device, void* stream, qtt_ctx** out) {
 
 void qtt_ctx_destroy(qtt_ctx* c) {
   if (!c) return;
-  dcache_release(c);
+  c->blocks.finish();
   cudaStreamSynchronize(c->stream);
   prof_clear(c);
   if (c->d_sweeps) cudaFree(c->d_sweeps);

@@ -36,72 +36,24 @@ int dalloc(qtt_ctx* c, void** p, size_t bytes) {
     if (c->fail_alloc_after == 0) return QTT_ERR_OOM;  // injected failure (qtt_ctx_fail_alloc_after)
     --c->fail_alloc_after;
   }
-  // size classes: eight per power of two, at least 512 bytes
-  size_t cls = 512;
-  if (bytes > cls) {
-    int sh = 0;
-    while ((bytes - 1) >> (sh + 4)) ++sh;
-    cls = (((bytes - 1) >> sh) + 1) << sh;
-  }
-  BlockCache& bc = c->blocks;
-  // under stream capture the allocation becomes a node of the graph: such a
-  // block never enters the cache, and none is taken from it
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) cudaGetLastError();
-  const bool capturing = cap != cudaStreamCaptureStatusNone;
-  if (!capturing) {
-    std::lock_guard<std::mutex> lk(bc.mu);
-    auto it = bc.free_lists.find(cls);
-    if (it != bc.free_lists.end() && !it->second.empty()) {
-      *p = it->second.back();
-      it->second.pop_back();
-      bc.cached -= cls;
-      return QTT_OK;
-    }
-  }
-  if (cudaMallocAsync(p, cls, c->stream) != cudaSuccess) {
-    cudaGetLastError();
-    *p = nullptr;
-    if (capturing) return QTT_ERR_OOM;
-    dcache_release(c);
-    if (cudaMallocAsync(p, cls, c->stream) != cudaSuccess) {
-      cudaGetLastError();
-      *p = nullptr;
-      return QTT_ERR_OOM;
-    }
-  }
-  if (capturing) return QTT_OK;
-  std::lock_guard<std::mutex> lk(bc.mu);
-  bc.size_of[*p] = cls;
-  return QTT_OK;
+  return c->blocks.alloc(p, bytes) ? QTT_OK : QTT_ERR_OOM;
 }
 void dfree(qtt_ctx* c, void* p) {
-  if (!p) return;
-  BlockCache& bc = c->blocks;
-  {
-    std::lock_guard<std::mutex> lk(bc.mu);
-    auto it = bc.size_of.find(p);
-    const size_t cls = it == bc.size_of.end() ? 0 : it->second;
-    if (cls && cls <= BlockCache::kMaxBlock && bc.cached + cls <= BlockCache::kMaxTotal) {
-      bc.free_lists[cls].push_back(p);
-      bc.cached += cls;
-      return;
-    }
-    if (cls) bc.size_of.erase(it);
-  }
-  cudaFreeAsync(p, c->stream);
+  if (p) c->blocks.free(p);
 }
-void dcache_release(qtt_ctx* c) {
-  BlockCache& bc = c->blocks;
-  std::lock_guard<std::mutex> lk(bc.mu);
-  for (auto& l : bc.free_lists)
-    for (void* p : l.second) {
-      bc.size_of.erase(p);
-      cudaFreeAsync(p, c->stream);
-    }
-  bc.free_lists.clear();
-  bc.cached = 0;
+bool qtt_ctx::Driver::alloc(void** p, size_t bytes) {
+  if (cudaMallocAsync(p, bytes, c->stream) == cudaSuccess) return true;
+  cudaGetLastError();
+  *p = nullptr;
+  return false;
 }
+void qtt_ctx::Driver::release(void* p) { cudaFreeAsync(p, c->stream); }
+bool qtt_ctx::Driver::capturing() {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) cudaGetLastError();
+  return cap != cudaStreamCaptureStatusNone;
+}
+void qtt_ctx::Driver::settle() { cudaStreamSynchronize(c->stream); }
 
 int sync_read(qtt_ctx* c, void* host, const void* dev, size_t bytes) {
   if (cudaMemcpyAsync(host, dev, bytes, cudaMemcpyDeviceToHost, c->stream) != cudaSuccess) return QTT_ERR_CUDA;

@@ -4,12 +4,10 @@
 #include <stdint.h>
 
 #include <algorithm>
-#include <map>
-#include <mutex>
-#include <unordered_map>
 #include <vector>
 
 #include "../../include/qtt.h"
+#include "blocks.h"
 #include "common.cuh"
 #include "kernels.h"
 
@@ -26,22 +24,6 @@ struct ProfRec {
   int variant;           // GEMM: tile edge (32, 64; 128 = tensor cores) x 100 + split-K; else 0
 };
 
-// Device blocks that a context has freed, kept for its next allocations of the
-// same size class.  All work of a context runs on its one stream, so a block
-// may be handed out again at once: its new user's kernels come after its last
-// user's.  Bounded (a block above 64 MiB, or beyond 512 MiB in all, goes back
-// to the driver), emptied when an allocation fails and when the context is
-// destroyed, and locked, as several host threads may use one context.  It
-// saves two driver calls per buffer; a solve's six load-case threads queue on
-// the driver's lock (about 30 buffers per rounded core).
-struct BlockCache {
-  static constexpr size_t kMaxBlock = (size_t)64 << 20, kMaxTotal = (size_t)512 << 20;
-  std::mutex mu;
-  std::unordered_map<void*, size_t> size_of;       // every live or cached block
-  std::map<size_t, std::vector<void*>> free_lists; // by size class
-  size_t cached = 0;
-};
-
 struct qtt_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
@@ -56,7 +38,17 @@ struct qtt_ctx {
   bool tc_sketch = false;    // the sketch contractions of sketched roundings on the tensor cores, 1 pass
   bool in_sketch = false;    // set while those contractions are issued
   int* d_tcerr = nullptr;    // bounded-wait failure flag of the tensor-core GEMM
-  BlockCache blocks;
+  // the driver's stream-ordered allocations, for `blocks` (engine.cu)
+  struct Driver final : BlockDevice {
+    qtt_ctx* c;
+    explicit Driver(qtt_ctx* ctx) : c(ctx) {}
+    int id() override { return c->device; }
+    bool alloc(void** p, size_t bytes) override;
+    void release(void* p) override;
+    bool capturing() override;
+    void settle() override;
+  } driver{this};
+  BlockCache blocks{&driver};
   int64_t fail_alloc_after = -1;  // test hook: allocations left before dalloc fails (-1: off)
   // profiler totals handed over by contexts that worked for this one (the
   // load-case workers of ms_homogenize), per kernel class
@@ -144,7 +136,6 @@ struct qtt_mpo {
 
 size_t dtype_size(qtt_dtype t);
 int dalloc(qtt_ctx* c, void** p, size_t bytes);
-void dcache_release(qtt_ctx* c);  // every cached block back to the driver
 void dfree(qtt_ctx* c, void* p);
 int sync_read(qtt_ctx* c, void* host, const void* dev, size_t bytes);
 qtt_tt* tt_alloc(qtt_ctx* c, int d, const std::vector<int>& n, const std::vector<int>& r, qtt_dtype dt, int* st);
