@@ -118,7 +118,8 @@ QTT_API int qtt_ctx_profile_read(qtt_ctx* ctx, int kclass, double* total_ms, int
  * total ms, model flops -- GEMM: M, N, K, batch and variant = tile edge x 100
  * + split-K count (the FP32 tile's edge, the FP64 kernel has smaller ones;
  * tile edge 128: the tensor-core kernel, + its TF32 passes); QR: m, n, 0, batch, variant 1 when the explicit Q was formed;
- * Jacobi: rows p, columns q, 0, batch, 0.  *n_rows = the number of distinct
+ * Jacobi: rows p, columns q, 0, batch, variant 1 for the FP32 rotations that an FP64 SVD starts with (their flops are
+ * FP32 ones).  *n_rows = the number of distinct
  * shapes (may exceed max_rows).  Synchronises the stream.  QTT_ERR_ARG on a
  * bad class or null pointers. */
 QTT_API int qtt_ctx_profile_shapes(qtt_ctx* ctx, int kclass, double* rows, int64_t max_rows, int64_t* n_rows);

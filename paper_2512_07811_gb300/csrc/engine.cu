@@ -624,7 +624,13 @@ static int svd_right(qtt_ctx* c, const cplx<R>* in, MIdx inB, MIdx rowI, MIdx co
       TRY(GV.alloc(c, (size_t)batch * n * q * sizeof(zc)));
       zc *v = V.as<zc>(), *e[2] = {v + batch * qq, v + 2 * batch * qq}, *v1 = V1.as<zc>();
       c->launches++;
-      TRY(qtt_svd_pre(G.as<zc>(), v, delta, deltas, (int)n, (int)q, (int)batch, nullptr, c->stream));
+      int pidx;
+      int* pslot = prof_sweep_slot(c, &pidx);
+      cudaEvent_t pev = prof_begin(c);
+      TRY(qtt_svd_pre(G.as<zc>(), v, delta, deltas, (int)n, (int)q, (int)batch, pslot, c->stream));
+      prof_end(c, pev, PK_JACOBI, 0.0, (double)batch * (n + 3.0 * q) * q * sizeof(zc), pidx,
+               batch * jacobi_sweep_flops((double)n, (double)q));
+      prof_shape(c, pev, n, q, 0, batch, 1);
       for (int it = 0; it < 2; ++it) {
         // E = 3/2 - V^H V / 2, V <- V E (V stored transposed)
         TRY(simt_gemm<double>(c, bgemm<double>(batch, q, q, q, qq, L1(q, q), L1(q, 1), qq, L1(q, 1), L1(q, q), qq,

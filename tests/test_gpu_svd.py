@@ -167,3 +167,22 @@ def test_cosines_left_by_the_last_sweep(Q, ctx):
         assert b.shape == (2, 8)
         worst = max(worst, float(abs((b[0].conj() * b[1]).sum())))
     assert worst <= 6 * 2.0 ** -53
+
+
+def test_profile_counts_the_fp32_start(Q, ctx):
+    """An FP64 SVD of 64 columns starts with FP32 rotations: a Jacobi launch of its own in the profiler."""
+    rng = np.random.default_rng(2)
+    x = Q.TT.from_cores(ctx, [(_unitary(rng, 64, 64) * np.logspace(0, -6, 64))[None],
+                              _unitary(rng, 64, 64).conj().T[:, :, None]], Q.C128)
+    ctx.profile(True)
+    try:
+        Q.tt_round(ctx, x, 1e-9)
+        rows = {r["variant"]: r for r in ctx.profile_shapes("jacobi")}
+        total = ctx.profile_read("jacobi")
+    finally:
+        ctx.profile(False)
+    assert sorted(rows) == [0, 1] and total["launches"] == 2
+    for r in rows.values():
+        assert r["dims"] == (64, 64, 0) and r["launches"] == 1 and r["ms"] > 0 and r["flops"] > 0
+    # the sweeps of the two: several in FP32, then two or three
+    assert rows[1]["flops"] > rows[0]["flops"]
