@@ -202,7 +202,7 @@ static int tc_route(qtt_ctx* c, const GemmDesc& g0, cc alpha, cc beta, const cc*
 }
 
 // ------------------------------------------------------ GEMM tile autotuner
-// The first FP32 CUDA-core GEMM of a shape (element size, M, N, K, batch and which
+// The first FP32 CUDA-core GEMM of a shape (M, N, K, batch and which
 // operand indices are contiguous) with enough work times the two tile edges
 // (32, 64) once, at the split count the rule gives the shape, with CUDA
 // events on the caller's stream into a scratch output, and caches the
@@ -211,16 +211,15 @@ static int tc_route(qtt_ctx* c, const GemmDesc& g0, cc alpha, cc beta, const cc*
 // across contexts, threads and processes.  GEMMs that accumulate into C
 // (beta != 0) or are too small to matter keep the rule's choice.
 struct TuneKey {
-  int64_t v[7];
-  bool operator<(const TuneKey& o) const { return std::lexicographical_compare(v, v + 7, o.v, o.v + 7); }
+  int64_t v[6];
+  bool operator<(const TuneKey& o) const { return std::lexicographical_compare(v, v + 6, o.v, o.v + 6); }
 };
 static std::mutex g_tune_mu;
 static std::map<TuneKey, std::pair<int, int>> g_tune;  // -> (tile, splits)
 
 static bool unit_inner(const MIdx& m) { return (m.n2 == 1 ? m.s1 : m.s2) == 1; }
 
-template <class R>
-static int tune_gemm(qtt_ctx* c, const GemmDesc& g, const cplx<R>* A, const cplx<R>* B, int* tile, int* splits) {
+static int tune_gemm(qtt_ctx* c, const GemmDesc& g, const cc* A, const cc* B, int* tile, int* splits) {
   GemmDesc d = g;  // dense scratch output
   d.bC = MIdx{g.batch, 1, g.M * g.N, 0};
   d.mC = MIdx{g.M, 1, g.N, 0};
@@ -236,10 +235,10 @@ static int tune_gemm(qtt_ctx* c, const GemmDesc& g, const cplx<R>* A, const cplx
   int maxs = 1;
   for (auto& cs : cand) maxs = std::max(maxs, cs.second);
   void* buf = nullptr;
-  const size_t outb = (size_t)g.batch * g.M * g.N * sizeof(cplx<R>);
+  const size_t outb = (size_t)g.batch * g.M * g.N * sizeof(cc);
   if (dalloc(c, &buf, outb * (1 + (maxs > 1 ? maxs : 0)))) return QTT_ERR_OOM;
-  cplx<R>* Cs = reinterpret_cast<cplx<R>*>(buf);
-  cplx<R>* Ps = Cs + (size_t)g.batch * g.M * g.N;
+  cc* Cs = reinterpret_cast<cc*>(buf);
+  cc* Ps = Cs + (size_t)g.batch * g.M * g.N;
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
@@ -249,7 +248,7 @@ static int tune_gemm(qtt_ctx* c, const GemmDesc& g, const cplx<R>* A, const cplx
     float ms = 0.f;
     for (int rep = 0; rep < 2 && st == QTT_OK; ++rep) {  // first run warms up
       cudaEventRecord(e0, c->stream);
-      st = qtt_gemm_ex<R>(d, cplx<R>(1, 0), cplx<R>(0, 0), A, B, Cs, cs.second, Ps, c->stream, cs.first);
+      st = qtt_gemm_ex<float>(d, cc(1, 0), cc(0, 0), A, B, Cs, cs.second, Ps, c->stream, cs.first);
       cudaEventRecord(e1, c->stream);
       if (cudaEventSynchronize(e1) != cudaSuccess) st = QTT_ERR_CUDA;
       cudaEventElapsedTime(&ms, e0, e1);
@@ -272,21 +271,23 @@ template <class R>
 static int simt_gemm(qtt_ctx* c, const GemmDesc& g, cplx<R> alpha, cplx<R> beta, const cplx<R>* A, const cplx<R>* B,
                      cplx<R>* C) {
   int tile = 0, splits = sizeof(R) == 8 ? qtt_gemm_splits_f64(g) : qtt_gemm_splits(g);
-  const bool beta0 = beta.re == R(0) && beta.im == R(0);
-  if (sizeof(R) == 4 && beta0 && (double)g.M * g.N * g.K * g.batch >= 4.0e6) {
-    const bool a_kfast = unit_inner(g.kA) && !unit_inner(g.mA);
-    const bool b_kfast = unit_inner(g.kB) && !unit_inner(g.nB);
-    const TuneKey key{{(int64_t)sizeof(R), g.M, g.N, g.K, g.batch, (int64_t)a_kfast, (int64_t)b_kfast}};
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    auto it = g_tune.find(key);
-    if (it == g_tune.end()) {
-      int t = qtt_gemm_tile_rule(g), sp = splits;
-      const int ts = tune_gemm<R>(c, g, A, B, &t, &sp);
-      if (ts != QTT_OK) return ts;
-      it = g_tune.emplace(key, std::make_pair(t, sp)).first;
+  [[maybe_unused]] const bool beta0 = beta.re == R(0) && beta.im == R(0);
+  if constexpr (sizeof(R) == 4) {  // (an FP64 contraction's tile follows from its shape)
+    if (beta0 && (double)g.M * g.N * g.K * g.batch >= 4.0e6) {
+      const bool a_kfast = unit_inner(g.kA) && !unit_inner(g.mA);
+      const bool b_kfast = unit_inner(g.kB) && !unit_inner(g.nB);
+      const TuneKey key{{g.M, g.N, g.K, g.batch, (int64_t)a_kfast, (int64_t)b_kfast}};
+      std::lock_guard<std::mutex> lk(g_tune_mu);
+      auto it = g_tune.find(key);
+      if (it == g_tune.end()) {
+        int t = qtt_gemm_tile_rule(g), sp = splits;
+        const int ts = tune_gemm(c, g, A, B, &t, &sp);
+        if (ts != QTT_OK) return ts;
+        it = g_tune.emplace(key, std::make_pair(t, sp)).first;
+      }
+      tile = it->second.first;
+      splits = it->second.second;
     }
-    tile = it->second.first;
-    splits = it->second.second;
   }
   void* P = nullptr;
   splits = (int)std::min<int64_t>(splits, std::max<int64_t>(1, 65535 / std::max<int64_t>(1, g.batch)));

@@ -197,7 +197,6 @@ template <class R>
 int gemm_ab(qtt_ctx* c, const GemmDesc& g, cplx<R> alpha, cplx<R> beta, const cplx<R>* A, const cplx<R>* B,
             cplx<R>* C);
 
-// z = a x + b y (ranks add) and a synchronous host -> device copy (engine.cu)
 // cores of a train handed to a table kernel QTT_TABLE at a time: fn(first, count)
 template <class F>
 inline int each_table(int d, F fn) {
@@ -213,6 +212,7 @@ inline int each_table(int d, F fn) {
 template <class R>
 int control_sums(qtt_ctx* c, const qtt_tt* x, const qtt_tt* chi, double* out);
 
+// z = a x + b y (ranks add) and a synchronous host -> device copy (engine.cu)
 template <class R>
 int add_dev(qtt_ctx* c, cplx<R> a, const qtt_tt* x, cplx<R> b, const qtt_tt* y, qtt_tt** out);
 int upload(qtt_ctx* c, void* dst, const void* src, size_t bytes);

@@ -71,6 +71,27 @@ def test_projection_onto_an_explicit_q(Q, ctx, m, n, fp32):
     assert np.linalg.norm(full - ref) <= 4 * _tol(max(m, n), fp32) * np.linalg.norm(ref)
 
 
+# FP32 matrices too wide for a cluster's shared memory: the blocked kernel's instances, then the panel kernel
+WIDE = [(120, 3000), (250, 1500), (288, 1300), (400, 700), (500, 700)]
+
+
+@pytest.mark.parametrize("m,n", WIDE)
+def test_norm_of_a_wide_train(Q, ctx, m, n):
+    test_norm_of_a_two_core_train(Q, ctx, m, n, True)
+
+
+@pytest.mark.parametrize("m,n", WIDE)
+def test_projection_of_a_wide_sketch(Q, ctx, m, n):
+    """The explicit Q (m x m) of an m x n sketched unfolding of rank 2: Q Q^H = 1."""
+    rng = np.random.default_rng(m * 1000 + n + 9)
+    x = [_rand(rng, 1, m, 2), _rand(rng, 2, 2, 1)]
+    sk = [_rand(rng, 1, m, n), _rand(rng, n, 2, 1)]
+    y, _ = Q.tt_round_sketched(ctx, [(1.0, None, Q.TT.from_cores(ctx, x, Q.C64))], Q.TT.from_cores(ctx, sk, Q.C64), 0.0)
+    a, b = [c.astype(np.complex128) for c in y.cores()]
+    full, ref = a[0] @ b[:, :, 0], x[0][0] @ x[1][:, :, 0]
+    assert np.linalg.norm(full - ref) <= 4 * _tol(m, True) * np.linalg.norm(ref)
+
+
 @pytest.mark.parametrize("scale", [1e-28, 1e-15, 1e15])
 def test_fp32_range(Q, ctx, scale):
     """Squares of the entries leave the FP32 range; the kernel scales by a power of two."""
