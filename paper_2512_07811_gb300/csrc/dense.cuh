@@ -69,7 +69,10 @@ __device__ __forceinline__ double rcp_nr(double x) {
   return fma(y, fma(-x, y, 1.0), y);
 }
 
-// Compensated accumulation (Knuth's TwoSum): hi + lo += t.
+// Compensated sums in working precision: a partial sum carries its rounding
+// error (Knuth's TwoSum), so that a sum of squares over a column is good to a few
+// units in the last place however many terms it has, without FP64 arithmetic
+// (slow on this part).  hi + lo += t.
 template <class R>
 __device__ __forceinline__ void add_comp(R& hi, R& lo, R t) {
   const R s = hi + t, bb = s - hi;
@@ -103,5 +106,16 @@ __device__ __forceinline__ void unit_norm(cplx<float> (&x)[N]) {
 #pragma unroll
   for (int u = 0; u < N; ++u) x[u] = cplx<float>(fmaf(x[u].re, k, x[u].re), fmaf(x[u].im, k, x[u].im));
 }
+
+// Exponent of a positive finite value, at least `least`, which also stands for
+// zero and for what is not finite; 2^e.
+__device__ __forceinline__ int exponent_of(float a, int least) {
+  return a > 0 && a <= FLT_MAX ? max(ilogbf(a), least) : least;
+}
+__device__ __forceinline__ int exponent_of(double a, int least) {
+  return a > 0 && a <= DBL_MAX ? max(ilogb(a), least) : least;
+}
+__device__ __forceinline__ float pow2(float, int e) { return ldexpf(1.f, e); }
+__device__ __forceinline__ double pow2(double, int e) { return ldexp(1.0, e); }
 
 }  // namespace dense

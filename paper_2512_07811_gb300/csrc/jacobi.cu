@@ -246,11 +246,6 @@ __device__ __forceinline__ int rotate_pair(cplx<R> (&x)[RT], cplx<R> (&y)[RT], R
   return code;
 }
 
-__device__ __forceinline__ int jac_exponent(float a) { return a > 0 && a <= FLT_MAX ? max(ilogbf(a), -110) : -110; }
-__device__ __forceinline__ int jac_exponent(double a) { return a > 0 && a <= DBL_MAX ? max(ilogb(a), -1000) : -1000; }
-__device__ __forceinline__ float jac_pow2(float, int e) { return ldexpf(1.f, e); }
-__device__ __forceinline__ double jac_pow2(double, int e) { return ldexp(1.0, e); }
-
 template <class R, int LP, int RPL, bool PRE>
 __global__ void __launch_bounds__(JacThreads<R, RPL, PRE>::value, 1)
 jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
@@ -314,7 +309,7 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
     });
   }
   {
-    const int ex = __reduce_max_sync(0xffffffffu, jac_exponent(amax));
+    const int ex = __reduce_max_sync(0xffffffffu, dense::exponent_of(amax, sizeof(S) == 4 ? -110 : -1000));
     int* wex = reinterpret_cast<int*>(sorted);
     if (lane == 0) wex[warp] = ex;
     __syncthreads();
@@ -327,7 +322,7 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
   int esc = flags[32];
   for (int i = 1; i < NC; ++i) esc = max(esc, flags[32 + i]);
   if (sizeof(R) == 4) esc -= 14;
-  const S sg = jac_pow2(S(0), -esc);
+  const S sg = dense::pow2(S(0), -esc);
   if (a.adapt) {
     // Trailing columns whose whole norm is at most eps ||G|| (one rounding of G)
     // and a quarter of the truncation threshold are left out: in a rounding
@@ -366,7 +361,7 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
       for (int j = lane; j < q; j += 32) tot += (double)cn[j];
       tot = dense::wsum(tot);
       constexpr double eps = sizeof(S) == 4 ? (double)FLT_EPSILON : DBL_EPSILON;
-      const double ds = 0.25 * (a.deltas ? a.deltas[bt] : a.delta) * jac_pow2(0.0, -esc);
+      const double ds = 0.25 * (a.deltas ? a.deltas[bt] : a.delta) * dense::pow2(0.0, -esc);
       double thr2 = eps * eps * tot;
       if (!(ds * ds >= thr2)) thr2 = ds * ds;  // (a NaN drops nothing)
       double out = 0;
@@ -627,7 +622,7 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
     }
     return;
   }
-  const R sb = jac_pow2(R(0), esc);
+  const R sb = dense::pow2(R(0), esc);
   for (int k0 = 0; k0 < qa; k0 += ng) {
     const int c = min(k0 + w, qa - 1), rk = place(c);
     if (gl == 0 && k0 + w < qa) sorted[rk] = norms[c] * sb;
@@ -635,14 +630,14 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
   __syncthreads();
   if (a.sigma && rank == 0)
     for (int i = threadIdx.x; i < q; i += nthr)  // (the dropped columns' norm as one value)
-      a.sigma[bt * q + i] = i < qa ? sorted[i] : i == qa ? (R)(sqrt(scan[0]) * jac_pow2(0.0, esc)) : R(0);
+      a.sigma[bt * q + i] = i < qa ? sorted[i] : i == qa ? (R)(sqrt(scan[0]) * dense::pow2(0.0, esc)) : R(0);
   int keep = qa;
   if (a.trunc) {
     // smallest t >= 1 with sqrt(sum_{j >= t} s_j^2) <= delta, sums in double
     // by a suffix scan over the lanes, 32 values at a time from the end
     if (threadIdx.x < 32) {
       const double delta = a.deltas ? a.deltas[bt] : a.delta;
-      const double sq = jac_pow2(0.0, esc);
+      const double sq = dense::pow2(0.0, esc);
       double tail = qa < q ? scan[0] * sq * sq : 0.0;
       int t = qa;
       bool stop = false;

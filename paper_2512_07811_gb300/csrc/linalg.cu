@@ -15,6 +15,7 @@
 #include <utility>
 
 #include "common.cuh"
+#include "dense.cuh"
 #include "kernels.h"
 
 namespace {
@@ -855,27 +856,9 @@ int qtt_allow_max_smem(const void* func) {
   return QTT_OK;
 }
 
-// Compensated sums in working precision: each partial sum carries its
-// rounding error (Knuth's TwoSum), so a sum of squares over a column is
-// accurate to a few units in the last place however many terms it has,
-// without FP64 arithmetic (slow on this part).
-template <class R>
-__device__ __forceinline__ void two_sum_acc(R& hi, R& lo, R t) {
-  const R s = hi + t;
-  const R bb = s - hi;
-  lo += (hi - (s - bb)) + (t - bb);
-  hi = s;
-}
-
 template <class R>
 __device__ __forceinline__ R warp_sum_compensated(R hi, R lo) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const R ohi = __shfl_xor_sync(0xffffffffu, hi, o);
-    const R olo = __shfl_xor_sync(0xffffffffu, lo, o);
-    lo += olo;
-    two_sum_acc(hi, lo, ohi);
-  }
+  dense::wsum_comp(hi, lo);
   return hi + lo;
 }
 
@@ -1037,7 +1020,7 @@ qr_panel_kernel(const cplx<R>* __restrict__ in, MIdx inB, MIdx rowI, MIdx colI, 
         const int i = lane + 32 * u;
         if (i < m) {
           pc[i] = x[u];
-          if (warp == 0 && i > p0) two_sum_acc(hi, lo, abs2(x[u]));
+          if (warp == 0 && i > p0) dense::add_comp(hi, lo, abs2(x[u]));
         }
       }
       if (warp == 0 && pw > 0) {
@@ -1075,7 +1058,7 @@ qr_panel_kernel(const cplx<R>* __restrict__ in, MIdx inB, MIdx rowI, MIdx colI, 
 #pragma unroll
           for (int u = 0; u < RPL; ++u) {
             const int i = lane + 32 * u;
-            if (i >= j + 2 && i < m) two_sum_acc(hi, lo, abs2(xr[u]));
+            if (i >= j + 2 && i < m) dense::add_comp(hi, lo, abs2(xr[u]));
           }
           const R below = warp_sum_compensated(hi, lo);
           qr_reflector_warp<R, MP>(colc, j + 1, m, below, zero_thresh2, lane, s_taus, s_ivs, tw,
@@ -1360,7 +1343,7 @@ qr_blocked_kernel(const cplx<R>* __restrict__ in, MIdx inB, MIdx rowI, MIdx colI
 #pragma unroll
         for (int u = 0; u < RPL; ++u) {
           const int i = lane + 32 * u;
-          if (i > j && i < m) two_sum_acc(hi, lo, abs2(xr[u]));
+          if (i > j && i < m) dense::add_comp(hi, lo, abs2(xr[u]));
           if (i == j) x0 = xr[u];
         }
         const R below = warp_sum_compensated(hi, lo);

@@ -185,16 +185,6 @@ __device__ __forceinline__ cplx<R> load_l2(const cplx<R>* p) {
   }
 }
 
-// power of two below the largest component, as an exponent; 0 where there is none or it is not finite
-__device__ __forceinline__ int exponent_of(float a) {
-  return a > 0 && a <= FLT_MAX ? max(ilogbf(a), -120) : -120;
-}
-__device__ __forceinline__ int exponent_of(double a) {
-  return a > 0 && a <= DBL_MAX ? max(ilogb(a), -1000) : -1000;
-}
-__device__ __forceinline__ float pow2(float, int e) { return ldexpf(1.f, e); }
-__device__ __forceinline__ double pow2(double, int e) { return ldexp(1.0, e); }
-
 template <class R, int RPL>
 __global__ void __launch_bounds__(QrThreads<R>::value, 1)
 qr_cluster_kernel(const __grid_constant__ QrArgs<R> a) {
@@ -285,11 +275,11 @@ qr_cluster_kernel(const __grid_constant__ QrArgs<R> a) {
       R t = lane < NW ? parts[lane] : R(0);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) t = fmax(t, __shfl_xor_sync(0xffffffffu, t, o));
-      if (lane == 0) exps[16] = exponent_of(t);
+      if (lane == 0) exps[16] = dense::exponent_of(t, sizeof(R) == 4 ? -120 : -1000);
     }
     __syncthreads();
     const int el = exps[16];
-    const R sl = pow2(R(0), -el);
+    const R sl = dense::pow2(R(0), -el);
     R part = 0;
     for (int e = threadIdx.x; e < tot * LD; e += QT) part += abs2(sl * cols[e]);
     part = dense::wsum(part);
@@ -307,9 +297,9 @@ qr_cluster_kernel(const __grid_constant__ QrArgs<R> a) {
     esc = exps[0];
     for (int i = 1; i < NC; ++i) esc = max(esc, exps[i]);
     R fro2 = 0;
-    for (int i = 0; i < NC; ++i) fro2 += parts[16 + i] * pow2(R(0), max(2 * (exps[i] - esc), sizeof(R) == 4 ? -120 : -1000));
+    for (int i = 0; i < NC; ++i) fro2 += parts[16 + i] * dense::pow2(R(0), max(2 * (exps[i] - esc), sizeof(R) == 4 ? -120 : -1000));
     zero2 = Lim<R>::eps * Lim<R>::eps * fro2;
-    const R sg = pow2(R(0), -esc);
+    const R sg = dense::pow2(R(0), -esc);
     for (int e = threadIdx.x; e < tot * LD; e += QT) cols[e] = sg * cols[e];
     __syncthreads();
   }
@@ -422,7 +412,7 @@ qr_cluster_kernel(const __grid_constant__ QrArgs<R> a) {
   }
   if (a.out) {
     __syncthreads();
-    const R sb = pow2(R(0), esc);
+    const R sb = dense::pow2(R(0), esc);
     C* o = a.out + bt * a.out_bstride;
     for (int lc = warp; lc < a.slots * b; lc += NW) {
       const int sl = lc / b, c = (sl * NC + rank) * b + (lc - sl * b);
