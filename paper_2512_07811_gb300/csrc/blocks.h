@@ -24,6 +24,7 @@
 #include <stddef.h>
 
 #include <algorithm>
+#include <atomic>
 #include <map>
 #include <mutex>
 #include <unordered_map>
@@ -140,13 +141,15 @@ class BlockCache {
     auto& r = registry();
     r.erase(std::remove(r.begin(), r.end(), this), r.end());
   }
-  // false where the bound does not allow it
+  // false where the bound does not allow it (one counter for all contexts, no lock: every
+  // allocation and release of a solve's threads comes here)
   static bool add_cached(ptrdiff_t n) {
-    static std::mutex& m = *new std::mutex;
-    static size_t total = 0;
-    std::lock_guard<std::mutex> lk(m);
-    if (n > 0 && total + (size_t)n > kMaxTotal) return false;
-    total += n;
+    static std::atomic<ptrdiff_t>& total = *new std::atomic<ptrdiff_t>(0);
+    const ptrdiff_t now = total.fetch_add(n) + n;
+    if (n > 0 && now > (ptrdiff_t)kMaxTotal) {
+      total.fetch_sub(n);
+      return false;
+    }
     return true;
   }
   static std::mutex& registry_mu() {
