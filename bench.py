@@ -54,9 +54,9 @@ E2E_OP_TOL = 1e-6   # the float path's operators in float (ms_setup)
 # dominant kernel class, from the one-kernel ncu captures summarised in
 # profiles/ (file named in the line); None where no current capture exists.
 TRAFFIC = {
-    "jacobi_cluster2_kernel": {"bytes": 368.64e3, "profile": "profiles/jacobi_cluster2_kernel_sphere32.md"},
-    "qr_cluster_kernel": {"bytes": 372.48e3, "profile": "profiles/qr_cluster_kernel_sphere32.md"},
-    "gemm_midx_kernel": {"bytes": 554.496e3, "profile": "profiles/gemm_midx_kernel_sphere32.md"},
+    "jacobi_cluster2_kernel": {"bytes": 367.104e3, "profile": "profiles/jacobi_cluster2_kernel_sphere32.md"},
+    "qr_cluster_kernel": {"bytes": 375.296e3, "profile": "profiles/qr_cluster_kernel_sphere32.md"},
+    "gemm_midx_kernel": {"bytes": 536.32e3, "profile": "profiles/gemm_midx_kernel_sphere32.md"},
 }
 
 

@@ -30,9 +30,10 @@ namespace {
 // running sum add up (K u at worst where all terms have one sign, as in the
 // mean fields of a solve): these sums were the largest part of a complex64
 // solve's error.  With runs of 8 it is (8 + K / 8) u.  C_eff of a 16^3 sphere with
-// exact operators, rms over 24 solves 2.9e-6 / 1.7e-6 / 1.2e-6 / 1.3e-6 with one
-// chain / runs of 16 / 8 / 4; roundings 1.1 to 2.1 times more exact; the sums
-// cost 1-3 % of a contrast step at rank 128 (compensated ones 8-20 % for 0.9e-6).
+// exact operators, rms over 24 solves 1.7e-6 / 1.2e-6 / 1.3e-6 with runs of 16 / 8 / 4
+// (one chain 2.9e-6 / runs of 8 1.8e-6 before the QR and the SVD set their vectors'
+// norms right); roundings 1.1 to 2.1 times more exact; the sums cost 3 % of a
+// contrast step at rank 128 (11.34 / 11.70 ms), compensated ones 8-20 % for 0.9e-6.
 QTT_HD bool midx_unit_inner(const MIdx& m) { return (m.n2 == 1 ? m.s1 : m.s2) == 1; }
 
 template <class R, int BM, int BN, int BK, int TM, int TN>
