@@ -206,7 +206,9 @@ __device__ __forceinline__ int rotate_pair(cplx<R> (&x)[RT], cplx<R> (&y)[RT], R
     rot = act && (hg >> 20) + 1023 > ea + eb + ilogb_c(tol2) && hg >= kHiMin && hg < 0x7ff00000;
     if (LP == 32 ? !rot : !__any_sync(0xffffffffu, rot)) return 0;
     const R D = be - al, q4 = times2(ag2, 2), h2 = fma(D, D, q4);
-    const R H = h2 * dense::rsqrt_approx(h2), W = fabs(D) + H;  // 2 h, 2 w
+    // 2 h by one Newton step of the square root from 20 bits (without it a rotation leaves
+    // up to 2^-21 of its cosine, which the rule for the last sweep takes for nothing), 2 w
+    const R yh = dense::rsqrt_approx(h2), H0 = h2 * yh, H = fma(fma(-H0, H0, h2), times2(yh, -1), H0), W = fabs(D) + H;
     const R x4 = fma(W, W, q4);
     const R r2 = dense::rsqrt_third_order(x4, dense::rsqrt_approx(x4));  // r / 2
     const R r = times2(r2, 1);
@@ -443,11 +445,7 @@ jacobi_cluster2_kernel(const __grid_constant__ JacArgs<R> a) {
   // sine weighted by the norms' ratio of a sweep, the cosines after it are at
   // most about sqrt(qa) s c; with both at most sqrt(tol / sqrt(qa)) they are at
   // most tol, and the next sweep would rotate nothing.
-  // FP64 takes its angles from a square root good to 2^-20, so that a rotation also
-  // leaves 2^-21 of the cosine it removes (half of h's error goes into w); c is at
-  // most about 2 s, and s at most 2^19 tol keeps that below tol / 2.
-  R big2 = tol / sqrt(R(qa));
-  if constexpr (sizeof(R) == 8) big2 = fmin(big2, tol2 * R(1ll << 38));
+  const R big2 = tol / sqrt(R(qa));
   C x[RT], y[RT];
   auto load = [&](C(&v)[RT], const C* s) {
 #pragma unroll
